@@ -179,7 +179,8 @@ __device__ __forceinline__ long long warp_sum(long long s)
 // bytes are shifted by its misalignment with the neighbouring lane's, and only the first and
 // the last lane of the tile store partial words. A thread per 8 genes with element accesses
 // and two atomics each, which this replaces, spent its time on 1.3 M contended atomics and
-// on single-byte stores (512 x 10,007 genes, whole call: 164 us, now 18 us).
+// on single-byte stores (512 x 10,007 genes, a whole call with its rotation: 170 us, now 27 us; this
+// kernel 19 us, of which its first loads and the last block's scan are about a third).
 constexpr int kTileGenes = 256;
 
 template <int kThr>
@@ -214,20 +215,28 @@ __global__ void __launch_bounds__(kThreads, 3) noalloc_observe_kernel(const __gr
             v[i] = i < nv ? a.v[j0 + i] : 0;
             any |= (uint32_t)w[i] | (uint32_t)v[i];
         }
-        // items below 2^16 (the usual case): a row's 256 items sum below 2^24
-        const bool small = __all_sync(0xffffffffu, any < 0x10000u);
+        // Items below 2^8: a lane's 8 alleles and both sums fit one word (allele bits from bit
+        // 22, sum v from bit 11, sum w), one add per allele; below 2^16: 32-bit sums (a row's
+        // 256 items stay below 2^24); else 64-bit ones. Uniform over the warp.
+        const int form = __all_sync(0xffffffffu, any < 0x100u) ? 0 : __all_sync(0xffffffffu, any < 0x10000u) ? 1 : 2;
+        if (form == 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) w[i] |= (v[i] << 11) | (1 << (22 + i));
+        }
+        auto load_row = [&](int32_t c) -> uint4 {
+            const size_t row = (size_t)c * a.ng;
+            if (nv == 8) return load_half8(a.k, row + j0, total);
+            uint32_t q[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+                if (i < nv) q[i >> 1] |= (uint32_t)(uint16_t)a.k[row + j0 + i] << (16 * (i & 1));
+            return make_uint4(q[0], q[1], q[2], q[3]);
+        };
+        uint4 hn = load_row((int32_t)c_begin);
         for (int32_t c = (int32_t)c_begin; c < c_end; ++c) {
             const size_t row = (size_t)c * a.ng;
-            uint4 h = make_uint4(0u, 0u, 0u, 0u);
-            if (nv == 8) {
-                h = load_half8(a.k, row + j0, total);
-            } else if (nv > 0) {
-                uint32_t q[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-                for (int i = 0; i < 7; ++i)
-                    if (i < nv) q[i >> 1] |= (uint32_t)(uint16_t)a.k[row + j0 + i] << (16 * (i & 1));
-                h = make_uint4(q[0], q[1], q[2], q[3]);
-            }
+            const uint4 h = hn;
+            if (c + 1 < c_end) hn = load_row(c + 1);        // in flight while this row is computed
             // angle indices outside [-K, K] are invalid input; they are clamped so that the
             // table lookup stays inside the table; 4(k + K) is T's byte offset
             uint32_t sp[4] = {h.x, h.y, h.z, h.w};
@@ -236,40 +245,57 @@ __global__ void __launch_bounds__(kThreads, 3) noalloc_observe_kernel(const __gr
             const qieo::Draw4 d0 = qieo::philox4x32_10((uint32_t)(j0 / 4u), (uint32_t)c, (uint32_t)a.t, 0u, a.seed, a.inst);
             const qieo::Draw4 d1 = qieo::philox4x32_10((uint32_t)(j0 / 4u) + 1u, (uint32_t)c, (uint32_t)a.t, 0u, a.seed, a.inst);
             const uint32_t u[8] = {d0.a, d0.b, d0.c, d0.d, d1.a, d1.b, d1.c, d1.d};
+            uint32_t xbits;
+            long long sw, sv;
             bool x[8];
-            uint32_t b0 = 0u, b1 = 0u;                      // the alleles as bytes
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const uint32_t off = (i & 1) ? (sp[i >> 1] >> 16) : (sp[i >> 1] & 0xffffu);
                 x[i] = u[i] < *reinterpret_cast<const uint32_t *>(thr_bytes + off) || off == off_top;
-                if (x[i]) (i < 4 ? b0 : b1) |= 1u << (8 * (i & 3));
             }
             // the sums (items past the row's end are 0)
-            long long sw, sv;
-            if (small) {
-                uint32_t lw = 0u, lv = 0u;
+            if (form == 0) {
+                uint32_t acc = 0u;
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    if (x[i]) {
-                        lw += (uint32_t)w[i];
-                        lv += (uint32_t)v[i];
-                    }
-                sw = (long long)__reduce_add_sync(0xffffffffu, lw);
-                sv = (long long)__reduce_add_sync(0xffffffffu, lv);
+                    if (x[i]) acc += (uint32_t)w[i];
+                xbits = acc >> 22;
+                const uint32_t both = __reduce_add_sync(0xffffffffu, (acc & 0x7ffu) | ((acc & 0x3ff800u) << 5));
+                sw = (long long)(both & 0xffffu);
+                sv = (long long)(both >> 16);
             } else {
-                long long lw = 0, lv = 0;
+                xbits = 0u;
+                if (form == 1) {
+                    uint32_t lw = 0u, lv = 0u;
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (x[i]) {
-                        lw += w[i];
-                        lv += v[i];
-                    }
-                sw = warp_sum(lw);
-                sv = warp_sum(lv);
+                    for (int i = 0; i < 8; ++i)
+                        if (x[i]) {
+                            xbits |= 1u << i;
+                            lw += (uint32_t)w[i];
+                            lv += (uint32_t)v[i];
+                        }
+                    sw = (long long)__reduce_add_sync(0xffffffffu, lw);
+                    sv = (long long)__reduce_add_sync(0xffffffffu, lv);
+                } else {
+                    long long lw = 0, lv = 0;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (x[i]) {
+                            xbits |= 1u << i;
+                            lw += w[i];
+                            lv += v[i];
+                        }
+                    sw = warp_sum(lw);
+                    sv = warp_sum(lv);
+                }
             }
             if (lane < 2)
                 atomicAdd(reinterpret_cast<unsigned long long *>(a.sums + 2 * (size_t)c + lane),
                           (unsigned long long)(lane ? sv : sw));
+            // the alleles as bytes: the multiplier moves bit i of a nibble to bit 8i, and the
+            // sixteen partial products all land on different bits
+            const uint32_t b0 = ((xbits & 15u) * 0x00204081u) & 0x01010101u;
+            const uint32_t b1 = ((xbits >> 4) * 0x00204081u) & 0x01010101u;
             // the alleles: lane l stores the aligned word that starts b bytes before its own
             uint8_t *const xp = a.x + row + j0;
             const uint32_t b = (uint32_t)(reinterpret_cast<uintptr_t>(xp) & 7u);
@@ -287,13 +313,43 @@ __global__ void __launch_bounds__(kThreads, 3) noalloc_observe_kernel(const __gr
                 const bool last = lane == 31 || left <= 8;   // no lane after this one holds genes
                 if (lane > 0 && nv == 8)
                     *reinterpret_cast<uint64_t *>(xp - b) = (prev >> (64u - 8u * b)) | (own << (8u * b));
-                if (lane > 0 && nv > 0 && nv < 8)           // the previous lane's last b bytes
-                    for (uint32_t i = 0; i < b; ++i) xp[(int)i - (int)b] = (uint8_t)(prev >> (64u - 8u * b + 8u * i));
-                if (nv > 0 && (lane == 0 || nv < 8)) {      // up to the next aligned word
-                    for (int i = 0; i < (nv < 8 ? nv : 8 - (int)b); ++i) xp[i] = (uint8_t)(own >> (8 * i));
+                if (lane == 0 && nv == 8) {                 // up to the next aligned word
+                    const uint32_t n = 8u - b;
+                    uint64_t v8 = own;
+                    uint8_t *q = xp;
+                    if (n & 1u) {
+                        *q = (uint8_t)v8;
+                        q += 1;
+                        v8 >>= 8;
+                    }
+                    if (n & 2u) {
+                        *reinterpret_cast<uint16_t *>(q) = (uint16_t)v8;
+                        q += 2;
+                        v8 >>= 16;
+                    }
+                    if (n & 4u) *reinterpret_cast<uint32_t *>(q) = (uint32_t)v8;
                 }
-                if (nv == 8 && last)                        // the last b bytes, with no lane after
-                    for (uint32_t i = 8u - b; i < 8u; ++i) xp[i] = (uint8_t)(own >> (8u * i));
+                if (nv == 8 && last) {                      // the last b bytes, with no lane after
+                    uint64_t v8 = own >> (64u - 8u * b);
+                    uint8_t *q = xp + (8u - b);
+                    if (b & 4u) {
+                        *reinterpret_cast<uint32_t *>(q) = (uint32_t)v8;
+                        q += 4;
+                        v8 >>= 32;
+                    }
+                    if (b & 2u) {
+                        *reinterpret_cast<uint16_t *>(q) = (uint16_t)v8;
+                        q += 2;
+                        v8 >>= 16;
+                    }
+                    if (b & 1u) *q = (uint8_t)v8;
+                }
+                if (nv > 0 && nv < 8) {                     // the row's last genes
+                    if (lane > 0)                           // the previous lane's last b bytes
+                        for (uint32_t i = 0; i < b; ++i)
+                            xp[(int)i - (int)b] = (uint8_t)(prev >> (64u - 8u * b + 8u * i));
+                    for (int i = 0; i < nv; ++i) xp[i] = (uint8_t)(own >> (8 * i));
+                }
             }
         }
     }
@@ -503,10 +559,10 @@ qieo_status launch_noalloc(const qieo_problem &problem, const qieo_params &param
     a.seed = params.seed;
     a.inst = params.instance_id;
     fill_thresholds(params.dtheta_den, a.thr);
-    // Rows per warp: about two waves of the 24 warps an SM holds, so that the last wave is
-    // short, and at most 64 rows (the items are then loaded once per 16,384 genes).
+    // Rows per warp: one wave of the 24 warps an SM holds, and at most 64 rows (the items are
+    // then loaded once per 16,384 genes).
     a.ntile = (int32_t)(((int64_t)ng + kTileGenes - 1) / kTileGenes);
-    const int64_t units = (int64_t)a.ntile * np, warps = (int64_t)48 * sms;
+    const int64_t units = (int64_t)a.ntile * np, warps = (int64_t)24 * sms;
     a.rows = (int32_t)std::max<int64_t>(1, std::min<int64_t>(64, (units + warps - 1) / warps));
     const int64_t items = (int64_t)a.ntile * (((int64_t)np + a.rows - 1) / a.rows);
     const int64_t obs_blocks = (items + kThreads / 32 - 1) / (kThreads / 32);
