@@ -366,6 +366,7 @@ def run_gpu(a):
     inst = Q.Instance(prob, np_, seed=c["seed"], inst=c["inst"] + rank,
                       stream=stream.cuda_stream, flags=flags)
     shape = inst.shape()
+    column = not (a.state_i8 or a.streamed or a.no_fixed_words)   # the default form of rule R1
     state_bytes = np_ * ((ng + 7) // 8) * (8 if a.state_i8 else 16)
     flush = state_bytes < 2 * L2_BYTES
     flush_buf = torch.empty(512 * 1024 * 1024, dtype=torch.uint8, device="cuda") if flush else None
@@ -437,7 +438,12 @@ def run_gpu(a):
                                    ceiling.grid_ctas, ceiling.reps)}
     roof["frac_hbm_4B_formula"] = hbm_achieved / hbm_peak
     roof["fixed_words"] = bool(shape.fixed_words)
-    if shape.fixed_words:
+    if column:
+        roof["note"] = ("column form: the rows of the population share one row of angle indices (rule R1), so "
+                        "no state is streamed, and genes that have reached a bound are not drawn any more "
+                        "(identical results); the 4 B and full-draw per gene-update formula behind frac can "
+                        "exceed 1")
+    elif shape.fixed_words:
         roof["note"] = ("fixed-vector words: generations in which most vectors are fixed skip their "
                         "draws and state traffic exactly (identical results), so the 4 B and full-draw "
                         "per gene-update formula behind frac can exceed 1; phases.work_adjusted is "
@@ -449,19 +455,22 @@ def run_gpu(a):
         roof["t_hbm_us"] = t_hbm * 1e6
         roof["t_int_us"] = t_int * 1e6
     roof["state_in_l2"] = l2_resident
-    kname = ("resident_run_kernel" if shape.resident else "run_kernel" if shape.persistent
-             else "generation_kernel")
+    kname = ("column_run_kernel" if column else "resident_run_kernel" if shape.resident
+             else "run_kernel" if shape.persistent else "generation_kernel")
     roof["traffic"] = None if a.state_i8 else profile_traffic(kname, a.workload)
-    roof["traffic_per"] = ("generation (one launch per generation)" if not shape.persistent
+    roof["traffic_per"] = ("generation (one launch per generation)" if not (column or shape.persistent)
                            else "generation (the run's launch divided by its generations)")
     if roof["traffic"]:
         roof["frac_dram_measured"] = roof["traffic"] / launch_s / 1e9 / hbm_peak
-    roof["kernel"] = ("resident_run_kernel (one cooperative launch per run, state in shared memory)"
+    roof["kernel"] = ("column_run_kernel, column_small_kernel (cooperative launches of a whole run; one row of "
+                      "angle indices stands for all, whose rows are equal under rule R1)"
+                      if column else
+                      "resident_run_kernel (one cooperative launch per run, state in shared memory)"
                       if shape.resident else
                       "run_kernel (one cooperative launch per run)" if shape.persistent
                       else "generation_kernel (one launch per generation)")
     roof["us_per_generation"] = launch_s * 1e6
-    if not a.no_phases and (shape.resident or not shape.persistent):
+    if not a.no_phases and (column or shape.resident or not shape.persistent):
         roof["phases"] = generation_phases(Q, prob, c, np_, G, rank, flags, stream, torch,
                                            hbm_peak, int_peak)
 
@@ -502,6 +511,7 @@ def run_gpu(a):
                            ("segments of decreasing size (<= %d tile-rows) from a queue"
                             % shape.rows_per_cta) if shape.rows_per_cta >= 64
                            else "equal static shares of <= %d tile-rows" % shape.rows_per_cta,
+                           "the column form's cooperative launches" if column else
                            "one cooperative launch per run with the state resident in shared memory"
                            if shape.resident else "one cooperative launch per run" if shape.persistent
                            else "one launch per generation")),
@@ -510,9 +520,11 @@ def run_gpu(a):
                 "d2h_bytes_per_step": d2h,
                 "what": "qieo_create_instance from host arrays + qieo_run + qieo_get_best + "
                         "qieo_destroy_instance per step"},
-        # per step: the reset's init launch, then either one cooperative launch + the
-        # end-of-run launch, or G generation launches + the final CIP + the end-of-run launch
-        "gpu_launches": a.steps * (1 + (2 if shape.persistent else G + 2)),
+        # per step: the reset's launch, then the column form's run (one launch, two where the
+        # blocks' shares are long at first), allele plane and end; or one cooperative launch +
+        # the end-of-run launch; or G generation launches + the final CIP + the end-of-run launch
+        "gpu_launches": a.steps * (1 + ((4 if a.workload != "c1" else 3) if column
+                                        else 2 if shape.persistent else G + 2)),
         "clocks": clocks,
         "wall_s_timed": wall,
     }
@@ -566,7 +578,8 @@ def generation_phases(Q, prob, c, np_, G, rank, flags, stream, torch, hbm_peak, 
            "what": "device clock at each generation's start (resident form) or CUDA events before "
                    "every generation launch of one run (launches serialised)"}
     if drawn is not None and int_peak:
-        out["work_adjusted"] = work_adjusted(ms, drawn, np_ * ((ng + 7) // 8), hbm_peak, int_peak)
+        column = not flags & (Q.QIEO_FLAG_STATE_I8 | Q.QIEO_FLAG_STREAMED | Q.QIEO_FLAG_NO_FIXED_WORDS)
+        out["work_adjusted"] = work_adjusted(ms, drawn, np_ * ((ng + 7) // 8), hbm_peak, int_peak, column)
     return out
 
 
@@ -575,17 +588,18 @@ def generation_phases(Q, prob, c, np_, G, rank, flags, stream, torch, hbm_peak, 
 STABLE_BYTES = 1.0 / 8.0 + 1.0 + 1.0
 
 
-def work_adjusted(ms, drawn, nvec, hbm_peak, int_peak):
+def work_adjusted(ms, drawn, nvec, hbm_peak, int_peak, column=False):
     """The roofline of the work each generation actually needed. A vector that drew (the
     qieo_get_drawn_vectors count) needs its 8 draws at the measured integer ceiling and its
     32 B of state (read and written); one that did not needs its fixed-vector bit and its
     previous alleles read and its alleles written (STABLE_BYTES = 1/8 + 1 + 1 B). Per
     generation the bound is the slower of the two; the fraction is the sum of the bounds
-    over the sum of the measured times."""
+    over the sum of the measured times. column: the column form, whose rows share one row of
+    angle indices and store no alleles: the draws alone."""
     import numpy as np
     d = np.asarray(drawn, dtype=np.float64)
     t_int = 8.0 * d / int_peak
-    t_hbm = (32.0 * d + STABLE_BYTES * (nvec - d)) / (hbm_peak * 1e9)
+    t_hbm = (32.0 * d + STABLE_BYTES * (nvec - d)) / (hbm_peak * 1e9) * (0.0 if column else 1.0)
     bound = np.maximum(t_int, t_hbm)
     meas = np.asarray(ms, dtype=np.float64) * 1e-3
     return {"frac": float(bound.sum() / meas.sum()),

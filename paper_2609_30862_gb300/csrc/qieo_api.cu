@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "../../include/qieo.h"
+#include "qieo_column.cuh"
 #include "qieo_kernels.cuh"
 
 namespace {
@@ -141,6 +142,7 @@ struct qieo_instance {
     // a launch takes gp and replaces these fields
     bool sixteen = false;
     int32_t max_item = 0;          // largest weight or value
+    bool small_items = false;      // 0 <= w, v < 2^20
     int32_t ntile2 = 0, seg_rows_max2 = 0, nsegs2 = 0;
     int64_t units2 = 0;
     const int4 *segq2_view = nullptr;
@@ -192,6 +194,18 @@ struct qieo_instance {
                                        // the tile sums after them stay
     bool fword_dirty = false;          // a run since the last clear may have written words
     std::vector<uint32_t> tile_sums;   // per tile of 256 vectors: sum of weights, of values
+
+    // column form (rule R1; qieo_column.cuh): its device words (in the instance's block), the item-sum
+    // form (0 packed, 1 32-bit, 2 64-bit) and the cooperative grid
+    void *col_mem = nullptr;
+    qieo::ColParams cp{};
+    int col_form = 0, col_grid = 1, col_small_grid = 1;
+    bool col_large = false;        // runs may start with long shares (column_run_kernel)
+    int col_small_blocks = 1;      // blocks column_small_kernel needs at most
+    bool rows_equal = true;        // the state's rows are known to be equal (rule R1)
+    bool state_valid = false;      // the full state holds the population
+    bool col_valid = false;        // cp's state between runs holds it
+    bool force_rows = false;       // autotuning: time the row-by-row forms
 };
 
 namespace {
@@ -265,6 +279,32 @@ ResidentFn resident_fn(const qieo_instance *q)
 {
     if (q->narrow) return q->rule ? &qieo::resident_run_kernel<true, 1, false> : &qieo::resident_run_kernel<true, 0, true>;
     return q->rule ? &qieo::resident_run_kernel<false, 1, false> : &qieo::resident_run_kernel<false, 0, true>;
+}
+
+// Runs in the column form: rule R1 from equal rows, the packed elite key, 16-bit state; not
+// where a flag asks for one of the row-by-row forms or a solve sits in a server's arena.
+bool column_capable(const qieo_instance *q)
+{
+    return q->rule == 0 && q->key_ok && !q->state8 && !q->host_de && !q->row_block && q->owns_block &&
+           !(q->flags & (QIEO_FLAG_UNFUSED | QIEO_FLAG_COOPERATIVE | QIEO_FLAG_REGISTER_PREFETCH |
+                         QIEO_FLAG_PER_GENERATION | QIEO_FLAG_STREAMED | QIEO_FLAG_SIXTEEN |
+                         QIEO_FLAG_NO_FIXED_WORDS | QIEO_FLAG_SPARSE_ALWAYS | QIEO_FLAG_STATE_I8));
+}
+
+bool use_column(const qieo_instance *q)
+{
+    return q->col_mem && q->rows_equal && !q->force_rows && column_capable(q);
+}
+
+typedef void (*ColumnFn)(qieo::GenParams, qieo::ColParams, int32_t);
+ColumnFn column_fn(int form)
+{
+    return form == 0 ? &qieo::column_run_kernel<0> : form == 1 ? &qieo::column_run_kernel<1> : &qieo::column_run_kernel<2>;
+}
+ColumnFn column_small_fn(int form)
+{
+    return form == 0 ? &qieo::column_small_kernel<0>
+                     : form == 1 ? &qieo::column_small_kernel<1> : &qieo::column_small_kernel<2>;
 }
 
 // Lets the device's default memory pool keep up to 1 GiB of released blocks, so that
@@ -738,6 +778,60 @@ void build_thresholds(int32_t D, std::vector<uint64_t> &T) { ::build_thresholds(
 
 namespace {
 
+// Device memory of the column form: the state between runs, the two parities, the recorded best
+// alleles and the two lists (16 B a vector each), then the counts, the control words and the
+// blocks' posts.
+size_t column_bytes(int32_t svec)
+{
+    return 5 * align_up((size_t)svec * 16, 256) + 512 + 2 * qieo::kColPosted * sizeof(qieo::ColSync);
+}
+
+// The column form's words (in q->col_mem) and grids, once per instance.
+qieo_status configure_column(qieo_instance *q)
+{
+    if (!q->col_mem) return QIEO_OK;
+    const size_t sv = (size_t)q->svec;
+    // packed sums as in the row-by-row forms (items in [0, 255], row sums below 2^26, at most
+    // 4,095 tiles of 256 vectors); items in [0, 2^20) keep a tile-row's sum below 2^31
+    const bool wide = (q->flags & QIEO_FLAG_FORCE_WIDE) != 0;
+    if (!wide && q->narrow_items && q->sum_w < (1ll << 26) && q->sum_v < (1ll << 26) && sv <= (size_t)4095 * qieo::kThreads)
+        q->col_form = 0;
+    else
+        q->col_form = !wide && q->small_items ? 1 : 2;
+    int bps = 0;
+    qieo_status st = resident_blocks(q->device, reinterpret_cast<const void *>(column_fn(q->col_form)), 0, &bps);
+    if (st != QIEO_OK) return st;
+    q->col_grid = q->sm_count * std::max(1, std::min(bps, kBlocksPerSm));
+    st = resident_blocks(q->device, reinterpret_cast<const void *>(column_small_fn(q->col_form)), 0, &bps);
+    if (st != QIEO_OK) return st;
+    q->col_small_grid = q->sm_count * std::max(1, std::min(bps, 2));
+    {
+        // passes of the full list (tiles of 256 items; a short list takes several rows a pass)
+        const int64_t ntile = ((int64_t)sv + qieo::kThreads - 1) / qieo::kThreads;
+        const int64_t rpp = ntile > 1 ? 1 : qieo::kThreads / pow2_ceil((int)sv);
+        const int64_t units = ntile * ((q->np + rpp - 1) / rpp);
+        q->col_large = units >= (int64_t)qieo::kColSmallShare * q->col_grid || ntile > qieo::kColSmallTiles;
+        // a shorter list never has more passes than the bound of a small share
+        q->col_small_blocks = q->col_large ? q->col_small_grid : (int)std::min<int64_t>(q->col_small_grid, units);
+    }
+    char *b = static_cast<char *>(q->col_mem);
+    const size_t rows = align_up(sv * 16, 256);
+    qieo::ColParams &c = q->cp;
+    c.canon = reinterpret_cast<uint2 *>(b);
+    c.rows = reinterpret_cast<uint2 *>(b + rows);
+    c.best_nib = reinterpret_cast<int2 *>(b + 3 * rows);
+    c.lists = reinterpret_cast<int32_t *>(b + 4 * rows);
+    char *const words = b + 5 * rows;
+    c.slot = reinterpret_cast<qieo::ColSlot *>(words);
+    c.head = c.slot + 3;
+    c.rest = c.slot + 4;
+    c.ctl = reinterpret_cast<int32_t *>(words + 256);
+    c.qctr = reinterpret_cast<unsigned int *>(words + 320);
+    c.sync = reinterpret_cast<qieo::ColSync *>(words + 384);
+    c.post = reinterpret_cast<qieo::ColSync *>(words + 512);
+    return QIEO_OK;
+}
+
 qieo_status ensure_history(qieo_instance *q, int32_t need)
 {
     if (need <= q->hist_cap) return QIEO_OK;
@@ -775,6 +869,7 @@ qieo_status ensure_history(qieo_instance *q, int32_t need)
     q->gp.hist_e = e;
     q->gp.hist_f = f;
     q->gp.hist_d = d;
+    q->gp.hist_cap_d = (size_t)cap;
     drop_graphs(q);
     return QIEO_OK;
 }
@@ -932,11 +1027,112 @@ qieo_status run_cooperative(qieo_instance *q, int32_t G)
     return QIEO_OK;
 }
 
+int plane_tiles(const qieo_instance *q) { return (q->svec + qieo::kThreads - 1) / qieo::kThreads; }
+
+// Launches column_end_kernel (its from_rows form when `from_rows`).
+cudaError_t launch_column_end(qieo_instance *q, int32_t from_rows)
+{
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = launch_config(q, dim3(plane_tiles(q)), 0, attr);
+    return cudaLaunchKernelEx(&cfg, qieo::column_end_kernel, q->gp, q->cp, from_rows);
+}
+
+// The full state for the row-by-row forms (and, for batches, whatever the batched kernels read).
+qieo_status ensure_state(qieo_instance *q)
+{
+    if (q->state_valid) return QIEO_OK;
+    const size_t total = (size_t)q->np * q->svec;
+    const int blocks = (int)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)q->sm_count * 8));
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = launch_config(q, dim3(blocks), 0, attr);
+    CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_expand_kernel, q->gp, q->cp));
+    if (q->fword_state_bytes) {    // no vector known to be fixed
+        CUDA_TRY(cudaMemsetAsync(q->fword_mem, 0, q->fword_state_bytes, q->stream));
+        q->fword_dirty = false;
+    }
+    q->state_valid = true;
+    return QIEO_OK;
+}
+
+// The column form's state from row 0 of the full state (whose rows are equal).
+qieo_status ensure_column(qieo_instance *q)
+{
+    if (q->col_valid) return QIEO_OK;
+    CUDA_TRY(cudaMemsetAsync(q->cp.head, 0, sizeof(qieo::ColSlot), q->stream));
+    CUDA_TRY(launch_column_end(q, 1));
+    q->col_valid = true;
+    return QIEO_OK;
+}
+
+// A run in the column form: one cooperative launch, the allele plane, the state between runs.
+qieo_status run_column(qieo_instance *q, int32_t G)
+{
+    const bool timing = (q->flags & QIEO_FLAG_TIME_KERNELS) != 0, stamps = (q->flags & QIEO_FLAG_TIME_GENERATIONS) != 0;
+    qieo_status st = ensure_column(q);
+    if (st != QIEO_OK) return st;
+    if (timing) CUDA_TRY(cudaEventRecord(q->ev0, q->stream));
+    if (stamps && q->gen_ns_cap < G + 1) {
+        if (q->gen_ns) cudaFreeAsync(q->gen_ns, q->stream);
+        q->gen_ns = nullptr;
+        q->gen_ns_cap = 0;
+        CUDA_TRY(cudaMallocAsync(&q->gen_ns, (size_t)(G + 1) * sizeof(unsigned long long), q->stream));
+        q->gen_ns_cap = G + 1;
+    }
+    // the barrier counts G x grid arrivals in 32 bits: longer runs are split
+    const int32_t chunk = (int32_t)std::max<int64_t>(1, std::min<int64_t>(G, ((int64_t)1 << 30) / std::max(1, q->col_grid)));
+    const int tiles = plane_tiles(q);
+    const int parts = std::max(1, std::min(q->np, 4 * q->sm_count / tiles));
+    for (int32_t done = 0; done < G; done += chunk) {
+        qieo::GenParams p = q->gp;
+        p.gen_ns = stamps ? q->gen_ns + done : nullptr;
+        cudaLaunchAttribute attr[1];
+        cudaLaunchConfig_t cfg = {};
+        cfg.blockDim = dim3(qieo::kThreads);
+        cfg.stream = q->stream;
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        // the blocks' shares are long at first (as many passes as the full list can have)
+        if (q->col_large) {
+            cfg.gridDim = dim3(q->col_grid);
+            CUDA_TRY(cudaLaunchKernelEx(&cfg, column_fn(q->col_form), p, q->cp, std::min(chunk, G - done)));
+        }
+        cfg.gridDim = dim3(q->col_small_blocks);
+        CUDA_TRY(cudaLaunchKernelEx(&cfg, column_small_fn(q->col_form), p, q->cp, std::min(chunk, G - done)));
+        cudaLaunchAttribute attr1[1];
+        cudaLaunchConfig_t plane = launch_config(q, dim3(tiles * parts), 0, attr1);
+        CUDA_TRY(cudaLaunchKernelEx(&plane, qieo::column_plane_kernel, q->gp, q->cp, tiles));
+        CUDA_TRY(launch_column_end(q, 0));
+    }
+    q->state_valid = false;
+    if (stamps) {
+        q->gen_ev_n = G;
+        q->gen_ns_last = true;
+    }
+    if (timing) {
+        CUDA_TRY(cudaEventRecord(q->ev1, q->stream));
+        st = wait_stream(q->stream);
+        if (st != QIEO_OK) return st;
+        float ms = 0.f;
+        CUDA_TRY(cudaEventElapsedTime(&ms, q->ev0, q->ev1));
+        q->kernel_ms += ms;
+        q->kernel_launches += 1;
+    }
+    return QIEO_OK;
+}
+
 qieo_status run_device(qieo_instance *q, int32_t G)
 {
     if (q->flags & QIEO_FLAG_TIME_KERNELS) {
         qieo_status st = ensure_events(q);
         if (st != QIEO_OK) return st;
+    }
+    if (use_column(q)) return run_column(q, G);
+    if (q->col_mem) {
+        qieo_status st = ensure_state(q);
+        if (st != QIEO_OK) return st;
+        q->col_valid = false;
     }
     if (use_resident(q) || use_cooperative(q)) return run_cooperative(q, G);
     if (q->gp.fword) q->fword_dirty = true;
@@ -1233,6 +1429,7 @@ qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
     q->inst_id = pa->instance_id;
     q->narrow_items = max_w <= 255 && max_v <= 255 && min_v >= 0;
     q->max_item = std::max(max_w, max_v);
+    q->small_items = max_w < (1 << 20) && max_v < (1 << 20) && min_v >= 0;
     q->sum_w = sum_w;
     q->sum_v = sum_v;
     q->sum_absv = sum_absv;
@@ -1267,10 +1464,12 @@ qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
         // stream-ordered allocation from the device's pool: no device-wide synchronisation
         // at allocation or release, and a freed block is reused by the next instance
         keep_pool_memory(q->device);
-        ce = cudaMallocAsync(&q->block, total, q->stream);
+        const size_t col = column_capable(q) ? column_bytes(q->svec) : 0;
+        ce = cudaMallocAsync(&q->block, total + col, q->stream);
         if (ce != cudaSuccess)
             return bail(fail(ce == cudaErrorMemoryAllocation ? QIEO_ERR_OOM : QIEO_ERR_CUDA,
-                             "device allocation of %zu bytes: %s", total, cudaGetErrorString(ce)));
+                             "device allocation of %zu bytes: %s", total + col, cudaGetErrorString(ce)));
+        if (col) q->col_mem = static_cast<char *>(q->block) + total;
     }
     char *b = (char *)q->block;
     qieo::GenParams &g = q->gp;
@@ -1364,6 +1563,7 @@ qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
         }
     }
     qieo_status st = configure(q);
+    if (st == QIEO_OK) st = configure_column(q);
     if (st != QIEO_OK) return bail(st);
     if (ext) {
         q->hist_e = (int32_t *)(b + off[16]);
@@ -1431,13 +1631,19 @@ qieo_status qieo_reset(qieo_instance *q)
     if (st != QIEO_OK) return st;
     const size_t words = (size_t)q->np * q->svec * (q->state8 ? 2 : 4);
     const size_t xbytes = 2 * (size_t)q->np * q->xstride;
-    const int blocks = std::max(1, std::min(q->sm_count * 4, (int)((words + 255) / 256)));
-    qieo::init_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, words, xbytes,
-                                                               (size_t)q->np * 2);
+    const int blocks = std::max(1, std::min(q->sm_count * 4, (int)std::min<size_t>((words + 255) / 256, 1 << 20)));
+    q->rows_equal = true;
+    if (q->col_mem && column_capable(q)) {
+        qieo::column_reset_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, q->cp, xbytes, (size_t)q->np * 2);
+        q->col_valid = true;
+        q->state_valid = false;
+    } else {
+        qieo::init_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, words, xbytes, (size_t)q->np * 2);
+        q->col_valid = false;
+        q->state_valid = true;
+    }
     CUDA_TRY(cudaGetLastError());
-    if (q->hist_d)
-        CUDA_TRY(cudaMemsetAsync(q->hist_d, 0, (size_t)q->hist_cap * sizeof(unsigned long long), q->stream));
-    q->fword_dirty = false;   // init_kernel clears the words with the state
+    q->fword_dirty = false;   // the words are cleared with the state (ensure_state)
     q->t = 0;
     q->rows_t = -1;
     if (q->flags & QIEO_FLAG_SYNC_RUN) return wait_stream(q->stream);
@@ -1545,6 +1751,12 @@ qieo_status qieo_get_state(qieo_instance *q, int16_t *k_out, int32_t *t_out)
             for (int32_t j = 0; j < q->ng; ++j)
                 k_out[(size_t)c * q->ng + j] =
                     (int16_t)((int32_t)(s[(size_t)c * q->svec * 8 + j] >> 2) - q->K);
+    } else if (k_out && !q->state_valid) {   // every row is the column form's
+        std::vector<uint16_t> s((size_t)q->svec * 8);
+        st = fetch(q, s.data(), q->cp.canon, s.size() * 2);
+        if (st != QIEO_OK) return st;
+        for (int32_t j = 0; j < q->ng; ++j) k_out[j] = (int16_t)((int32_t)(s[(size_t)j] >> 2) - q->K);
+        for (int32_t c = 1; c < q->np; ++c) std::memcpy(k_out + (size_t)c * q->ng, k_out, (size_t)q->ng * sizeof(int16_t));
     } else if (k_out) {
         std::vector<uint16_t> s((size_t)q->np * q->svec * 8);
         st = fetch(q, s.data(), q->gp.state, s.size() * 2);
@@ -1762,6 +1974,7 @@ qieo_status qieo_create_row_block(const qieo_problem *problem, const qieo_params
     q->row_block = true;
     q->gp.row0 = row0;
     st = configure(q);   // a row block keeps no fixed-vector words
+    if (st == QIEO_OK) st = qieo_reset(q);   // ... and the full state
     if (st != QIEO_OK) {
         qieo_destroy_instance(q);
         return st;
@@ -1941,8 +2154,13 @@ qieo_status qieo_checkpoint_save(qieo_instance *q, void *buffer, size_t bytes)
     p += (size_t)h.t * sizeof(int32_t);
     if (st == QIEO_OK && h.t > 0) st = fetch(q, p, q->hist_f, (size_t)h.t * sizeof(int64_t));
     p += (size_t)h.t * sizeof(int64_t);
-    if (st == QIEO_OK) st = fetch(q, p, q->gp.state, h.state_bytes);
-    return st;
+    if (st != QIEO_OK) return st;
+    if (q->state_valid) return fetch(q, p, q->gp.state, h.state_bytes);
+    const size_t row = (size_t)q->svec * sizeof(uint4);   // every row is the column form's
+    st = fetch(q, p, q->cp.canon, row);
+    if (st != QIEO_OK) return st;
+    for (int32_t c = 1; c < q->np; ++c) std::memcpy(p + (size_t)c * row, p, row);
+    return QIEO_OK;
 }
 
 qieo_status qieo_checkpoint_load(qieo_instance *q, const void *buffer, size_t bytes)
@@ -1971,6 +2189,16 @@ qieo_status qieo_checkpoint_load(qieo_instance *q, const void *buffer, size_t by
     if (st == QIEO_OK) st = upload(q, q->hist_f, p, (size_t)h.t * sizeof(int64_t));
     p += (size_t)h.t * sizeof(int64_t);
     if (st == QIEO_OK) st = upload(q, q->gp.state, p, h.state_bytes);
+    if (st != QIEO_OK) return st;
+    if (q->col_mem) {   // the column form needs equal rows
+        const size_t row = h.state_bytes / (size_t)q->np;
+        bool equal = true;
+        for (int32_t c = 1; c < q->np && equal; ++c) equal = std::memcmp(p, p + (size_t)c * row, row) == 0;
+        q->rows_equal = equal;
+        q->state_valid = true;
+        q->col_valid = false;
+        q->fword_dirty = true;
+    }
     if (st == QIEO_OK) st = clear_fword(q, q->stream);   // the words of the reset state
     if (st == QIEO_OK) st = upload(q, q->gp.conv, h.conv, sizeof h.conv);
     if (st == QIEO_OK) st = upload(q, q->gp.best, h.best, sizeof h.best);
@@ -2351,6 +2579,12 @@ qieo_status qieo_batch_run(qieo_batch *bt, int32_t G)
         qieo_status st = upload_group(bt, g);
         if (st != QIEO_OK) return st;
     }
+    for (qieo_instance *q : bt->members) {       // the batched kernels read the full state
+        if (!q->col_mem) continue;
+        qieo_status st = ensure_state(q);
+        if (st != QIEO_OK) return st;
+        q->col_valid = false;
+    }
     for (cudaStream_t s : bt->other_streams) {   // pending work of the members' own streams
         CUDA_TRY(cudaEventRecord(bt->ev_in, s));
         CUDA_TRY(cudaStreamWaitEvent(bt->stream, bt->ev_in, 0));
@@ -2416,6 +2650,7 @@ qieo_status qieo_autotune(qieo_instance *q, int32_t trials, qieo_launch_shape *s
     const int old_lanes = q->lanes, old_warps = q->warps, old_grid = q->grid_override;
     const int old_flags = q->flags;
     q->flags &= ~(QIEO_FLAG_TIME_KERNELS | QIEO_FLAG_SYNC_RUN);
+    q->force_rows = true;        // the tile shapes are those of the row-by-row forms
     float best_ms = 1e30f;
     std::pair<int, int> best = {old_lanes, old_warps};
     for (const auto &c : cands) {
@@ -2445,6 +2680,7 @@ qieo_status qieo_autotune(qieo_instance *q, int32_t trials, qieo_launch_shape *s
         }
     }
     q->flags = old_flags;
+    q->force_rows = false;
     q->lanes = best.first;
     q->warps = best.second;
     q->grid_override = old_grid;

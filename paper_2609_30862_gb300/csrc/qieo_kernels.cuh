@@ -162,6 +162,7 @@ struct GenParams {
     unsigned long long *hist_d;   // [capacity] vectors that did not draw, per generation
                                   // (copied from fcnt once the generation is complete), or
                                   // NULL
+    size_t hist_cap_d;            // entries of hist_d (0: NULL)
     unsigned long long *fprev;    // [np] packed row totals (SV << 26 | SW) of the last
                                   // generation, kept by the kernel that keeps F
     const uint32_t *ftile;        // [2 ntile] sums of the weights and of the values of each
@@ -2777,23 +2778,23 @@ __global__ void __launch_bounds__(kThreads) gather_stop_kernel(int32_t *const *c
 }
 
 // Generation 0 state: every qubit at theta = pi/4 (n = K), no elite, no best record.
-__global__ void __launch_bounds__(kThreads) init_kernel(GenParams p, size_t state_words,
-                                                        size_t xbytes, size_t acc_words)
+// state_words = 0 leaves the full state and the fixed-vector words as they are.
+__device__ __forceinline__ void init_words(const GenParams &p, size_t state_words, size_t xbytes, size_t acc_words)
 {
-    grid_dependency_wait();
     const uint32_t kk = (uint32_t)(4 * p.K) * (p.state8 ? 0x01010101u : 0x00010001u);
     uint32_t *s = reinterpret_cast<uint32_t *>(p.state);
     const size_t stride = (size_t)gridDim.x * kThreads;
     const size_t i0 = (size_t)blockIdx.x * kThreads + threadIdx.x;
     for (size_t i = i0; i < state_words; i += stride) s[i] = kk;
-    for (size_t i = i0; i < xbytes; i += stride) p.xbits[i] = 0;
+    uint4 *x = reinterpret_cast<uint4 *>(p.xbits);   // rows and planes are whole 16-byte words
+    for (size_t i = i0; i < xbytes / 16; i += stride) x[i] = make_uint4(0u, 0u, 0u, 0u);
     for (size_t i = i0; i < (size_t)p.xstride; i += stride) p.best_row[i] = 0;
     for (size_t i = i0; i < acc_words; i += stride) p.acc[i] = 0ull;
     for (size_t i = i0; i < (size_t)p.np; i += stride) {
         p.fitness[i] = 0;
         p.cnt[i] = 0u;
     }
-    if (p.fword) {   // no qubit at a bound: every fixed-vector word 0
+    if (p.fword && state_words) {   // no qubit at a bound: every fixed-vector word 0
         uint4 *f = reinterpret_cast<uint4 *>(p.fword);
         const size_t n = (size_t)p.np * (size_t)(p.fstride >> 5) / 4;
         for (size_t i = i0; i < n; i += stride) f[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -2803,6 +2804,7 @@ __global__ void __launch_bounds__(kThreads) init_kernel(GenParams p, size_t stat
         if (i0 == 0)
             for (int i = 0; i < 7; ++i) p.fcnt[i] = 0ull;
     }
+    for (size_t i = i0; i < p.hist_cap_d; i += stride) p.hist_d[i] = 0ull;
     if (i0 == 0) {
         *p.gen = 0;
         *p.ticket = 0u;
@@ -2818,6 +2820,13 @@ __global__ void __launch_bounds__(kThreads) init_kernel(GenParams p, size_t stat
         p.best[1] = -1;
         p.best[2] = -1;
     }
+}
+
+__global__ void __launch_bounds__(kThreads) init_kernel(GenParams p, size_t state_words,
+                                                        size_t xbytes, size_t acc_words)
+{
+    grid_dependency_wait();
+    init_words(p, state_words, xbytes, acc_words);
 }
 
 __global__ void philox_kernel(const uint32_t *ck, uint32_t *out, int32_t n)

@@ -1,0 +1,151 @@
+"""The column form of a run (rule R1 from equal rows: one row of angle indices stands for the
+population), bit for bit against the CPU oracle.
+
+The cases lie where its cuts change: shares short enough for one block, for blocks that meet
+through posts, for the grid barrier, and long ones taken from a queue; lists that shrink from
+whole vectors to single quads to nothing inside a run and across runs; ragged last vectors; the
+three item-sum forms; and every way the population enters or leaves the form (checkpoints with
+equal and with different rows, batches, autotuning, reset). All results are whole numbers: the
+tolerance is zero."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2609_30862_gb300 import qieo as Q
+from paper_2609_30862_gb300 import workload as W
+from saturated import load_state
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    Q.load()
+
+
+def _problem(ng, items):
+    if items == "byte":
+        return W.knapsack(ng, ng + 11)
+    r = np.random.RandomState(ng)
+    if items == "mid":           # items below 2^20, at the limit
+        w = r.randint(0, 1 << 20, ng)
+        w[::2] = (1 << 20) - 1
+        v = np.full(ng, (1 << 20) - 1)
+    else:
+        w = r.randint(0, 2**31 - 1, ng)
+        v = r.randint(-2**31 + 1, 2**31 - 1, ng)
+    return W.custom_problem(w, v, int(w.astype(np.int64).sum()) // 2)
+
+
+def check(I, st, gens):
+    k, t = I.state()
+    assert t == gens == int(st.t[0])
+    e, f = I.history(0, gens)
+    assert np.array_equal(e, st.hist_e), int(np.argmax(e != st.hist_e))
+    assert np.array_equal(f, st.hist_f)
+    assert np.array_equal(k, st.k), "angle indices differ"
+    assert np.array_equal(I.fitness(), st.f)
+    assert np.array_equal(I.alleles(), st.x), "alleles differ"
+    assert np.array_equal(I.allele_row(len(st.f) - 1), st.x[-1])
+    bits, bf, bg, bc = I.best()
+    assert (bf, bg, bc) == tuple(int(v) for v in st.best)
+    assert np.array_equal(bits, st.best_x)
+
+
+@pytest.mark.parametrize("ng,np_,D,items,chunks", [
+    (1, 1, 100, "byte", [5]), (4, 7, 4, "byte", [1, 1, 6]), (9, 2, 12, "wide", [40]),
+    (33, 511, 100, "byte", [30, 1, 1]), (100, 64, 100, "byte", [500]), (257, 513, 40, "mid", [25, 30]),
+    (1023, 40, 100, "byte", [150, 60]), (2048, 300, 100, "byte", [70]), (2049, 65, 8, "wide", [20, 5]),
+    (4100, 130, 100, "mid", [60, 90]), (6000, 16, 4000, "byte", [40]), (20003, 3, 100, "byte", [120]),
+    (300, 20000, 100, "byte", [25, 90]), (20000, 4000, 12, "byte", [30]), (300001, 40, 100, "byte", [12]),
+    (70, 50000, 100, "wide", [60]),
+])
+def test_column_form(ng, np_, D, items, chunks):
+    prob = _problem(ng, items)
+    gens = sum(chunks)
+    st = O.run(prob, np_, gens, seed=ng, inst=3, D=D, lam=2, kind="omp")
+    with Q.Instance(prob, np_, seed=ng, inst=3, D=D, lam=2) as I:
+        for g in chunks:
+            I.run(g)
+        check(I, st, gens)
+        I.reset()                # a second solve on the same words
+        for g in chunks:
+            I.run(g)
+        check(I, st, gens)
+
+
+def test_state_moves_between_the_forms():
+    """Batches and other row-by-row runs between column runs; the checkpoint of a column run
+    loaded elsewhere; a checkpoint whose rows differ, which the column form cannot hold."""
+    prob, np_, seed = W.knapsack(2603, 5), 90, 5
+    st = O.run(prob, np_, 155, seed=seed)
+    with Q.Instance(prob, np_, seed=seed) as I, Q.Instance(prob, np_, seed=seed) as J:
+        I.autotune(2)
+        I.run(40)
+        with Q.Batch([I]) as b:
+            b.run(30)
+        I.run(25)
+        J.run(3)
+        J.load(I.save())
+        J.run(60)
+        check(J, st, 155)
+        I.run(60)
+        check(I, st, 155)
+    rng = np.random.default_rng(9)
+    for rows_equal in (True, False):
+        k0 = rng.integers(-25, 26, size=(1 if rows_equal else np_, 2603)).astype(np.int16).repeat(np_ if rows_equal else 1, 0)
+        st = O.State(np_, prob.ng)
+        st.k[:] = k0
+        O.run(prob, np_, 70, seed=seed, state=st)
+        with Q.Instance(prob, np_, seed=seed) as I:
+            load_state(I, k0)
+            assert np.array_equal(I.state()[0], k0)
+            I.run(30)
+            I.run(40)
+            check(I, st, 70)
+            I.reset()
+            I.run(20)
+            check(I, O.run(prob, np_, 20, seed=seed), 20)
+
+
+@pytest.mark.parametrize("ng,np_", [(40, 30), (600, 50), (3000, 700)])
+def test_convergence_stop(ng, np_):
+    """The stop inside a run, with the generation after it never run, and a stop while the list
+    is already empty; the allele plane of the last generation."""
+    prob = W.knapsack(ng, 21)
+    ref = O.run(prob, np_, 600, seed=21, window=20)
+    n = int(ref.t[0])
+    assert ref.stopped
+    for chunks in ([600], [n - 1, 40], [n, 7], [11] * 60):
+        with Q.Instance(prob, np_, seed=21, flags=Q.QIEO_FLAG_CONVERGE) as I:
+            for g in chunks:
+                I.run(g)
+            k, t = I.state()
+            assert t == n and np.array_equal(k, ref.k)
+            e, f = I.history(0, n)
+            assert np.array_equal(e, ref.hist_e) and np.array_equal(f, ref.hist_f)
+            bits, bf, bg, bc = I.best()
+            assert (bf, bg, bc) == tuple(int(v) for v in ref.best) and np.array_equal(bits, ref.best_x)
+            assert np.array_equal(I.fitness(), ref.f)
+            assert I.convergence() == (True, 20)
+
+
+def test_wait_that_runs_out_is_reported():
+    """A 1 ns bound on the wait between generations ends the run with a timeout, no trap and no
+    hang; after a reset the instance runs correctly again."""
+    for ng, np_ in ((400, 300), (2000, 300), (5000, 100)):
+        prob = W.knapsack(ng, 16)
+        with Q.Instance(prob, np_, seed=16) as I:
+            I.set_wait_timeout(1)
+            I.run(30)
+            try:
+                I.synchronize()
+            except Q.QieoError as e:
+                assert e.status == Q.QIEO_ERR_TIMEOUT
+            I.set_wait_timeout(10 * 10**9)
+            I.reset()
+            I.run(30)
+            check(I, O.run(prob, np_, 30, seed=16), 30)
