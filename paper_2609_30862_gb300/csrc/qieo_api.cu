@@ -199,7 +199,7 @@ struct qieo_instance {
     // form (0 packed, 1 32-bit, 2 64-bit) and the cooperative grid
     void *col_mem = nullptr;
     qieo::ColParams cp{};
-    int col_form = 0, col_grid = 1, col_small_grid = 1;
+    int col_form = 0, col_per_sm = 2, col_grid = 1, col_small_grid = 1;
     bool col_large = false;        // runs may start with long shares (column_run_kernel)
     int col_small_blocks = 1;      // blocks column_small_kernel needs at most
     bool rows_equal = true;        // the state's rows are known to be equal (rule R1)
@@ -297,10 +297,35 @@ bool use_column(const qieo_instance *q)
 }
 
 typedef void (*ColumnFn)(qieo::GenParams, qieo::ColParams, int32_t);
-ColumnFn column_fn(int form)
+ColumnFn column_fn(int form, int per_sm)
 {
-    return form == 0 ? &qieo::column_run_kernel<0> : form == 1 ? &qieo::column_run_kernel<1> : &qieo::column_run_kernel<2>;
+    if (per_sm == 2)
+        return form == 0 ? &qieo::column_run_kernel<0, 2>
+                         : form == 1 ? &qieo::column_run_kernel<1, 2> : &qieo::column_run_kernel<2, 2>;
+    return form == 0 ? &qieo::column_run_kernel<0, 3>
+                     : form == 1 ? &qieo::column_run_kernel<1, 3> : &qieo::column_run_kernel<2, 2>;
 }
+
+// Cost of a generation of the full list with `per_sm` blocks on each SM, in warp-rows of one SM
+// (see column_home: tiles narrowed to divide the blocks evenly, whole warps, and whole rows where
+// shares are short). A pass of the kernel built for two blocks per SM takes 0.955 of the other's.
+double column_cost(int64_t svec, int64_t np, int sms, int per_sm)
+{
+    const int64_t grid = (int64_t)sms * per_sm;
+    int64_t ntile = (svec + qieo::kThreads - 1) / qieo::kThreads, group = 1, turns = 1;
+    if (ntile <= grid) {
+        group = grid / ntile;
+        if (ntile > 1) ntile = grid / group;
+    } else {
+        turns = (ntile + grid - 1) / grid;
+        ntile = turns * grid;
+    }
+    const int64_t warps = ((svec + ntile - 1) / ntile + 31) / 32;
+    double rows = (double)np / (double)group;
+    if (rows < (double)qieo::kColQueueShare) rows = std::ceil(rows);
+    return per_sm * (double)warps * rows * (double)turns * (per_sm == 2 ? 0.955 : 1.0);
+}
+
 ColumnFn column_small_fn(int form)
 {
     return form == 0 ? &qieo::column_small_kernel<0>
@@ -783,7 +808,8 @@ namespace {
 // blocks' posts.
 size_t column_bytes(int32_t svec)
 {
-    return 5 * align_up((size_t)svec * 16, 256) + 512 + 2 * qieo::kColPosted * sizeof(qieo::ColSync);
+    return 5 * align_up((size_t)svec * 16, 256) + 512 + 2 * qieo::kColPosted * sizeof(qieo::ColSync) +
+           4 * qieo::kColQueues * sizeof(unsigned int);
 }
 
 // The column form's words (in q->col_mem) and grids, once per instance.
@@ -799,9 +825,11 @@ qieo_status configure_column(qieo_instance *q)
     else
         q->col_form = !wide && q->small_items ? 1 : 2;
     int bps = 0;
-    qieo_status st = resident_blocks(q->device, reinterpret_cast<const void *>(column_fn(q->col_form)), 0, &bps);
+    q->col_per_sm = q->col_form == 2 || column_cost((int64_t)sv, q->np, q->sm_count, 2) <=
+                                            column_cost((int64_t)sv, q->np, q->sm_count, 3) ? 2 : 3;
+    qieo_status st = resident_blocks(q->device, reinterpret_cast<const void *>(column_fn(q->col_form, q->col_per_sm)), 0, &bps);
     if (st != QIEO_OK) return st;
-    q->col_grid = q->sm_count * std::max(1, std::min(bps, kBlocksPerSm));
+    q->col_grid = std::min(q->sm_count * std::max(1, std::min(bps, q->col_per_sm)), qieo::kColQueues);
     st = resident_blocks(q->device, reinterpret_cast<const void *>(column_small_fn(q->col_form)), 0, &bps);
     if (st != QIEO_OK) return st;
     q->col_small_grid = q->sm_count * std::max(1, std::min(bps, 2));
@@ -817,6 +845,7 @@ qieo_status configure_column(qieo_instance *q)
     char *b = static_cast<char *>(q->col_mem);
     const size_t rows = align_up(sv * 16, 256);
     qieo::ColParams &c = q->cp;
+    c.one = 1u;
     c.canon = reinterpret_cast<uint2 *>(b);
     c.rows = reinterpret_cast<uint2 *>(b + rows);
     c.best_nib = reinterpret_cast<int2 *>(b + 3 * rows);
@@ -826,9 +855,9 @@ qieo_status configure_column(qieo_instance *q)
     c.head = c.slot + 3;
     c.rest = c.slot + 4;
     c.ctl = reinterpret_cast<int32_t *>(words + 256);
-    c.qctr = reinterpret_cast<unsigned int *>(words + 320);
     c.sync = reinterpret_cast<qieo::ColSync *>(words + 384);
     c.post = reinterpret_cast<qieo::ColSync *>(words + 512);
+    c.qctr = reinterpret_cast<unsigned int *>(words + 512 + 2 * qieo::kColPosted * sizeof(qieo::ColSync));
     return QIEO_OK;
 }
 
@@ -1096,7 +1125,7 @@ qieo_status run_column(qieo_instance *q, int32_t G)
         // the blocks' shares are long at first (as many passes as the full list can have)
         if (q->col_large) {
             cfg.gridDim = dim3(q->col_grid);
-            CUDA_TRY(cudaLaunchKernelEx(&cfg, column_fn(q->col_form), p, q->cp, std::min(chunk, G - done)));
+            CUDA_TRY(cudaLaunchKernelEx(&cfg, column_fn(q->col_form, q->col_per_sm), p, q->cp, std::min(chunk, G - done)));
         }
         cfg.gridDim = dim3(q->col_small_blocks);
         CUDA_TRY(cudaLaunchKernelEx(&cfg, column_small_fn(q->col_form), p, q->cp, std::min(chunk, G - done)));

@@ -68,12 +68,13 @@ struct ColParams {
     int32_t *lists;               // [2][2 svec] vectors at [0, svec), single quads at [svec, 2 svec)
     int2 *best_nib;               // [2 svec] (generation, alleles) of the last best row recorded
     ColSync *sync;                // [4] generation t in t & 3 (arrived: blocks)
-    unsigned int *qctr;           // [4] next segment of generation t in t & 3
+    unsigned int *qctr;           // [4][kColQueues] next rows of a tile, generation t in t & 3
     ColSync *post;                // [2][kColPosted] a block's generation t in parity t & 1 (arrived: t + 1)
     ColSlot *slot;                // [3] the counts of a rebuilt list, rebuild r of the run in r % 3
     ColSlot *head;                // the list at the start of a run (in list 0)
     ColSlot *rest;                // the list and the dropped quads' sums at the hand-over
     int32_t *ctl;                 // [16]
+    uint32_t one;                 // 1 (see mad_add)
 };
 
 __device__ __forceinline__ uint2 *column_parity(const ColParams &c, int32_t svec, int32_t t)
@@ -86,9 +87,10 @@ __device__ __forceinline__ int32_t *column_list(const ColParams &c, int32_t svec
     return c.lists + (size_t)which * 2u * (size_t)svec;
 }
 
-constexpr int kColRows = 256;               // rows summed in shared memory at once
+constexpr int kColRows = 256;               // rows summed in shared memory at once (one a thread)
 constexpr int kColLocalPasses = 2;          // at most this many passes: one block that meets nobody
-constexpr int kColQueueShare = 64;          // passes per block from which segments are queued
+constexpr int kColQueueShare = 32;          // passes per block from which a tile's rows are queued
+constexpr int kColQueues = 1024;            // tiles that can have a queue
 constexpr int kColSmallShare = 4;           // fewer passes per block: column_small_kernel
 constexpr int kColSmallTiles = 128;         // most tiles of a small share (fewer than the blocks)
 constexpr int kColSmallRows = 512;          // column_small_kernel: rows summed in shared memory at once
@@ -98,6 +100,7 @@ template <int kForm>
 struct ColItem {
     int32_t qa, qb;               // quad indices, -1: none
     bool whole;                   // qa, qb are the two quads of one vector
+    bool none;                    // no lane of the warp has a quad
     uint2 sa, sb;                 // their angle indices (4n)
     uint32_t wv[8];               // kForm 0: items (v << 16 | w); else weights
     int32_t v[kForm == 0 ? 1 : 8];
@@ -106,10 +109,10 @@ struct ColItem {
 // How a generation's work is cut, from the list's counts (the same in every block).
 struct ColGeom {
     int items, ntile, width;      // thread items, tiles, items per tile
-    int lanes, warps, rpp;        // a tile's threads; rows per pass
+    int lanes, warps, rpp;        // a tile's threads; rows per pass (a power of two)
     int nu;                       // passes per tile
     int nb;                       // blocks that take part
-    bool queued, small;
+    bool small;                   // column_small_kernel's
 };
 
 __device__ __forceinline__ ColGeom column_geometry(uint32_t nv, uint32_t ns, int np, int grid)
@@ -133,9 +136,72 @@ __device__ __forceinline__ ColGeom column_geometry(uint32_t nv, uint32_t ns, int
     m.nu = (np + m.rpp - 1) / m.rpp;
     const uint32_t units = (uint32_t)m.ntile * (uint32_t)m.nu;    // (the population fits memory)
     m.nb = (int)max(min((uint32_t)grid, units), 1u);
-    m.queued = m.nb > 1 && (m.ntile > m.nb || units >= (uint32_t)(kColQueueShare * m.nb));
-    m.small = !m.queued && m.ntile <= kColSmallTiles && units < (uint32_t)kColSmallShare * (uint32_t)grid;
+    m.small = m.ntile <= kColSmallTiles && units < (uint32_t)kColSmallShare * (uint32_t)grid;
     return m;
+}
+
+// The cut of column_run_kernel: every block has a home tile, whose item it keeps in registers
+// from generation to generation, and a tile's rows are shared by the same number of blocks
+// (`group`); the tiles are made a little narrower so that the blocks divide evenly among them (a
+// warp whose lanes all lie past the tile's width does no work). With more tiles than blocks
+// every block has `turns` tiles and all their rows.
+//
+// The blocks that share an SM do not get equal issue slots, so long shares are taken from the
+// tile's counter in pieces of decreasing size: round l of one piece a block takes half of what
+// is left. (A queue of segments over all tiles, the form before, made a block load and
+// rotate an item for every segment: about 400 instructions for 19 rows on average.)
+struct ColHome {
+    int home, part, group, turns; // first tile, index in the group, blocks per tile, tiles per block
+    int stride;                   // distance of a block's tiles
+    int share;                    // passes per block
+    bool queued;                  // its rows come from the tile's counter
+    int round, start, size;       // the round of the last piece, its first pass and its pieces' passes
+};
+
+__device__ __forceinline__ ColHome column_home(ColGeom &m, int grid)
+{
+    ColHome h;
+    h.turns = 1;
+    if (m.ntile <= grid) {
+        h.group = grid / m.ntile;
+        if (m.ntile > 1) m.ntile = grid / h.group;
+        h.stride = m.ntile;
+    } else {
+        h.group = 1;
+        h.turns = (m.ntile + grid - 1) / grid;
+        m.ntile = h.turns * grid;
+        h.stride = grid;
+    }
+    if (m.ntile > 1) m.width = (m.items + m.ntile - 1) / m.ntile;
+    h.group = min(h.group, m.nu);
+    m.nb = h.stride * h.group;
+    h.home = (int)(blockIdx.x % (unsigned int)h.stride);
+    h.part = (int)(blockIdx.x / (unsigned int)h.stride);
+    h.share = m.nu / h.group;
+    h.queued = h.share >= kColQueueShare && h.group > 1;
+    return h;
+}
+
+// Passes [ua, ub) of piece i of a tile (ua >= nu: none); i grows from call to call of a generation,
+// from i < group.
+__device__ __forceinline__ void column_piece(const ColGeom &m, ColHome &h, int i, int &ua, int &ub)
+{
+    if (!h.queued) {
+        ua = (int)((int64_t)m.nu * i / h.group);
+        ub = (int)((int64_t)m.nu * (i + 1) / h.group);
+        return;
+    }
+    if (i < h.group) {
+        h.round = h.start = 0;
+        h.size = h.share / 2;
+    }
+    while (i - h.round >= h.group) {
+        h.round += h.group;
+        h.start += h.group * h.size;
+        h.size = max(h.size / 2, 2);
+    }
+    ua = h.start + (i - h.round) * h.size;
+    ub = min(m.nu, ua + h.size);
 }
 
 __device__ __forceinline__ bool quad_fixed(uint2 s, uint32_t off_top)
@@ -192,6 +258,7 @@ __device__ __forceinline__ void column_item(const GenParams &p, ColItem<kForm> &
             if (j + 1u < ns) it.qb = __ldcg(list + p.svec + j + 1);
         }
     }
+    it.none = !__any_sync(0xffffffffu, it.qa >= 0);
     it.sa = it.sb = make_uint2(0u, 0u);
     if (it.qa >= 0) it.sa = __ldcg(state + it.qa);
     if (it.qb >= 0) it.sb = __ldcg(state + it.qb);
@@ -209,6 +276,50 @@ __device__ __forceinline__ void column_item(const GenParams &p, ColItem<kForm> &
         it.v[0] = d.x; it.v[1] = d.y; it.v[2] = d.z; it.v[3] = d.w;
         it.v[4] = e.x; it.v[5] = e.y; it.v[6] = e.z; it.v[7] = e.w;
     }
+}
+
+// Philox4x32-10 of counter (q, row, t, 0) for a fixed q and t over many rows. Of the first three
+// rounds only two products depend on the row: M0 n0 of the second, the same for every q
+// (row_product), and M1 c2 of the third; the rest is four words per quad (quad_words), with the
+// round keys folded in.
+struct QuadWords {
+    uint32_t b, d, h, l;          // second round's n2 without the row's part; third round: n0's and n2's xor, c3
+};
+
+__device__ __forceinline__ QuadWords quad_words(const GenParams &p, uint32_t q, uint32_t t)
+{
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * q;
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(p0 >> 32) ^ p.rk1[0]);
+    const uint32_t lo_t = (uint32_t)((uint64_t)kPhiloxM1 * t);
+    const uint64_t p2 = (uint64_t)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ lo_t ^ p.rk0[1]);
+    QuadWords w = {(uint32_t)p0 ^ p.rk1[1], (uint32_t)p1 ^ p.rk0[2], (uint32_t)(p2 >> 32) ^ p.rk1[2], (uint32_t)p2};
+    // (kept in registers: the compiler otherwise computes them again for every row)
+    asm volatile("" : "+r"(w.b), "+r"(w.d), "+r"(w.h), "+r"(w.l));
+    return w;
+}
+
+__device__ __forceinline__ uint64_t row_product(const GenParams &p, uint32_t row, uint32_t t)
+{
+    const uint32_t hi_t = (uint32_t)(((uint64_t)kPhiloxM1 * t) >> 32);
+    return (uint64_t)kPhiloxM0 * (hi_t ^ row ^ p.rk0[0]);
+}
+
+__device__ __forceinline__ Draw4 quad_draw(const GenParams &p, const QuadWords &w, uint64_t z)
+{
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(z >> 32) ^ w.b);
+    uint32_t c0 = (uint32_t)(p1 >> 32) ^ w.d, c1 = (uint32_t)p1, c2 = (uint32_t)z ^ w.h, c3 = w.l;
+#pragma unroll
+    for (int r = 3; r < 10; ++r) {
+        const uint64_t a = (uint64_t)kPhiloxM0 * (uint64_t)c0;
+        const uint64_t b = (uint64_t)kPhiloxM1 * (uint64_t)c2;
+        const uint32_t n0 = (uint32_t)(b >> 32) ^ c1 ^ p.rk0[r];
+        const uint32_t n2 = (uint32_t)(a >> 32) ^ c3 ^ p.rk1[r];
+        c1 = (uint32_t)b;
+        c3 = (uint32_t)a;
+        c0 = n0;
+        c2 = n2;
+    }
+    return {c0, c1, c2, c3};
 }
 
 // Sum over the warp of a 64-bit value of magnitude below 2^36, as two 32-bit reductions: 21
@@ -257,18 +368,26 @@ __device__ __forceinline__ void column_thresholds(const ColItem<kForm> &it, cons
     }
 }
 
+// a + x as a multiply-add by a word that holds 1: the compiler would make a plain add of it, on the
+// ALU pipe, which the compares and Philox's xors keep busy; the multiply pipe has room (a pass of
+// the loop in column_rows: 188 -> 179 cycles per 256 genes).
+__device__ __forceinline__ void mad_add(uint32_t &a, uint32_t x, uint32_t one)
+{
+    asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(a) : "r"(x), "r"(one));
+}
+
 template <int kForm>
 __device__ __forceinline__ ColSum<kForm> column_sum(const ColItem<kForm> &it, const uint32_t (&T)[8],
-                                                    const ColSum<kForm> &base, const uint32_t (&u)[8])
+                                                    const ColSum<kForm> &base, const uint32_t (&u)[8], uint32_t one)
 {
     ColSum<kForm> s = base;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         if (u[i] < T[i]) {
-            if constexpr (kForm == 0) s.a += it.wv[i];
+            if constexpr (kForm == 0) mad_add(s.a, it.wv[i], one);
             else if constexpr (kForm == 1) {
                 s.a += it.wv[i];
-                s.b += (uint32_t)it.v[i];
+                mad_add(s.b, (uint32_t)it.v[i], one);
             } else {
                 s.w += (int32_t)it.wv[i];
                 s.v += it.v[i];
@@ -279,13 +398,14 @@ __device__ __forceinline__ ColSum<kForm> column_sum(const ColItem<kForm> &it, co
 }
 
 template <int kForm>
-__device__ __forceinline__ ColSum<kForm> column_row(const GenParams &p, const ColItem<kForm> &it, const uint32_t (&T)[8],
-                                                    const ColSum<kForm> &base, uint32_t row, uint32_t t)
+__device__ __forceinline__ ColSum<kForm> column_row(const GenParams &p, uint32_t one, const ColItem<kForm> &it, const uint32_t (&T)[8],
+                                                    const ColSum<kForm> &base, const QuadWords &wa,
+                                                    const QuadWords &wb, uint32_t row, uint32_t t)
 {
-    const Draw4 r0 = philox4x32_10_rk((uint32_t)it.qa, row, t, 0u, p.rk0, p.rk1);
-    const Draw4 r1 = philox4x32_10_rk((uint32_t)it.qb, row, t, 0u, p.rk0, p.rk1);
+    const uint64_t z = row_product(p, row, t);
+    const Draw4 r0 = quad_draw(p, wa, z), r1 = quad_draw(p, wb, z);
     const uint32_t u[8] = {r0.a, r0.b, r0.c, r0.d, r1.a, r1.b, r1.c, r1.d};
-    return column_sum<kForm>(it, T, base, u);
+    return column_sum<kForm>(it, T, base, u, one);
 }
 
 // Adds lane sums of a row (whole warp) into one lane's keeper; see column_rows.
@@ -368,81 +488,81 @@ __device__ __forceinline__ unsigned long long column_row_done(const GenParams &p
     return elite_key(f, c);
 }
 
-// The block's sums of rows ra .. ra + n - 1 (n <= kColRows) of one tile: added to the rows, and
-// the rows that are complete evaluated (eq. (1)) and offered to the elite key, one atomic per
-// warp. Called by the whole block; leaves the accumulators 0.
+// The block's sums in accumulators 0 .. n - 1 (n <= kColRows), of rows s_row[i] of one tile: added
+// to the rows, and the rows that are complete evaluated (eq. (1)) and offered to the elite key,
+// one atomic per warp. Called by the whole block; leaves the accumulators 0.
 template <int kForm>
-__device__ __forceinline__ void column_flush(const GenParams &p, int ntile, int ra, int n, const int64_t *s_fix,
-                                             unsigned long long *key, uint32_t *s_acc32,
+__device__ __forceinline__ void column_flush(const GenParams &p, int ntile, const int32_t *s_row, int n,
+                                             const int64_t *s_fix, unsigned long long *key, uint32_t *s_acc32,
                                              unsigned long long *s_acc64)
 {
     __syncthreads();
     const int i = threadIdx.x;
-    if (i >= ((n + 31) & ~31)) {
-        __syncthreads();
-        return;
+    if (i < ((n + 31) & ~31)) {
+        const unsigned long long best =
+            i < n ? column_row_done<kForm>(p, ntile, s_row[i], i, s_fix, s_acc32, s_acc64) : 0ull;
+        const uint32_t hi = (uint32_t)(best >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+        const uint32_t lo = hi == mh ? (uint32_t)best : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+        if ((i & 31) == 0 && (mh | ml) != 0u) atomicMax(key, ((unsigned long long)mh << 32) | ml);
     }
-    const unsigned long long best = i < n ? column_row_done<kForm>(p, ntile, ra + i, i, s_fix, s_acc32, s_acc64) : 0ull;
-    const uint32_t hi = (uint32_t)(best >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
-    const uint32_t lo = hi == mh ? (uint32_t)best : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
-    if ((i & 31) == 0 && (mh | ml) != 0u) atomicMax(key, ((unsigned long long)mh << 32) | ml);
     __syncthreads();
 }
 
-// Rows ra .. rb - 1 of one tile.
+// The sums of rows ra .. ra + n - 1 of one tile into accumulators acc .. acc + n - 1.
 template <int kForm>
-__device__ __forceinline__ void column_rows(const GenParams &p, const ColGeom &m, const BlockShare &b,
+__device__ __forceinline__ void column_rows(const GenParams &p, uint32_t one, const ColGeom &m, const BlockShare &b,
                                             const ColItem<kForm> &it, const uint32_t (&T)[8], const ColSum<kForm> &base,
-                                            int ra, int rb, uint32_t t, const int64_t *s_fix, unsigned long long *key,
-                                            uint32_t *s_acc32, unsigned long long *s_acc64)
+                                            int ra, int n, int acc, uint32_t t, uint32_t *s_acc32,
+                                            unsigned long long *s_acc64)
 {
     const int lane = threadIdx.x & 31;
-    for (int r0 = ra; r0 < rb; r0 += kColRows) {
-        const int n = min(kColRows, rb - r0);
-        if (m.lanes == 32) {
-            // Two rows per step (four independent Philox chains). Lane i keeps the warp's sums
-            // of its row i mod 32 of the pass sequence and adds them once per 32 rows.
+    const QuadWords wa = quad_words(p, (uint32_t)it.qa, t), wb = quad_words(p, (uint32_t)it.qb, t);
+    if (m.lanes == 32) {
+        // Two rows per step (four independent Philox chains). Lane i keeps the warp's sums of
+        // row i of each 32 and adds them at once.
+        const int sh = __ffs(m.rpp) - 1;
+        const int mypass = (n - b.r_sub + m.rpp - 1) >> sh;          // passes with a row of this thread
+        const int passes = it.none ? 0 : (n + m.rpp - 1) >> sh;      // (none: past the tile's width)
+        uint32_t row = (uint32_t)(ra + b.r_sub);
+        const uint32_t step = (uint32_t)m.rpp;
+        for (int q0 = 0; q0 < passes; q0 += 32) {
+            const int nq = min(32, passes - q0);
             ColSum<kForm> mine = {0u, 0u, 0, 0};
-            const int mypass = (n - b.r_sub + m.rpp - 1) / m.rpp;        // passes with a row of this thread
-            const int passes = (n + m.rpp - 1) / m.rpp;
-            const uint32_t row = (uint32_t)(r0 + b.r_sub);
-            auto put = [&](int q) {               // after the sums of pass q: the 32 rows' atomics
-                const int mq = (q & ~31) + lane;
-                if (mq <= q && mq < mypass) column_add<kForm>(mine, mq * m.rpp + b.r_sub, s_acc32, s_acc64);
-            };
             int q = 0;
-            for (; q + 1 < passes; q += 2) {
-                const ColSum<kForm> a = column_row<kForm>(p, it, T, base, row + (uint32_t)(q * m.rpp), t);
-                const ColSum<kForm> c = column_row<kForm>(p, it, T, base, row + (uint32_t)((q + 1) * m.rpp), t);
+#pragma unroll 1
+            for (; q + 1 < nq; q += 2) {
+                const ColSum<kForm> a = column_row<kForm>(p, one, it, T, base, wa, wb, row, t);
+                const ColSum<kForm> c = column_row<kForm>(p, one, it, T, base, wa, wb, row + step, t);
+                row += 2u * step;
                 const ColSum<kForm> as = column_warp_sum<kForm>(a), cs = column_warp_sum<kForm>(c);
-                if (lane == (q & 31)) mine = as;
-                if (lane == ((q + 1) & 31)) mine = cs;
-                if (((q + 2) & 31) == 0 || q + 2 == passes) put(q + 1);
+                if (lane == q) mine = as;
+                if (lane == q + 1) mine = cs;
             }
-            if (q < passes) {
-                const ColSum<kForm> as = column_warp_sum<kForm>(column_row<kForm>(p, it, T, base, row + (uint32_t)(q * m.rpp), t));
-                if (lane == (q & 31)) mine = as;
-                put(q);
+            if (q < nq) {
+                const ColSum<kForm> as = column_warp_sum<kForm>(column_row<kForm>(p, one, it, T, base, wa, wb, row, t));
+                row += step;
+                if (lane == q) mine = as;
             }
-        } else {
-            for (int q = b.r_sub; q < n + b.r_sub; q += m.rpp) {         // the same trips for every thread
-                ColSum<kForm> s = column_row<kForm>(p, it, T, base, (uint32_t)(r0 + q), t);
+            if (lane < nq && q0 + lane < mypass)
+                column_add<kForm>(mine, acc + (q0 + lane) * m.rpp + b.r_sub, s_acc32, s_acc64);
+        }
+    } else {
+        for (int q = b.r_sub; q < n + b.r_sub; q += m.rpp) {         // the same trips for every thread
+            ColSum<kForm> s = column_row<kForm>(p, one, it, T, base, wa, wb, (uint32_t)(ra + q), t);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    if (o < m.lanes) {
-                        if constexpr (kForm == 2) {
-                            s.w += __shfl_xor_sync(0xffffffffu, s.w, o);
-                            s.v += __shfl_xor_sync(0xffffffffu, s.v, o);
-                        } else {
-                            s.a += __shfl_xor_sync(0xffffffffu, s.a, o);
-                            if constexpr (kForm == 1) s.b += __shfl_xor_sync(0xffffffffu, s.b, o);
-                        }
+            for (int o = 16; o > 0; o >>= 1) {
+                if (o < m.lanes) {
+                    if constexpr (kForm == 2) {
+                        s.w += __shfl_xor_sync(0xffffffffu, s.w, o);
+                        s.v += __shfl_xor_sync(0xffffffffu, s.v, o);
+                    } else {
+                        s.a += __shfl_xor_sync(0xffffffffu, s.a, o);
+                        if constexpr (kForm == 1) s.b += __shfl_xor_sync(0xffffffffu, s.b, o);
                     }
                 }
-                if (b.leader && q < n) column_add<kForm>(s, q, s_acc32, s_acc64);
             }
+            if (b.leader && q < n) column_add<kForm>(s, acc + q, s_acc32, s_acc64);
         }
-        column_flush<kForm>(p, m.ntile, r0, n, s_fix, key, s_acc32, s_acc64);
     }
 }
 
@@ -789,16 +909,21 @@ __device__ __forceinline__ void column_begin(const GenParams &p, const ColParams
 }
 
 // The generations of a run whose blocks have several passes each (at least kColSmallShare):
-// segments of a tile's rows, from a queue where shares are long and fixed otherwise. Every
-// block follows the same sequence of lists, elites and records from the same device words. Once
-// the list is short the rest of the run is handed to column_small_kernel.
+// every block has a home tile (ColHome). Every block follows the same sequence of lists, elites and
+// records from the same device words. Once the list is short the rest of the run is handed to
+// column_small_kernel.
 //
 // Bound by the integer pipes: per 8 genes and row two Philox calls (32 wide multiplies, 35 xors),
 // 8 compares and 8 adds. Wide multiplies hold the FMA-heavy pipe for four cycles and the ALU's
 // issue for two, so a pass costs about 2.13 cycles per ALU instruction plus 2 per wide multiply;
-// the row-by-row pass spends 108 ALU instructions where this one spends about 55.
-template <int kForm>
-__global__ void __launch_bounds__(kThreads, kForm == 2 ? 2 : 3) column_run_kernel(const GenParams p, const ColParams c,
+// the row-by-row pass spends 108 ALU instructions where this one spends about 48.
+//
+// kPerSm blocks per SM: two (up to 128 registers a thread) pass 4-5 % faster than three (up to
+// 80), but three cut some populations more evenly; the host takes the cheaper (column_cost).
+// Measured, us per generation with every qubit drawn: 4,096 x 100,000 248 with two and 260 with
+// three (the row-by-row form 424); 6,001 x 70,001 273 and 260 (441).
+template <int kForm, int kPerSm>
+__global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenParams p, const ColParams c,
                                                                                   int32_t G)
 {
     __shared__ uint32_t s_thr[kMaxThr];
@@ -808,7 +933,10 @@ __global__ void __launch_bounds__(kThreads, kForm == 2 ? 2 : 3) column_run_kerne
     __shared__ int32_t s_ok;
     __shared__ ColSlot s_slot;
     __shared__ int64_t s_fix[2];                  // item sums of the dropped quads
-    __shared__ uint32_t s_seg;
+    __shared__ uint32_t s_seg[2];
+    __shared__ float s_debt;                      // generations' worth of draws of fixed quads
+    __shared__ int32_t s_shorter;                 // build a shorter list
+    __shared__ int32_t s_row[kColRows];           // rows of the accumulators
     const int tid = threadIdx.x;
     load_thresholds(p, s_thr);
     for (int i = tid; i < 2 * kColRows; i += kThreads) {
@@ -822,10 +950,13 @@ __global__ void __launch_bounds__(kThreads, kForm == 2 ? 2 : 3) column_run_kerne
     const int grid = (int)gridDim.x;
     ColGeom m = column_geometry(nv, ns, p.np, grid);
     if (m.small) return;                          // the whole run is column_small_kernel's
+    ColHome h = column_home(m, grid);
+    if ((int)blockIdx.x >= m.nb) return;
     if (tid == 0) {
         s_fix[0] = (int64_t)c.head->fw;
         s_fix[1] = (int64_t)c.head->fv;
         s_slot = ColSlot{};
+        s_debt = 0.0f;
     }
     const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(s_thr);
     const uint32_t off_top = (uint32_t)(8 * p.K), k8 = off_top * 0x00010001u;
@@ -854,12 +985,17 @@ __global__ void __launch_bounds__(kThreads, kForm == 2 ? 2 : 3) column_run_kerne
         const int32_t t = t0 + g;
         if (g > 0) {
             // generation t - 1 is complete once every block has arrived
-            if (tid == 0) s_ok = column_wait(p, c.sync + ((t - 1) & 3), (unsigned int)m.nb, s_snap) ? 1 : 0;
+            if (tid == 0) {
+                s_ok = column_wait(p, c.sync + ((t - 1) & 3), (unsigned int)m.nb, s_snap) ? 1 : 0;
+                const uint32_t nq = 2u * nv + ns;
+                if (g >= g_check) s_debt += (float)s_snap.drops / (float)nq;
+                s_shorter = g >= g_check && (s_debt * (float)h.share >= 15.0f || s_snap.drops == nq) ? 1 : 0;
+                if (s_shorter) s_debt = 0.0f;
+            }
             __syncthreads();
             if (!s_ok) return;
             e = (int32_t)(0xffffffu - (uint32_t)(s_snap.key & 0xffffffull));
             const int64_t f = (int64_t)(s_snap.key >> 24) - kKeyBias;
-            const uint32_t drops = s_snap.drops;
             if (e < 0 || e >= p.np) {             // every row finishes in every generation
                 if (rec) atomicOr(p.error, kErrEliteRange);
                 e = 0;
@@ -876,10 +1012,10 @@ __global__ void __launch_bounds__(kThreads, kForm == 2 ? 2 : 3) column_run_kerne
                 if (p.gen_ns) p.gen_ns[g] = global_ns();
             }
             if (g == G || stop) break;
-            // A shorter list once a thirty-second of the quads are fixed (an eighth where a block
-            // keeps its item from generation to generation; a rebuild costs about 3 us).
-            const uint32_t nq = 2u * nv + ns;
-            if (g >= g_check && drops >= (m.queued ? nq / 32u : nq / 8u) && drops != 0u) {
+            // A shorter list once the passes spent on fixed quads have cost what building it costs
+            // (about 8 us; a pass of a block takes 0.55 us). The count is that of generation
+            // t - 2, whose angle indices every block can read by now.
+            if (s_shorter) {
                 if (!column_rebuild<kForm>(p, c, it, m.nb, m.items, nv, ns, cur, t, rebuilds, rb_target, &s_slot, &s_ok))
                     return;
                 g_check = g + 2;
@@ -891,8 +1027,8 @@ __global__ void __launch_bounds__(kThreads, kForm == 2 ? 2 : 3) column_run_kerne
                     s_fix[0] += (int64_t)s_slot.fw;
                     s_fix[1] += (int64_t)s_slot.fv;
                 }
+                const int before = m.nb;          // (blocks that have left do not come back)
                 m = column_geometry(nv, ns, p.np, grid);
-                b = tile_geometry(m.lanes, m.warps);
                 loaded = false;
                 if (m.small) {
                     if (rec) {
@@ -911,67 +1047,59 @@ __global__ void __launch_bounds__(kThreads, kForm == 2 ? 2 : 3) column_run_kerne
                     }
                     return;
                 }
+                h = column_home(m, before);
+                if ((int)blockIdx.x >= m.nb) return;
+                b = tile_geometry(m.lanes, m.warps);
             }
         }
         // Words are cleared two generations ahead: the blocks' parts of t + 1 may be written as
         // soon as their own of t are done.
         ColSync *const sy = c.sync + (t & 3);
-        if (rec) {
-            c.sync[(t + 2) & 3] = ColSync{};
-            c.qctr[(t + 2) & 3] = 0u;
-        }
+        if (rec) c.sync[(t + 2) & 3] = ColSync{};
         const uint2 *state = g == 0 ? c.canon : column_parity(c, p.svec, t + 1);
-        // The block's segments: with a queue, from a counter in order of decreasing size, round l
-        // of nb segments taking half of what is left (at least 4 passes each), so that the
-        // blocks, which do not progress equally, stay busy to the end; otherwise one fixed
-        // share of one tile's passes (its item stays in registers).
-        const uint32_t units = (uint32_t)m.ntile * (uint32_t)m.nu;
-        uint32_t u0 = 0u, u1 = 0u, lstart = 0u, level = 0u, size = max(units / (uint32_t)m.nb / 2u, 4u);
-        bool taken = false;
-        for (;;) {
-            if (u0 >= u1) {
-                if (m.queued) {
-                    if (tid == 0) s_seg = atomicAdd(c.qctr + (t & 3), 1u);
-                    __syncthreads();
-                    const uint32_t idx = s_seg;
-                    __syncthreads();
-                    while (level < idx / (uint32_t)m.nb) {
-                        lstart += size * (uint32_t)m.nb;
-                        size = max(size / 2u, 4u);
-                        ++level;
-                    }
-                    u0 = lstart + (idx - level * (uint32_t)m.nb) * size;
-                    if (u0 >= units) break;
-                    u1 = min(u0 + size, units);
-                } else {
-                    if (taken) break;
-                    taken = true;
-                    const uint32_t tile = blockIdx.x % (uint32_t)m.ntile, part = blockIdx.x / (uint32_t)m.ntile;
-                    const uint32_t parts = ((uint32_t)m.nb - tile + (uint32_t)m.ntile - 1u) / (uint32_t)m.ntile;
-                    u0 = tile * (uint32_t)m.nu + (uint32_t)((uint64_t)(uint32_t)m.nu * part / parts);
-                    u1 = tile * (uint32_t)m.nu + (uint32_t)((uint64_t)(uint32_t)m.nu * (part + 1u) / parts);
-                    if (u0 >= u1) break;
-                }
-            }
-            const uint32_t tile = u0 / (uint32_t)m.nu, ua = u0 - tile * (uint32_t)m.nu;
-            const uint32_t ub = min((uint32_t)m.nu, ua + (u1 - u0));
-            const int i = (int)tile * m.width + b.v_in;
+        for (int turn = 0; turn < h.turns; ++turn) {
+            const int tile = h.home + turn * h.stride;
+            unsigned int *const queue = c.qctr + (t & 3) * kColQueues + h.home;
+            if (h.queued && h.part == 0 && tid == 0) c.qctr[((t + 2) & 3) * kColQueues + h.home] = 0u;
+            const int i = tile * m.width + b.v_in;
             const bool active = b.v_in < m.width && i < m.items;
             if (!loaded) {
                 column_item<kForm>(p, it, column_list(c, p.svec, cur), nv, ns, i, active, state);
                 column_thresholds<kForm>(it, thr_bytes, off_top, T, top, base);
             }
-            loaded = !m.queued;
+            loaded = h.turns == 1;
             uint32_t x = 0u;
             if (g > 0) {
                 x = column_cip<kForm>(p, it, e, t, T, top, k8);
                 column_thresholds<kForm>(it, thr_bytes, off_top, T, top, base);
             }
-            if (ua == 0u)
+            if (h.part == 0)
                 column_lead<kForm>(p, c, it, x, t, improved, b.r_sub == 0 && active, &c.sync[(t + 1) & 3].drops);
-            column_rows<kForm>(p, m, b, it, T, base, (int)ua * m.rpp, min(p.np, (int)ub * m.rpp), (uint32_t)t, s_fix,
-                               &sy->key, s_acc32, s_acc64);
-            u0 += ub - ua;
+            // The sums of several pieces' rows are kept until the accumulators are full.
+            int ua, ub, used = 0;
+            column_piece(m, h, h.part, ua, ub);
+            for (uint32_t piece = 1u; ua < m.nu; ++piece) {
+                // the next piece's index arrives while this one is computed
+                uint32_t next = 0u;
+                if (h.queued && tid == 0) next = atomicAdd(queue, 1u);
+                const int rb = min(p.np, ub * m.rpp);
+                for (int ra = ua * m.rpp; ra < rb;) {
+                    const int n = min(kColRows - used, rb - ra);
+                    if (tid < n) s_row[used + tid] = ra + tid;
+                    column_rows<kForm>(p, c.one, m, b, it, T, base, ra, n, used, (uint32_t)t, s_acc32, s_acc64);
+                    ra += n;
+                    used += n;
+                    if (used == kColRows) {
+                        column_flush<kForm>(p, m.ntile, s_row, used, s_fix, &sy->key, s_acc32, s_acc64);
+                        used = 0;
+                    }
+                }
+                if (!h.queued) break;
+                if (tid == 0) s_seg[piece & 1u] = next;
+                __syncthreads();
+                column_piece(m, h, h.group + (int)s_seg[piece & 1u], ua, ub);
+            }
+            if (used) column_flush<kForm>(p, m.ntile, s_row, used, s_fix, &sy->key, s_acc32, s_acc64);
         }
         __syncthreads();
         if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(&sy->arrived) : "memory");
@@ -1039,12 +1167,13 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
     ColGeom m;
     BlockShare b;
     bool alone, posted, lead_share = false;
-    int tile = 0, row0 = 0, rows = 0, passes = 0, nb = 1;
+    int tile = 0, row0 = 0, rows = 0, passes = 0, nb = 1, most = 1;   // most: passes of the largest share
     auto cut = [&](int grid) {
         m = column_geometry(nv, ns, p.np, grid);
         const uint32_t units = (uint32_t)m.ntile * (uint32_t)m.nu;
         alone = m.items == 0 || (m.ntile == 1 && units <= (uint32_t)kColLocalPasses);
         nb = alone ? 1 : m.nb;
+        most = (int)((units + (uint32_t)nb - 1u) / (uint32_t)nb);
         // Rows of a single tile are complete within a block, so nothing but its best row's key
         // need reach the others: each block posts it with its generation number in one 16-byte
         // store and reads everyone's, which saves the key's atomic and the fence before an
@@ -1071,6 +1200,7 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
         column_thresholds<kForm>(it, thr_bytes, off_top, T, top, base);
     };
     int32_t g_check = g + 2;
+    float debt = 0.0f;                            // generations' worth of draws of fixed quads
     bool have = true;                             // generation t0 + g - 1's elite is known
     int q = 0;                                    // the pass of the pair below
     __syncthreads();
@@ -1113,8 +1243,12 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
                 if (p.gen_ns && rec) p.gen_ns[g] = global_ns();
                 if (g == G || stop) break;
                 have = true;
+                // A shorter list: when it halves (fewer blocks meet sooner), or when its passes have
+                // been worth the rebuild (about 5 us; a pass takes 0.3 us).
                 const uint32_t nq = 2u * nv + ns;
-                if (sn.drops >= nq / 8u && sn.drops != 0u && g >= g_check) {
+                if (g >= g_check) debt += (float)sn.drops / (float)nq;
+                if (g >= g_check && (2u * sn.drops >= nq || debt * (float)most >= 16.0f)) {
+                    debt = 0.0f;
                     if (rec) column_record(p, t - 1, e, f, improved, run, nv + ns);
                     // the posted wait orders nothing but the posts: the angle indices need a barrier
                     __syncthreads();
@@ -1160,7 +1294,7 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
             const uint32_t u[8] = {h ? c0.a : a0.a, h ? c0.b : a0.b, h ? c0.c : a0.c, h ? c0.d : a0.d,
                                    h ? c1.a : a1.a, h ? c1.b : a1.b, h ? c1.c : a1.c, h ? c1.d : a1.d};
             if (q + h >= passes) break;
-            ColSum<kForm> s = column_sum<kForm>(it, T, base, u);
+            ColSum<kForm> s = column_sum<kForm>(it, T, base, u, c.one);
             if (alone) {
                 uint32_t xb = 0u;
 #pragma unroll
@@ -1272,10 +1406,27 @@ __global__ void __launch_bounds__(kThreads) column_plane_kernel(const GenParams 
                 const uint8_t bits = (uint8_t)(quad_sides(sa) | (quad_sides(sb) << 4));
                 for (int r = ra; r < rb; ++r, x += p.xstride) *x = bits;
             } else {
+                // thresholds and the sides of the genes at pi/2 in registers, as in a run
+                const uint32_t sp[4] = {sa.x, sa.y, sb.x, sb.y};
+                uint32_t T[8], top = 0u;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t off = (i & 1) ? (sp[i >> 1] >> 16) : (sp[i >> 1] & 0xffffu);
+                    T[i] = *reinterpret_cast<const uint32_t *>(thr_bytes + off);      // 0 at both bounds
+                    if (off == off_top) top |= 1u << i;
+                }
+                const QuadWords wa = quad_words(p, 2u * (uint32_t)vec, (uint32_t)t);
+                const QuadWords wb = quad_words(p, 2u * (uint32_t)vec + 1u, (uint32_t)t);
+#pragma unroll 2
                 for (int r = ra; r < rb; ++r, x += p.xstride) {
-                    const Draw4 d0 = philox4x32_10_rk(2u * (uint32_t)vec, (uint32_t)r, (uint32_t)t, 0u, p.rk0, p.rk1);
-                    const Draw4 d1 = philox4x32_10_rk(2u * (uint32_t)vec + 1u, (uint32_t)r, (uint32_t)t, 0u, p.rk0, p.rk1);
-                    *x = (uint8_t)(observe_quad(d0, sa, thr_bytes, off_top) | (observe_quad(d1, sb, thr_bytes, off_top) << 4));
+                    const uint64_t z = row_product(p, (uint32_t)r, (uint32_t)t);
+                    const Draw4 d0 = quad_draw(p, wa, z), d1 = quad_draw(p, wb, z);
+                    const uint32_t u[8] = {d0.a, d0.b, d0.c, d0.d, d1.a, d1.b, d1.c, d1.d};
+                    uint32_t bits = top;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (u[i] < T[i]) bits |= 1u << i;
+                    *x = (uint8_t)bits;
                 }
             }
         }
@@ -1286,10 +1437,7 @@ __global__ void __launch_bounds__(kThreads) column_plane_kernel(const GenParams 
 __device__ __forceinline__ void column_clear_words(const ColParams &c)
 {
     for (int i = 0; i < 3; ++i) c.slot[i] = ColSlot{};
-    for (int i = 0; i < 4; ++i) {
-        c.sync[i] = ColSync{};
-        c.qctr[i] = 0u;
-    }
+    for (int i = 0; i < 4; ++i) c.sync[i] = ColSync{};
 }
 
 // Sums of the items of a fixed vector's quad (32-bit item arrays; zero on padding genes).
@@ -1321,6 +1469,7 @@ __global__ void __launch_bounds__(kThreads) column_end_kernel(const GenParams p,
     const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(s_thr);
     const uint32_t off_top = (uint32_t)(8 * p.K), k8 = off_top * 0x00010001u;
     for (int i = blockIdx.x * kThreads + threadIdx.x; i < 2 * kColPosted; i += gridDim.x * kThreads) c.post[i] = ColSync{};
+    for (int i = blockIdx.x * kThreads + threadIdx.x; i < 4 * kColQueues; i += gridDim.x * kThreads) c.qctr[i] = 0u;
     const bool ran = from_rows || c.ctl[kCtlRan] != 0;
     const bool rebuild = from_rows || (ran && c.ctl[kCtlRebuild] != 0);
     const int32_t t_last = c.ctl[kCtlLast], t0 = c.ctl[kCtlFirst];
@@ -1392,6 +1541,7 @@ __global__ void __launch_bounds__(kThreads) column_reset_kernel(const GenParams 
         column_list(c, p.svec, 0)[vec] = vec;
     }
     for (int i = i0; i < 2 * kColPosted; i += stride) c.post[i] = ColSync{};
+    for (int i = i0; i < 4 * kColQueues; i += stride) c.qctr[i] = 0u;
     if (i0 == 0) {
         ColSlot h{};
         h.nv = (unsigned int)p.svec;
