@@ -25,6 +25,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <queue>
 #include <unordered_map>
 #include <tuple>
 #include <new>
@@ -1131,7 +1132,7 @@ qieo_status run_column(qieo_instance *q, int32_t G)
         CUDA_TRY(cudaLaunchKernelEx(&cfg, column_small_fn(q->col_form), p, q->cp, std::min(chunk, G - done)));
         cudaLaunchAttribute attr1[1];
         cudaLaunchConfig_t plane = launch_config(q, dim3(tiles * parts), 0, attr1);
-        CUDA_TRY(cudaLaunchKernelEx(&plane, qieo::column_plane_kernel, q->gp, q->cp, tiles));
+        CUDA_TRY(cudaLaunchKernelEx(&plane, qieo::column_plane_kernel, q->gp, q->cp));
         CUDA_TRY(launch_column_end(q, 0));
     }
     q->state_valid = false;
@@ -2273,7 +2274,209 @@ qieo_status qieo_get_phase_times(qieo_instance *q, double ms[4], int64_t *genera
 // ---------------------------------------------------------------------------------------
 // Batches
 // ---------------------------------------------------------------------------------------
+namespace {
+
+// What the column form's batched kernels read of a set of members of one item form.
+struct ColumnBatch {
+    int form = 0, grid = 1;
+    std::vector<qieo::ColMember> members;
+    std::vector<qieo::ColTask> tasks, plane, end;
+    std::vector<int32_t> first;                     // tasks of block b: [first[b], first[b + 1])
+    const qieo::ColMember *d_members = nullptr;
+    const qieo::ColTask *d_tasks = nullptr, *d_plane = nullptr, *d_end = nullptr;
+    const int32_t *d_first = nullptr;
+};
+
+typedef void (*ColumnBatchFn)(const qieo::ColMember *, const qieo::ColTask *, const int32_t *, int32_t);
+ColumnBatchFn column_batch_fn(int form)
+{
+    return form == 0 ? &qieo::column_batch_kernel<0>
+                     : form == 1 ? &qieo::column_batch_kernel<1> : &qieo::column_batch_kernel<2>;
+}
+
+// Time of a generation of a member on s blocks, us: the chain from one generation's elite to the
+// next (2 to 4 us) and the passes of the block with the longest share (see column_geometry,
+// column_home). A pass takes 0.38 us with two blocks on the SM, and the list shortens during a
+// run; a tile that a block does not keep from generation to generation is loaded again. (Halving or
+// doubling either constant moves the time of a batch of 24, 96 or 256 members by at most 2 %.)
+constexpr double kBatchChainUs = 3.0, kBatchPassUs = 0.3;
+
+double column_member_time(const qieo_instance *q, int s)
+{
+    const int64_t items = q->svec;
+    int64_t ntile = 1, rpp = 1;
+    if (items > qieo::kThreads) ntile = (items + qieo::kThreads - 1) / qieo::kThreads;
+    else rpp = qieo::kThreads / pow2_ceil((int)items);
+    const int64_t nu = (q->np + rpp - 1) / rpp;
+    int64_t turns = 1, group = 1, cut = ntile;
+    if (ntile <= s) {
+        group = s / ntile;
+        if (ntile > 1) cut = s / group;
+        group = std::min(group, nu);
+    } else {
+        turns = (ntile + s - 1) / s;
+        cut = turns * s;
+    }
+    const double warps = ntile > 1 ? (double)(((items + cut - 1) / cut + 31) / 32) / 8.0 : 1.0;
+    return kBatchChainUs + (double)turns * ((double)((nu + group - 1) / group) * warps * kBatchPassUs + (turns > 1 ? 0.7 : 0.0));
+}
+
+// Cuts a cooperative grid's blocks among the members so that all blocks end at about the same time:
+// for a time per generation, a member that needs more than one block to keep it gets as many as
+// it needs, before all else on them, and the others follow, longest first, each on the block with
+// the least to do; the time is the smallest for which that works out
+// (a bisection).
+void plan_column_batch(const std::vector<qieo_instance *> &members, int sms, ColumnBatch &b)
+{
+    const int n = (int)members.size(), grid = b.grid;
+    b.members.clear();
+    std::vector<double> alone((size_t)n);
+    double lo = 0.0, total = 0.0, longest = 0.0;
+    for (int i = 0; i < n; ++i) {
+        qieo::ColMember m{};
+        m.p = members[(size_t)i]->gp;
+        m.c = members[(size_t)i]->cp;
+        b.members.push_back(m);
+        alone[(size_t)i] = column_member_time(members[(size_t)i], 1);
+        total += alone[(size_t)i];
+        longest = std::max(longest, alone[(size_t)i]);
+    }
+    std::vector<int> order((size_t)n);
+    for (int i = 0; i < n; ++i) order[(size_t)i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return alone[(size_t)x] > alone[(size_t)y]; });
+    typedef std::pair<double, int> Load;             // a block's time, the block
+    std::vector<std::vector<qieo::ColTask>> best, lists;
+    double hi = total / grid + longest;              // (every member on one block)
+    for (int round = 0; round < 14; ++round) {
+        const double t = round == 0 ? hi : 0.5 * (lo + hi);
+        lists.assign((size_t)grid, {});
+        int used = 0;
+        bool fits = true;
+        std::vector<int> singles;
+        std::priority_queue<Load, std::vector<Load>, std::greater<Load>> blocks;
+        for (int i : order) {
+            if (alone[(size_t)i] <= t) {
+                singles.push_back(i);
+                continue;
+            }
+            int need = std::max(2, (int)((alone[(size_t)i] - kBatchChainUs) / std::max(t - kBatchChainUs, 0.1)));
+            while (need <= grid - used && column_member_time(members[(size_t)i], need) > t) ++need;
+            if (need > grid - used) {
+                fits = false;
+                break;
+            }
+            const double each = column_member_time(members[(size_t)i], need);
+            for (int k = 0; k < need; ++k) {
+                lists[(size_t)(used + k)].push_back({i, k, need, 0});
+                blocks.push({each, used + k});
+            }
+            used += need;
+        }
+        for (int k = used; k < grid; ++k) blocks.push({0.0, k});
+        for (int i : singles) {
+            if (!fits) break;
+            Load l = blocks.top();
+            blocks.pop();
+            l.first += alone[(size_t)i];
+            // (at the first bound this always fits: the least loaded block has at most total / grid)
+            fits = l.first <= t || round == 0;
+            lists[(size_t)l.second].push_back({i, 0, 1, 0});
+            blocks.push(l);
+        }
+        if (fits) {
+            best = lists;
+            hi = t;
+        } else {
+            lo = t;
+        }
+        if (hi - lo < 0.02 * hi) break;
+    }
+    b.tasks.clear();
+    b.first.assign(1, 0);
+    for (const auto &l : best) {
+        b.tasks.insert(b.tasks.end(), l.begin(), l.end());
+        b.first.push_back((int32_t)b.tasks.size());
+    }
+    b.plane.clear();
+    b.end.clear();
+    // the allele planes: about four blocks per SM over all members, by bytes
+    double bytes = 0.0;
+    for (const qieo_instance *q : members) bytes += (double)q->np * q->svec;
+    for (int i = 0; i < n; ++i) {
+        const qieo_instance *q = members[(size_t)i];
+        const int tiles = plane_tiles(q);
+        const double share = (double)q->np * q->svec / bytes * 4.0 * sms;
+        const int parts = std::max(1, std::min(q->np, (int)(share / tiles + 0.5)));
+        for (int k = 0; k < tiles * parts; ++k) b.plane.push_back({i, k, tiles * parts, 0});
+        for (int k = 0; k < tiles; ++k) b.end.push_back({i, k, tiles, 0});
+    }
+}
+
+constexpr int kColumnBatchParts = 5;
+
+// Device layout of a plan: offsets of members | tasks | first | plane | end; the total.
+size_t column_batch_layout(const ColumnBatch &b, size_t at, size_t (&off)[kColumnBatchParts],
+                           const void *(&src)[kColumnBatchParts], size_t (&bytes)[kColumnBatchParts])
+{
+    src[0] = b.members.data(); bytes[0] = b.members.size() * sizeof(qieo::ColMember);
+    src[1] = b.tasks.data(); bytes[1] = b.tasks.size() * sizeof(qieo::ColTask);
+    src[2] = b.first.data(); bytes[2] = b.first.size() * sizeof(int32_t);
+    src[3] = b.plane.data(); bytes[3] = b.plane.size() * sizeof(qieo::ColTask);
+    src[4] = b.end.data(); bytes[4] = b.end.size() * sizeof(qieo::ColTask);
+    for (int i = 0; i < kColumnBatchParts; ++i) {
+        off[i] = at;
+        at = align_up(at + bytes[i], 256);
+    }
+    return at;
+}
+
+void place_column_batch(ColumnBatch &b, const char *dev, const size_t (&off)[kColumnBatchParts])
+{
+    b.d_members = (const qieo::ColMember *)(dev + off[0]);
+    b.d_tasks = (const qieo::ColTask *)(dev + off[1]);
+    b.d_first = (const int32_t *)(dev + off[2]);
+    b.d_plane = (const qieo::ColTask *)(dev + off[3]);
+    b.d_end = (const qieo::ColTask *)(dev + off[4]);
+}
+
+qieo_status column_batch_grid(const qieo_instance *q, ColumnBatch &b)
+{
+    int bps = 0;
+    qieo_status st = resident_blocks(q->device, reinterpret_cast<const void *>(column_batch_fn(b.form)), 0, &bps);
+    if (st != QIEO_OK) return st;
+    b.grid = q->sm_count * std::max(1, std::min(bps, 2));
+    return QIEO_OK;
+}
+
+// A run of the members of a plan: all generations in one cooperative launch, the allele planes, the
+// state between runs.
+qieo_status launch_column_batch(const ColumnBatch &b, int32_t G, cudaStream_t stream)
+{
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(b.grid);
+    cfg.blockDim = dim3(qieo::kThreads);
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CUDA_TRY(cudaLaunchKernelEx(&cfg, column_batch_fn(b.form), b.d_members, b.d_tasks, b.d_first, G));
+    qieo::column_batch_plane_kernel<<<(unsigned)b.plane.size(), qieo::kThreads, 0, stream>>>(b.d_members, b.d_plane);
+    CUDA_TRY(cudaGetLastError());
+    qieo::column_batch_end_kernel<<<(unsigned)b.end.size(), qieo::kThreads, 0, stream>>>(b.d_members, b.d_end);
+    CUDA_TRY(cudaGetLastError());
+    return QIEO_OK;
+}
+
+}  // namespace
+
 struct qieo_batch {
+    struct ColGroup {
+        std::vector<qieo_instance *> members;
+        ColumnBatch plan;
+        void *dev = nullptr;
+    };
     struct Group {
         bool narrow = false;
         int32_t rule = 0;
@@ -2289,6 +2492,8 @@ struct qieo_batch {
     bool persistent = false;   // runs are one cooperative launch per group (batch_run_kernel)
     std::vector<qieo_instance *> members;
     std::vector<Group> groups;
+    std::vector<ColGroup> col_groups;   // members in the column form, by item form
+    std::vector<char> as_column;        // per member: in col_groups
     int device = 0;
     cudaStream_t stream = nullptr;
     std::vector<cudaStream_t> other_streams;
@@ -2515,6 +2720,106 @@ qieo_status enqueue_batch_run(qieo_batch *bt, int32_t G)
     return QIEO_OK;
 }
 
+void free_groups(qieo_batch *bt)
+{
+    drop_batch_graphs(bt);
+    for (auto &g : bt->groups)
+        if (g.dev) cudaFree(g.dev);
+    for (auto &g : bt->col_groups)
+        if (g.dev) cudaFree(g.dev);
+    bt->groups.clear();
+    bt->col_groups.clear();
+}
+
+qieo_status build_col_group(qieo_batch *bt, qieo_batch::ColGroup &g)
+{
+    qieo_status st = column_batch_grid(g.members[0], g.plan);
+    if (st != QIEO_OK) return st;
+    plan_column_batch(g.members, g.members[0]->sm_count, g.plan);
+    size_t off[kColumnBatchParts], bytes[kColumnBatchParts];
+    const void *src[kColumnBatchParts];
+    const size_t total = column_batch_layout(g.plan, 0, off, src, bytes);
+    CUDA_TRY(cudaMalloc(&g.dev, total));
+    place_column_batch(g.plan, (const char *)g.dev, off);
+    for (int i = 0; i < kColumnBatchParts; ++i)
+        CUDA_TRY(cudaMemcpyAsync((char *)g.dev + off[i], src[i], bytes[i], cudaMemcpyHostToDevice, bt->stream));
+    return wait_stream(bt->stream);
+}
+
+// The members' words again, if any changed (a longer history, another wait limit).
+qieo_status upload_col_group(qieo_batch *bt, qieo_batch::ColGroup &g)
+{
+    bool same = true;
+    for (size_t i = 0; i < g.members.size(); ++i) {
+        qieo::ColMember m{};
+        m.p = g.members[i]->gp;
+        m.c = g.members[i]->cp;
+        if (std::memcmp(&m, &g.plan.members[i], sizeof m) == 0) continue;
+        g.plan.members[i] = m;
+        same = false;
+    }
+    if (same) return QIEO_OK;
+    CUDA_TRY(cudaMemcpyAsync(const_cast<qieo::ColMember *>(g.plan.d_members), g.plan.members.data(),
+                             g.members.size() * sizeof(qieo::ColMember), cudaMemcpyHostToDevice, bt->stream));
+    return QIEO_OK;
+}
+
+// Groups the members: those that run in the column form by item form, the others by item width and
+// rule. A member with QIEO_FLAG_PER_GENERATION keeps the whole batch row by row. Groups are built
+// again when a member changes form (a checkpoint whose rows differ).
+qieo_status group_members(qieo_batch *bt)
+{
+    bool per_gen = false;
+    for (const qieo_instance *q : bt->members) per_gen = per_gen || (q->flags & QIEO_FLAG_PER_GENERATION);
+    std::vector<char> as_column;
+    for (const qieo_instance *q : bt->members) as_column.push_back(!per_gen && use_column(q) ? 1 : 0);
+    if (as_column == bt->as_column) return QIEO_OK;
+    if (!bt->as_column.empty()) {
+        qieo_status st = wait_stream(bt->stream);
+        if (st != QIEO_OK) return st;
+        free_groups(bt);
+        bt->as_column.clear();
+    }
+    // One persistent launch per run unless a member asks for one launch per generation or
+    // uses the convergence test.
+    bt->persistent = true;
+    for (size_t i = 0; i < bt->members.size(); ++i) {
+        qieo_instance *q = bt->members[i];
+        if (as_column[i]) {
+            auto it = std::find_if(bt->col_groups.begin(), bt->col_groups.end(),
+                                   [&](const qieo_batch::ColGroup &g) { return g.plan.form == q->col_form; });
+            if (it == bt->col_groups.end()) {
+                bt->col_groups.emplace_back();
+                bt->col_groups.back().plan.form = q->col_form;
+                it = bt->col_groups.end() - 1;
+            }
+            it->members.push_back(q);
+            continue;
+        }
+        if (q->flags & (QIEO_FLAG_CONVERGE | QIEO_FLAG_PER_GENERATION)) bt->persistent = false;
+        auto it = std::find_if(bt->groups.begin(), bt->groups.end(), [&](const qieo_batch::Group &g) {
+            return g.narrow == (q->narrow != 0) && g.rule == q->rule;
+        });
+        if (it == bt->groups.end()) {
+            bt->groups.emplace_back();
+            bt->groups.back().narrow = q->narrow != 0;
+            bt->groups.back().rule = q->rule;
+            it = bt->groups.end() - 1;
+        }
+        it->members.push_back(q);
+    }
+    for (auto &g : bt->groups) {
+        qieo_status st = build_group(bt, g);
+        if (st != QIEO_OK) return st;
+    }
+    for (auto &g : bt->col_groups) {
+        qieo_status st = build_col_group(bt, g);
+        if (st != QIEO_OK) return st;
+    }
+    bt->as_column = as_column;
+    return QIEO_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -2554,27 +2859,8 @@ qieo_status qieo_create_batch(qieo_instance *const *instances, int32_t n, qieo_b
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&bt->ev_in, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&bt->ev_out, cudaEventDisableTiming);
     if (ce != cudaSuccess) return bail(fail(QIEO_ERR_CUDA, "batch setup: %s", cudaGetErrorString(ce)));
-    // One persistent launch per run unless a member asks for one launch per generation or
-    // uses the convergence test.
-    bt->persistent = true;
-    for (qieo_instance *q : members)
-        if (q->flags & (QIEO_FLAG_CONVERGE | QIEO_FLAG_PER_GENERATION)) bt->persistent = false;
-    for (qieo_instance *q : members) {
-        auto it = std::find_if(bt->groups.begin(), bt->groups.end(), [&](const qieo_batch::Group &g) {
-            return g.narrow == (q->narrow != 0) && g.rule == q->rule;
-        });
-        if (it == bt->groups.end()) {
-            bt->groups.emplace_back();
-            bt->groups.back().narrow = q->narrow != 0;
-            bt->groups.back().rule = q->rule;
-            it = bt->groups.end() - 1;
-        }
-        it->members.push_back(q);
-    }
-    for (auto &g : bt->groups) {
-        qieo_status st = build_group(bt, g);
-        if (st != QIEO_OK) return bail(st);
-    }
+    const qieo_status st = group_members(bt);
+    if (st != QIEO_OK) return bail(st);
     *out = bt;
     return QIEO_OK;
 }
@@ -2584,9 +2870,7 @@ qieo_status qieo_destroy_batch(qieo_batch *bt)
     if (!bt) return QIEO_OK;
     cudaSetDevice(bt->device);
     if (bt->stream) cudaStreamSynchronize(bt->stream);
-    drop_batch_graphs(bt);
-    for (auto &g : bt->groups)
-        if (g.dev) cudaFree(g.dev);
+    free_groups(bt);
     if (bt->ev_in) cudaEventDestroy(bt->ev_in);
     if (bt->ev_out) cudaEventDestroy(bt->ev_out);
     delete bt;
@@ -2604,22 +2888,38 @@ qieo_status qieo_batch_run(qieo_batch *bt, int32_t G)
         qieo_status st = ensure_history(q, q->t + G);
         if (st != QIEO_OK) return st;
     }
+    qieo_status grouped = group_members(bt);
+    if (grouped != QIEO_OK) return grouped;
     for (auto &g : bt->groups) {
         qieo_status st = upload_group(bt, g);
         if (st != QIEO_OK) return st;
     }
-    for (qieo_instance *q : bt->members) {       // the batched kernels read the full state
-        if (!q->col_mem) continue;
-        qieo_status st = ensure_state(q);
+    for (auto &g : bt->col_groups) {
+        qieo_status st = upload_col_group(bt, g);
         if (st != QIEO_OK) return st;
-        q->col_valid = false;
+    }
+    for (size_t i = 0; i < bt->members.size(); ++i) {
+        qieo_instance *q = bt->members[i];
+        if (!q->col_mem) continue;
+        qieo_status st = bt->as_column[i] ? ensure_column(q) : ensure_state(q);
+        if (st != QIEO_OK) return st;
+        (bt->as_column[i] ? q->state_valid : q->col_valid) = false;
     }
     for (cudaStream_t s : bt->other_streams) {   // pending work of the members' own streams
         CUDA_TRY(cudaEventRecord(bt->ev_in, s));
         CUDA_TRY(cudaStreamWaitEvent(bt->stream, bt->ev_in, 0));
     }
+    for (auto &g : bt->col_groups) {
+        // the words that count arrivals over a run have 32 bits: longer runs are split
+        const int32_t chunk = std::max(1, std::min(G, (1 << 30) / g.plan.grid));
+        for (int32_t done = 0; done < G; done += chunk) {
+            qieo_status st = launch_column_batch(g.plan, std::min(chunk, G - done), bt->stream);
+            if (st != QIEO_OK) return st;
+        }
+    }
     const bool first_time = bt->run_lengths_seen[G]++ == 0;
-    if (bt->persistent) {
+    if (bt->groups.empty()) {
+    } else if (bt->persistent) {
         qieo_status st = enqueue_batch_persistent(bt, G);
         if (st != QIEO_OK) return st;
     } else if (first_time && !bt->graphs.count(G)) {
@@ -2648,8 +2948,8 @@ qieo_status qieo_batch_run(qieo_batch *bt, int32_t G)
         }
         CUDA_TRY(cudaGraphLaunch(exec, bt->stream));
     }
-    for (qieo_instance *q : bt->members) {   // the batched kernels do not keep F
-        qieo_status st = clear_fword(q, bt->stream);
+    for (size_t i = 0; i < bt->members.size(); ++i) {   // the row-by-row batched kernels do not keep F
+        qieo_status st = bt->as_column[i] ? QIEO_OK : clear_fword(bt->members[i], bt->stream);
         if (st != QIEO_OK) return st;
     }
     if (!bt->other_streams.empty()) {

@@ -158,7 +158,7 @@ struct ColHome {
     int round, start, size;       // the round of the last piece, its first pass and its pieces' passes
 };
 
-__device__ __forceinline__ ColHome column_home(ColGeom &m, int grid)
+__device__ __forceinline__ ColHome column_home(ColGeom &m, int block, int grid)
 {
     ColHome h;
     h.turns = 1;
@@ -175,8 +175,8 @@ __device__ __forceinline__ ColHome column_home(ColGeom &m, int grid)
     if (m.ntile > 1) m.width = (m.items + m.ntile - 1) / m.ntile;
     h.group = min(h.group, m.nu);
     m.nb = h.stride * h.group;
-    h.home = (int)(blockIdx.x % (unsigned int)h.stride);
-    h.part = (int)(blockIdx.x / (unsigned int)h.stride);
+    h.home = (int)((unsigned int)block % (unsigned int)h.stride);
+    h.part = (int)((unsigned int)block / (unsigned int)h.stride);
     h.share = m.nu / h.group;
     h.queued = h.share >= kColQueueShare && h.group > 1;
     return h;
@@ -298,13 +298,27 @@ __device__ __forceinline__ QuadWords quad_words(const GenParams &p, uint32_t q, 
     return w;
 }
 
-__device__ __forceinline__ uint64_t row_product(const GenParams &p, uint32_t row, uint32_t t)
+// The round keys of the rest, and of the row's product.
+struct RowKeys {
+    uint32_t hi;                  // first round: the high word of M1 t, with the key
+    uint32_t k0[7], k1[7];        // rounds 3 .. 9
+};
+
+__device__ __forceinline__ RowKeys row_keys(const GenParams &p, uint32_t t)
 {
-    const uint32_t hi_t = (uint32_t)(((uint64_t)kPhiloxM1 * t) >> 32);
-    return (uint64_t)kPhiloxM0 * (hi_t ^ row ^ p.rk0[0]);
+    RowKeys k;
+    k.hi = (uint32_t)(((uint64_t)kPhiloxM1 * t) >> 32) ^ p.rk0[0];
+#pragma unroll
+    for (int r = 0; r < 7; ++r) {
+        k.k0[r] = p.rk0[r + 3];
+        k.k1[r] = p.rk1[r + 3];
+    }
+    return k;
 }
 
-__device__ __forceinline__ Draw4 quad_draw(const GenParams &p, const QuadWords &w, uint64_t z)
+__device__ __forceinline__ uint64_t row_product(const RowKeys &k, uint32_t row) { return (uint64_t)kPhiloxM0 * (k.hi ^ row); }
+
+__device__ __forceinline__ Draw4 quad_draw(const RowKeys &k, const QuadWords &w, uint64_t z)
 {
     const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(z >> 32) ^ w.b);
     uint32_t c0 = (uint32_t)(p1 >> 32) ^ w.d, c1 = (uint32_t)p1, c2 = (uint32_t)z ^ w.h, c3 = w.l;
@@ -312,8 +326,8 @@ __device__ __forceinline__ Draw4 quad_draw(const GenParams &p, const QuadWords &
     for (int r = 3; r < 10; ++r) {
         const uint64_t a = (uint64_t)kPhiloxM0 * (uint64_t)c0;
         const uint64_t b = (uint64_t)kPhiloxM1 * (uint64_t)c2;
-        const uint32_t n0 = (uint32_t)(b >> 32) ^ c1 ^ p.rk0[r];
-        const uint32_t n2 = (uint32_t)(a >> 32) ^ c3 ^ p.rk1[r];
+        const uint32_t n0 = (uint32_t)(b >> 32) ^ c1 ^ k.k0[r - 3];
+        const uint32_t n2 = (uint32_t)(a >> 32) ^ c3 ^ k.k1[r - 3];
         c1 = (uint32_t)b;
         c3 = (uint32_t)a;
         c0 = n0;
@@ -398,12 +412,12 @@ __device__ __forceinline__ ColSum<kForm> column_sum(const ColItem<kForm> &it, co
 }
 
 template <int kForm>
-__device__ __forceinline__ ColSum<kForm> column_row(const GenParams &p, uint32_t one, const ColItem<kForm> &it, const uint32_t (&T)[8],
+__device__ __forceinline__ ColSum<kForm> column_row(const RowKeys &k, uint32_t one, const ColItem<kForm> &it, const uint32_t (&T)[8],
                                                     const ColSum<kForm> &base, const QuadWords &wa,
-                                                    const QuadWords &wb, uint32_t row, uint32_t t)
+                                                    const QuadWords &wb, uint32_t row)
 {
-    const uint64_t z = row_product(p, row, t);
-    const Draw4 r0 = quad_draw(p, wa, z), r1 = quad_draw(p, wb, z);
+    const uint64_t z = row_product(k, row);
+    const Draw4 r0 = quad_draw(k, wa, z), r1 = quad_draw(k, wb, z);
     const uint32_t u[8] = {r0.a, r0.b, r0.c, r0.d, r1.a, r1.b, r1.c, r1.d};
     return column_sum<kForm>(it, T, base, u, one);
 }
@@ -516,6 +530,7 @@ __device__ __forceinline__ void column_rows(const GenParams &p, uint32_t one, co
                                             unsigned long long *s_acc64)
 {
     const int lane = threadIdx.x & 31;
+    const RowKeys k = row_keys(p, t);
     const QuadWords wa = quad_words(p, (uint32_t)it.qa, t), wb = quad_words(p, (uint32_t)it.qb, t);
     if (m.lanes == 32) {
         // Two rows per step (four independent Philox chains). Lane i keeps the warp's sums of
@@ -531,15 +546,15 @@ __device__ __forceinline__ void column_rows(const GenParams &p, uint32_t one, co
             int q = 0;
 #pragma unroll 1
             for (; q + 1 < nq; q += 2) {
-                const ColSum<kForm> a = column_row<kForm>(p, one, it, T, base, wa, wb, row, t);
-                const ColSum<kForm> c = column_row<kForm>(p, one, it, T, base, wa, wb, row + step, t);
+                const ColSum<kForm> a = column_row<kForm>(k, one, it, T, base, wa, wb, row);
+                const ColSum<kForm> c = column_row<kForm>(k, one, it, T, base, wa, wb, row + step);
                 row += 2u * step;
                 const ColSum<kForm> as = column_warp_sum<kForm>(a), cs = column_warp_sum<kForm>(c);
                 if (lane == q) mine = as;
                 if (lane == q + 1) mine = cs;
             }
             if (q < nq) {
-                const ColSum<kForm> as = column_warp_sum<kForm>(column_row<kForm>(p, one, it, T, base, wa, wb, row, t));
+                const ColSum<kForm> as = column_warp_sum<kForm>(column_row<kForm>(k, one, it, T, base, wa, wb, row));
                 row += step;
                 if (lane == q) mine = as;
             }
@@ -548,7 +563,7 @@ __device__ __forceinline__ void column_rows(const GenParams &p, uint32_t one, co
         }
     } else {
         for (int q = b.r_sub; q < n + b.r_sub; q += m.rpp) {         // the same trips for every thread
-            ColSum<kForm> s = column_row<kForm>(p, one, it, T, base, wa, wb, (uint32_t)(ra + q), t);
+            ColSum<kForm> s = column_row<kForm>(k, one, it, T, base, wa, wb, (uint32_t)(ra + q));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 if (o < m.lanes) {
@@ -773,7 +788,7 @@ __device__ __forceinline__ bool column_wait(const GenParams &p, const ColSync *s
             out.drops = (unsigned int)(hi >> 32);
             return true;
         }
-        if ((n & 15u) == 15u && (ld_acquire(p.error) != 0 || global_ns() > deadline)) break;
+        if (global_ns() > deadline || ((n & 15u) == 15u && ld_acquire(p.error) != 0)) break;
     }
     atomicOr(p.error, kErrBarrierTimeout);
     return false;
@@ -784,8 +799,8 @@ __device__ __forceinline__ bool column_wait(const GenParams &p, const ColSync *s
 // fixed then leave, and both parities hold their state. counts: the list's, in shared memory (and
 // the item sums of the quads that left). Whole block; false when a wait ran out.
 template <int kForm>
-__device__ __forceinline__ bool column_rebuild(const GenParams &p, const ColParams &c, ColItem<kForm> &it, int nb,
-                                               int items, uint32_t nv, uint32_t ns, int cur, int32_t t,
+__device__ __forceinline__ bool column_rebuild(const GenParams &p, const ColParams &c, ColItem<kForm> &it, int block,
+                                               int nb, int items, uint32_t nv, uint32_t ns, int cur, int32_t t,
                                                uint32_t rebuilds, uint32_t &target, ColSlot *counts, int32_t *s_ok)
 {
     const uint32_t off_top = (uint32_t)(8 * p.K);
@@ -793,7 +808,7 @@ __device__ __forceinline__ bool column_rebuild(const GenParams &p, const ColPara
     ColSlot *slot = nb > 1 ? c.slot + rebuilds % 3u : counts;
     const uint2 *state = column_parity(c, p.svec, t - 2);
     uint2 *other = column_parity(c, p.svec, t - 1);
-    for (int i0 = (int)blockIdx.x * kThreads; i0 < items; i0 += nb * kThreads) {
+    for (int i0 = block * kThreads; i0 < items; i0 += nb * kThreads) {
         const int i = i0 + tid;
         const bool mine = i < items;
         column_item<kForm>(p, it, column_list(c, p.svec, cur), nv, ns, i, mine, state);
@@ -816,7 +831,7 @@ __device__ __forceinline__ bool column_rebuild(const GenParams &p, const ColPara
             counts->ns = __ldcg(&slot->ns);
             counts->fw = __ldcg(&slot->fw);
             counts->fv = __ldcg(&slot->fv);
-            if (blockIdx.x == 0) c.slot[(rebuilds + 1u) % 3u] = ColSlot{};
+            if (block == 0) c.slot[(rebuilds + 1u) % 3u] = ColSlot{};
         }
     }
     __syncthreads();
@@ -892,10 +907,10 @@ __device__ __forceinline__ void column_finish(const GenParams &p, const ColParam
 
 // Start of a run or of its rest: whether there is anything to do, and the words that say how it
 // stands. Whole block; head values are read by every thread.
-__device__ __forceinline__ bool column_stopped(const GenParams &p, const ColParams &c)
+__device__ __forceinline__ bool column_stopped(const GenParams &p, const ColParams &c, int block)
 {
     if (!p.converge || *(volatile const int32_t *)(p.conv + 2) == kRunning) return false;
-    if (blockIdx.x == 0 && threadIdx.x == 0) c.ctl[kCtlRan] = 0;
+    if (block == 0 && threadIdx.x == 0) c.ctl[kCtlRan] = 0;
     return true;
 }
 
@@ -907,6 +922,21 @@ __device__ __forceinline__ void column_begin(const GenParams &p, const ColParams
     c.ctl[kCtlEarly] = 0;
     if (p.gen_ns) p.gen_ns[0] = global_ns();
 }
+
+template <int kForm>
+struct ColRunShared {
+    uint32_t thr[kMaxThr];
+    unsigned long long acc64[kForm == 2 ? 2 * kColRows : 1];
+    uint32_t acc32[kForm == 2 ? 1 : 2 * kColRows];
+    ColSync snap;                 // what thread 0 read of the generation before
+    int32_t ok;
+    ColSlot slot;
+    int64_t fix[2];               // item sums of the dropped quads
+    uint32_t seg[2];
+    float debt;                   // generations' worth of draws of fixed quads
+    int32_t shorter;              // build a shorter list
+    int32_t row[kColRows];        // rows of the accumulators
+};
 
 // The generations of a run whose blocks have several passes each (at least kColSmallShare):
 // every block has a home tile (ColHome). Every block follows the same sequence of lists, elites and
@@ -922,43 +952,31 @@ __device__ __forceinline__ void column_begin(const GenParams &p, const ColParams
 // 80), but three cut some populations more evenly; the host takes the cheaper (column_cost).
 // Measured, us per generation with every qubit drawn: 4,096 x 100,000 248 with two and 260 with
 // three (the row-by-row form 424); 6,001 x 70,001 273 and 260 (441).
-template <int kForm, int kPerSm>
-__global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenParams p, const ColParams c,
-                                                                                  int32_t G)
+template <int kForm, bool kMember>
+__device__ __forceinline__ void column_run(const GenParams &p, const ColParams &c, int32_t G, int block, int grid,
+                                           ColRunShared<kForm> &sh)
 {
-    __shared__ uint32_t s_thr[kMaxThr];
-    __shared__ unsigned long long s_acc64[kForm == 2 ? 2 * kColRows : 1];
-    __shared__ uint32_t s_acc32[kForm == 2 ? 1 : 2 * kColRows];
-    __shared__ ColSync s_snap;                    // what thread 0 read of the generation before
-    __shared__ int32_t s_ok;
-    __shared__ ColSlot s_slot;
-    __shared__ int64_t s_fix[2];                  // item sums of the dropped quads
-    __shared__ uint32_t s_seg[2];
-    __shared__ float s_debt;                      // generations' worth of draws of fixed quads
-    __shared__ int32_t s_shorter;                 // build a shorter list
-    __shared__ int32_t s_row[kColRows];           // rows of the accumulators
     const int tid = threadIdx.x;
-    load_thresholds(p, s_thr);
+    load_thresholds(p, sh.thr);
     for (int i = tid; i < 2 * kColRows; i += kThreads) {
-        if constexpr (kForm == 2) s_acc64[i] = 0ull;
-        else s_acc32[i] = 0u;
+        if constexpr (kForm == 2) sh.acc64[i] = 0ull;
+        else sh.acc32[i] = 0u;
     }
-    grid_dependency_wait();
-    if (column_stopped(p, c)) return;
+    if (!kMember) grid_dependency_wait();
+    if (column_stopped(p, c, block)) return;
     const int32_t t0 = *p.gen;
     uint32_t nv = c.head->nv, ns = c.head->ns;
-    const int grid = (int)gridDim.x;
     ColGeom m = column_geometry(nv, ns, p.np, grid);
-    if (m.small) return;                          // the whole run is column_small_kernel's
-    ColHome h = column_home(m, grid);
-    if ((int)blockIdx.x >= m.nb) return;
+    if (!kMember && m.small) return;              // the whole run is column_small_kernel's
+    ColHome h = column_home(m, block, grid);
+    if (block >= m.nb) return;
     if (tid == 0) {
-        s_fix[0] = (int64_t)c.head->fw;
-        s_fix[1] = (int64_t)c.head->fv;
-        s_slot = ColSlot{};
-        s_debt = 0.0f;
+        sh.fix[0] = (int64_t)c.head->fw;
+        sh.fix[1] = (int64_t)c.head->fv;
+        sh.slot = ColSlot{};
+        sh.debt = 0.0f;
     }
-    const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(s_thr);
+    const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(sh.thr);
     const uint32_t off_top = (uint32_t)(8 * p.K), k8 = off_top * 0x00010001u;
     // the records' running values, the same in every block
     int64_t best_f = __ldcg(p.best + 1) < 0 ? INT64_MIN : __ldcg(p.best), prev_f = 0;
@@ -967,8 +985,8 @@ __global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenP
         run = __ldcg(p.conv + ((t0 - 1) & 1));
         prev_f = __ldcg(p.hist_f + t0 - 1);
     }
-    const bool rec = blockIdx.x == 0 && tid == 0;
-    if (rec) column_begin(p, c, t0, true);
+    const bool rec = block == 0 && tid == 0;
+    if (rec) column_begin(p, c, t0, nv + ns != 0u);
     BlockShare b = tile_geometry(m.lanes, m.warps);
     int cur = 0;
     uint32_t rebuilds = 0u, rb_target = 0u;
@@ -981,21 +999,21 @@ __global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenP
     bool improved = false, stop = false;
     __syncthreads();
 
-    for (;; ++g) {
+    for (; !kMember || m.items != 0; ++g) {
         const int32_t t = t0 + g;
         if (g > 0) {
             // generation t - 1 is complete once every block has arrived
             if (tid == 0) {
-                s_ok = column_wait(p, c.sync + ((t - 1) & 3), (unsigned int)m.nb, s_snap) ? 1 : 0;
+                sh.ok = column_wait(p, c.sync + ((t - 1) & 3), (unsigned int)m.nb, sh.snap) ? 1 : 0;
                 const uint32_t nq = 2u * nv + ns;
-                if (g >= g_check) s_debt += (float)s_snap.drops / (float)nq;
-                s_shorter = g >= g_check && (s_debt * (float)h.share >= 15.0f || s_snap.drops == nq) ? 1 : 0;
-                if (s_shorter) s_debt = 0.0f;
+                if (g >= g_check) sh.debt += (float)sh.snap.drops / (float)nq;
+                sh.shorter = g >= g_check && (sh.debt * (float)h.share >= 15.0f || sh.snap.drops == nq) ? 1 : 0;
+                if (sh.shorter) sh.debt = 0.0f;
             }
             __syncthreads();
-            if (!s_ok) return;
-            e = (int32_t)(0xffffffu - (uint32_t)(s_snap.key & 0xffffffull));
-            const int64_t f = (int64_t)(s_snap.key >> 24) - kKeyBias;
+            if (!sh.ok) return;
+            e = (int32_t)(0xffffffu - (uint32_t)(sh.snap.key & 0xffffffull));
+            const int64_t f = (int64_t)(sh.snap.key >> 24) - kKeyBias;
             if (e < 0 || e >= p.np) {             // every row finishes in every generation
                 if (rec) atomicOr(p.error, kErrEliteRange);
                 e = 0;
@@ -1015,22 +1033,23 @@ __global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenP
             // A shorter list once the passes spent on fixed quads have cost what building it costs
             // (about 8 us; a pass of a block takes 0.55 us). The count is that of generation
             // t - 2, whose angle indices every block can read by now.
-            if (s_shorter) {
-                if (!column_rebuild<kForm>(p, c, it, m.nb, m.items, nv, ns, cur, t, rebuilds, rb_target, &s_slot, &s_ok))
+            if (sh.shorter) {
+                if (!column_rebuild<kForm>(p, c, it, block, m.nb, m.items, nv, ns, cur, t, rebuilds, rb_target, &sh.slot,
+                                           &sh.ok))
                     return;
                 g_check = g + 2;
                 ++rebuilds;
                 cur ^= 1;
-                nv = s_slot.nv;
-                ns = s_slot.ns;
+                nv = sh.slot.nv;
+                ns = sh.slot.ns;
                 if (tid == 0) {
-                    s_fix[0] += (int64_t)s_slot.fw;
-                    s_fix[1] += (int64_t)s_slot.fv;
+                    sh.fix[0] += (int64_t)sh.slot.fw;
+                    sh.fix[1] += (int64_t)sh.slot.fv;
                 }
                 const int before = m.nb;          // (blocks that have left do not come back)
                 m = column_geometry(nv, ns, p.np, grid);
                 loaded = false;
-                if (m.small) {
+                if (!kMember && m.small) {
                     if (rec) {
                         c.ctl[kCtlGen] = g;
                         c.ctl[kCtlCur] = cur;
@@ -1040,16 +1059,21 @@ __global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenP
                         ColSlot r{};
                         r.nv = nv;
                         r.ns = ns;
-                        r.fw = (unsigned long long)s_fix[0];
-                        r.fv = (unsigned long long)s_fix[1];
+                        r.fw = (unsigned long long)sh.fix[0];
+                        r.fv = (unsigned long long)sh.fix[1];
                         *c.rest = r;
                         c.ctl[kCtlPhase] = 1;
                     }
                     return;
                 }
-                h = column_home(m, before);
-                if ((int)blockIdx.x >= m.nb) return;
+                h = column_home(m, block, before);
+                if (block >= m.nb) return;
                 b = tile_geometry(m.lanes, m.warps);
+                if (kMember) {
+                    __syncthreads();
+                    if (tid == 0) sh.slot = ColSlot{};
+                    if (m.items == 0) break;
+                }
             }
         }
         // Words are cleared two generations ahead: the blocks' parts of t + 1 may be written as
@@ -1085,27 +1109,35 @@ __global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenP
                 const int rb = min(p.np, ub * m.rpp);
                 for (int ra = ua * m.rpp; ra < rb;) {
                     const int n = min(kColRows - used, rb - ra);
-                    if (tid < n) s_row[used + tid] = ra + tid;
-                    column_rows<kForm>(p, c.one, m, b, it, T, base, ra, n, used, (uint32_t)t, s_acc32, s_acc64);
+                    if (tid < n) sh.row[used + tid] = ra + tid;
+                    column_rows<kForm>(p, c.one, m, b, it, T, base, ra, n, used, (uint32_t)t, sh.acc32, sh.acc64);
                     ra += n;
                     used += n;
                     if (used == kColRows) {
-                        column_flush<kForm>(p, m.ntile, s_row, used, s_fix, &sy->key, s_acc32, s_acc64);
+                        column_flush<kForm>(p, m.ntile, sh.row, used, sh.fix, &sy->key, sh.acc32, sh.acc64);
                         used = 0;
                     }
                 }
                 if (!h.queued) break;
-                if (tid == 0) s_seg[piece & 1u] = next;
+                if (tid == 0) sh.seg[piece & 1u] = next;
                 __syncthreads();
-                column_piece(m, h, h.group + (int)s_seg[piece & 1u], ua, ub);
+                column_piece(m, h, h.group + (int)sh.seg[piece & 1u], ua, ub);
             }
-            if (used) column_flush<kForm>(p, m.ntile, s_row, used, s_fix, &sy->key, s_acc32, s_acc64);
+            if (used) column_flush<kForm>(p, m.ntile, sh.row, used, sh.fix, &sy->key, sh.acc32, sh.acc64);
         }
         __syncthreads();
         if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(&sy->arrived) : "memory");
     }
-    if (blockIdx.x == 0) column_finish(p, c, t0, g, G, t0 + g - 1, true, stop, best_f, prev_f, run, s_fix);
-    if (rec) c.ctl[kCtlPhase] = 2;
+    if (kMember) __syncthreads();
+    if (block == 0) column_finish(p, c, t0, g, G, t0 + g - 1, !kMember || m.items != 0, stop, best_f, prev_f, run, sh.fix);
+    if (!kMember && rec) c.ctl[kCtlPhase] = 2;
+}
+
+template <int kForm, int kPerSm>
+__global__ void __launch_bounds__(kThreads, kPerSm) column_run_kernel(const GenParams p, const ColParams c, int32_t G)
+{
+    __shared__ ColRunShared<kForm> sh;
+    column_run<kForm, false>(p, c, G, (int)blockIdx.x, (int)gridDim.x, sh);
 }
 
 // The generations of a run (or of the rest of one) in which a block has at most a few passes: bound
@@ -1137,7 +1169,7 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
     }
     grid_dependency_wait();
     const int32_t phase = c.ctl[kCtlPhase];
-    if (phase == 2 || (phase == 0 && column_stopped(p, c))) return;
+    if (phase == 2 || (phase == 0 && column_stopped(p, c, (int)blockIdx.x))) return;
     const int32_t t0 = phase ? c.ctl[kCtlFirst] : *p.gen;
     const ColSlot *from = phase ? c.rest : c.head;
     uint32_t nv = from->nv, ns = from->ns;
@@ -1253,7 +1285,8 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
                     // the posted wait orders nothing but the posts: the angle indices need a barrier
                     __syncthreads();
                     if (posted && !column_barrier(p, c, nb, rb_target, &s_ok)) return;
-                    if (!column_rebuild<kForm>(p, c, it, nb, m.items, nv, ns, cur, t, rebuilds, rb_target, &s_slot, &s_ok))
+                    if (!column_rebuild<kForm>(p, c, it, (int)blockIdx.x, nb, m.items, nv, ns, cur, t, rebuilds, rb_target,
+                                               &s_slot, &s_ok))
                         return;
                     g_check = g + 2;
                     ++rebuilds;
@@ -1379,19 +1412,17 @@ __device__ __forceinline__ uint2 observed_quad(const ColParams &c, int32_t svec,
 // The allele plane of the run's last generation (and, when the run stopped early, of the one
 // before, which the plane of the other parity holds): byte v of row r is the alleles of vector
 // v. A thread keeps one vector for its rows; vectors at the bounds store their sides.
-__global__ void __launch_bounds__(kThreads) column_plane_kernel(const GenParams p, const ColParams c, int32_t tiles)
+__device__ __forceinline__ void column_plane(const GenParams &p, const ColParams &c, int block, int blocks,
+                                             const uint32_t *s_thr)
 {
-    __shared__ uint32_t s_thr[kMaxThr];
-    load_thresholds(p, s_thr);
-    grid_dependency_wait();
-    __syncthreads();
     if (!c.ctl[kCtlRan]) return;
     // no block of this launch reads the head; the next launch fills it again
-    if (blockIdx.x == 0 && threadIdx.x == 0 && c.ctl[kCtlRebuild]) *c.head = ColSlot{};
+    if (block == 0 && threadIdx.x == 0 && c.ctl[kCtlRebuild]) *c.head = ColSlot{};
+    const int tiles = (p.svec + kThreads - 1) / kThreads;
     const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(s_thr);
     const uint32_t off_top = (uint32_t)(8 * p.K);
-    const int tile = (int)(blockIdx.x % (unsigned int)tiles), part = (int)(blockIdx.x / (unsigned int)tiles);
-    const int parts = (int)gridDim.x / tiles;
+    const int tile = block % tiles, part = block / tiles;
+    const int parts = blocks / tiles;
     if (part >= parts) return;
     const int ra = (int)((int64_t)p.np * part / parts), rb = (int)((int64_t)p.np * (part + 1) / parts);
     const int vec = tile * kThreads + (int)threadIdx.x;
@@ -1415,12 +1446,13 @@ __global__ void __launch_bounds__(kThreads) column_plane_kernel(const GenParams 
                     T[i] = *reinterpret_cast<const uint32_t *>(thr_bytes + off);      // 0 at both bounds
                     if (off == off_top) top |= 1u << i;
                 }
+                const RowKeys key = row_keys(p, (uint32_t)t);
                 const QuadWords wa = quad_words(p, 2u * (uint32_t)vec, (uint32_t)t);
                 const QuadWords wb = quad_words(p, 2u * (uint32_t)vec + 1u, (uint32_t)t);
 #pragma unroll 2
                 for (int r = ra; r < rb; ++r, x += p.xstride) {
-                    const uint64_t z = row_product(p, (uint32_t)r, (uint32_t)t);
-                    const Draw4 d0 = quad_draw(p, wa, z), d1 = quad_draw(p, wb, z);
+                    const uint64_t z = row_product(key, (uint32_t)r);
+                    const Draw4 d0 = quad_draw(key, wa, z), d1 = quad_draw(key, wb, z);
                     const uint32_t u[8] = {d0.a, d0.b, d0.c, d0.d, d1.a, d1.b, d1.c, d1.d};
                     uint32_t bits = top;
 #pragma unroll
@@ -1431,6 +1463,15 @@ __global__ void __launch_bounds__(kThreads) column_plane_kernel(const GenParams 
             }
         }
     }
+}
+
+__global__ void __launch_bounds__(kThreads) column_plane_kernel(const GenParams p, const ColParams c)
+{
+    __shared__ uint32_t s_thr[kMaxThr];
+    load_thresholds(p, s_thr);
+    grid_dependency_wait();
+    __syncthreads();
+    column_plane(p, c, (int)blockIdx.x, (int)gridDim.x, s_thr);
     allow_dependent_launch();
 }
 
@@ -1460,22 +1501,19 @@ __device__ __forceinline__ void quad_sums(const GenParams &p, int q, uint2 s, in
 // starts with; the last block advances the generation counter and clears the run's words.
 // from_rows: instead, the state between runs is taken from row 0 of the full state (whose rows
 // are equal), after a run in a row-by-row form or a checkpoint.
-__global__ void __launch_bounds__(kThreads) column_end_kernel(const GenParams p, const ColParams c, int32_t from_rows)
+__device__ __forceinline__ void column_end(const GenParams &p, const ColParams &c, int32_t from_rows, int block,
+                                           int blocks, const uint32_t *s_thr)
 {
-    __shared__ uint32_t s_thr[kMaxThr];
-    load_thresholds(p, s_thr);
-    grid_dependency_wait();
-    __syncthreads();
     const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(s_thr);
     const uint32_t off_top = (uint32_t)(8 * p.K), k8 = off_top * 0x00010001u;
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < 2 * kColPosted; i += gridDim.x * kThreads) c.post[i] = ColSync{};
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < 4 * kColQueues; i += gridDim.x * kThreads) c.qctr[i] = 0u;
+    for (int i = block * kThreads + threadIdx.x; i < 2 * kColPosted; i += blocks * kThreads) c.post[i] = ColSync{};
+    for (int i = block * kThreads + threadIdx.x; i < 4 * kColQueues; i += blocks * kThreads) c.qctr[i] = 0u;
     const bool ran = from_rows || c.ctl[kCtlRan] != 0;
     const bool rebuild = from_rows || (ran && c.ctl[kCtlRebuild] != 0);
     const int32_t t_last = c.ctl[kCtlLast], t0 = c.ctl[kCtlFirst];
     const int32_t e = *p.elite_idx;
     const int64_t tb = p.best[1];
-    const int vec = blockIdx.x * kThreads + threadIdx.x;
+    const int vec = block * kThreads + threadIdx.x;
     if (ran) {
         const bool act = vec < p.svec;
         uint2 s[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
@@ -1508,7 +1546,7 @@ __global__ void __launch_bounds__(kThreads) column_end_kernel(const GenParams p,
     }
     __shared__ int s_last;
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atom_add_acq_rel(reinterpret_cast<unsigned int *>(c.ctl + kCtlTicket), 1u) == gridDim.x - 1u ? 1 : 0;
+    if (threadIdx.x == 0) s_last = atom_add_acq_rel(reinterpret_cast<unsigned int *>(c.ctl + kCtlTicket), 1u) == (unsigned int)blocks - 1u ? 1 : 0;
     __syncthreads();
     if (!s_last || threadIdx.x != 0) return;
     c.ctl[kCtlTicket] = 0;
@@ -1523,6 +1561,15 @@ __global__ void __launch_bounds__(kThreads) column_end_kernel(const GenParams p,
     column_clear_words(c);
     c.ctl[kCtlRebuilt] = 0;
     c.ctl[kCtlPhase] = 0;
+}
+
+__global__ void __launch_bounds__(kThreads) column_end_kernel(const GenParams p, const ColParams c, int32_t from_rows)
+{
+    __shared__ uint32_t s_thr[kMaxThr];
+    load_thresholds(p, s_thr);
+    grid_dependency_wait();
+    __syncthreads();
+    column_end(p, c, from_rows, (int)blockIdx.x, (int)gridDim.x, s_thr);
 }
 
 // Generation 0 of an instance that runs in the column form: the words every form shares, one row
@@ -1559,6 +1606,69 @@ __global__ void __launch_bounds__(kThreads) column_expand_kernel(const GenParams
     const size_t total = (size_t)p.np * p.svec, stride = (size_t)gridDim.x * kThreads;
     for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < total; i += stride)
         p.state[i] = __ldg(row + i % (size_t)p.svec);
+}
+
+// Many instances in one launch (batches, a server's steps). The members do not depend on one
+// another, so each has its own blocks for the whole run: a list of tasks per block, where a member
+// that is worth several blocks has them to itself and small members follow one another on one
+// block (see plan_column_batch, which cuts the blocks so that all end at about the same time).
+struct ColMember {
+    GenParams p;
+    ColParams c;
+};
+
+struct ColTask {
+    int32_t member;
+    int32_t block, blocks;        // of the member's blocks
+    int32_t pad;
+};
+
+// A member's words in shared memory (whole block).
+__device__ __forceinline__ void load_member(ColMember &s_m, const ColMember *m)
+{
+    static_assert(sizeof(ColMember) % 4 == 0, "copied by words");
+    __syncthreads();
+    for (int i = threadIdx.x; i < (int)(sizeof(ColMember) / 4); i += kThreads)
+        reinterpret_cast<uint32_t *>(&s_m)[i] = __ldg(reinterpret_cast<const uint32_t *>(m) + i);
+    __syncthreads();
+}
+
+// Every generation of the members' runs in one cooperative launch: block b's tasks are
+// [first[b], first[b + 1]).
+template <int kForm>
+__global__ void __launch_bounds__(kThreads, 2) column_batch_kernel(const ColMember *members, const ColTask *tasks,
+                                                                   const int32_t *first, int32_t G)
+{
+    __shared__ ColMember s_m;
+    __shared__ ColRunShared<kForm> sh;
+    for (int i = first[blockIdx.x]; i < first[blockIdx.x + 1]; ++i) {
+        const ColTask k = tasks[i];
+        load_member(s_m, members + k.member);
+        column_run<kForm, true>(s_m.p, s_m.c, G, k.block, k.blocks, sh);
+    }
+}
+
+// column_plane_kernel for every member, task by task.
+__global__ void __launch_bounds__(kThreads) column_batch_plane_kernel(const ColMember *members, const ColTask *tasks)
+{
+    __shared__ ColMember s_m;
+    __shared__ uint32_t s_thr[kMaxThr];
+    const ColTask k = tasks[blockIdx.x];
+    load_member(s_m, members + k.member);
+    load_thresholds(s_m.p, s_thr);
+    __syncthreads();
+    column_plane(s_m.p, s_m.c, k.block, k.blocks, s_thr);
+}
+
+__global__ void __launch_bounds__(kThreads) column_batch_end_kernel(const ColMember *members, const ColTask *tasks)
+{
+    __shared__ ColMember s_m;
+    __shared__ uint32_t s_thr[kMaxThr];
+    const ColTask k = tasks[blockIdx.x];
+    load_member(s_m, members + k.member);
+    load_thresholds(s_m.p, s_thr);
+    __syncthreads();
+    column_end(s_m.p, s_m.c, 0, k.block, k.blocks, s_thr);
 }
 
 }  // namespace qieo

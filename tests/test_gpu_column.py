@@ -149,3 +149,62 @@ def test_wait_that_runs_out_is_reported():
             I.reset()
             I.run(30)
             check(I, O.run(prob, np_, 30, seed=16), 30)
+
+
+@pytest.mark.parametrize("sizes,copies,D,items,chunks", [
+    ([(1, 1), (40, 30)], 1, 4, "byte", [3, 1, 9]),                    # a member per block, empty lists
+    ([(20000, 60), (2048, 33), (700, 500), (31, 128)], 1, 12, "byte", [25, 8]),
+    ([(4500, 3), (260, 5), (9, 2)], 110, 20, "byte", [20, 4]),        # several members a block; three tiles on one
+    ([(4100, 90), (50, 20), (2500, 40)], 2, 100, "mid", [60, 20]),
+    ([(3000, 64), (257, 40), (12, 300)], 2, 100, "wide", [60, 20]),
+])
+def test_batched_column_form(sizes, copies, D, items, chunks):
+    """Members on several blocks, on one, and several on one, against the oracle; a second solve."""
+    specs = [(ng, np_, 10 * c + i) for c in range(copies) for i, (ng, np_) in enumerate(sizes)]
+    probs = {ng: _problem(ng, items) for ng, _ in sizes}
+    insts = [Q.Instance(probs[ng], np_, seed=7, inst=k, D=D, lam=2) for ng, np_, k in specs]
+    gens = sum(chunks)
+    sample = [i for i in range(len(specs)) if i < len(sizes) or i % 29 == 0]
+    refs = {i: O.run(probs[specs[i][0]], specs[i][1], gens, seed=7, inst=specs[i][2], D=D, lam=2) for i in sample}
+    with Q.Batch(insts) as b:
+        for solve in range(2):
+            for g in chunks:
+                b.run(g)
+            for i in sample:
+                check(insts[i], refs[i], gens)
+            for I in insts:
+                I.reset()
+    for I in insts:
+        I.close()
+
+
+def test_batch_whose_members_change_form():
+    """A member that loads a checkpoint with different rows leaves the column form for the
+    row-by-row one, and comes back after a reset; the others, one of rule R2 and one that stops by
+    convergence among them, go on."""
+    prob, np_ = W.knapsack(1500, 8), 40
+    k0 = np.random.default_rng(3).integers(-25, 26, size=(np_, 1500)).astype(np.int16)
+    conv = W.knapsack(200, 3)
+    ref = O.run(conv, 30, 400, seed=3, window=20)
+    insts = [Q.Instance(prob, np_, seed=i + 1, rule=1 if i == 2 else 0) for i in range(3)]
+    insts.append(Q.Instance(conv, 30, seed=3, flags=Q.QIEO_FLAG_CONVERGE))
+    with Q.Batch(insts) as b:
+        b.run(15)
+        load_state(insts[0], k0)         # (a checkpoint of generation 15 with other angles)
+        st = O.run(prob, np_, 15, seed=1)
+        st.k[:] = k0
+        st = O.run(prob, np_, 30, seed=1, state=st)
+        b.run(15)
+        b.run(15)
+        check(insts[0], st, 45)
+        check(insts[1], O.run(prob, np_, 45, seed=2), 45)
+        check(insts[2], O.run(prob, np_, 45, seed=3, rule=1), 45)
+        insts[0].reset()
+        b.run(355)
+        check(insts[0], O.run(prob, np_, 355, seed=1), 355)
+    k, t = insts[3].state()
+    assert ref.stopped and t == int(ref.t[0]) and np.array_equal(k, ref.k)
+    bits, bf, bg, bc = insts[3].best()
+    assert (bf, bg, bc) == tuple(int(v) for v in ref.best) and np.array_equal(bits, ref.best_x)
+    for I in insts:
+        I.close()
