@@ -283,10 +283,10 @@ ResidentFn resident_fn(const qieo_instance *q)
 }
 
 // Runs in the column form: rule R1 from equal rows, the packed elite key, 16-bit state; not
-// where a flag asks for one of the row-by-row forms or a solve sits in a server's arena.
+// where a flag asks for one of the row-by-row forms.
 bool column_capable(const qieo_instance *q)
 {
-    return q->rule == 0 && q->key_ok && !q->state8 && !q->host_de && !q->row_block && q->owns_block &&
+    return q->rule == 0 && q->key_ok && !q->state8 && !q->host_de && !q->row_block &&
            !(q->flags & (QIEO_FLAG_UNFUSED | QIEO_FLAG_COOPERATIVE | QIEO_FLAG_REGISTER_PREFETCH |
                          QIEO_FLAG_PER_GENERATION | QIEO_FLAG_STREAMED | QIEO_FLAG_SIXTEEN |
                          QIEO_FLAG_NO_FIXED_WORDS | QIEO_FLAG_SPARSE_ALWAYS | QIEO_FLAG_STATE_I8));
@@ -1490,6 +1490,10 @@ qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
         if (!ext->block || ext->bytes < total) return bail(fail(QIEO_ERR_INVALID, "placement too small"));
         q->block = ext->block;
         q->owns_block = false;
+        // A placed instance never leaves the column form (nothing reads its full state), so the
+        // form's words lie where the full state would, if they fit.
+        if (column_capable(q) && column_bytes(q->svec) <= (size_t)q->np * q->svec * 16)
+            q->col_mem = static_cast<char *>(q->block) + off[0];
     } else {
         // stream-ordered allocation from the device's pool: no device-wide synchronisation
         // at allocation or release, and a freed block is reused by the next instance
@@ -2326,7 +2330,7 @@ double column_member_time(const qieo_instance *q, int s)
 // it needs, before all else on them, and the others follow, longest first, each on the block with
 // the least to do; the time is the smallest for which that works out
 // (a bisection).
-void plan_column_batch(const std::vector<qieo_instance *> &members, int sms, ColumnBatch &b)
+void plan_column_batch(const std::vector<qieo_instance *> &members, int sms, bool planes, ColumnBatch &b)
 {
     const int n = (int)members.size(), grid = b.grid;
     b.members.clear();
@@ -2407,7 +2411,8 @@ void plan_column_batch(const std::vector<qieo_instance *> &members, int sms, Col
         const int tiles = plane_tiles(q);
         const double share = (double)q->np * q->svec / bytes * 4.0 * sms;
         const int parts = std::max(1, std::min(q->np, (int)(share / tiles + 0.5)));
-        for (int k = 0; k < tiles * parts; ++k) b.plane.push_back({i, k, tiles * parts, 0});
+        if (!planes) b.plane.push_back({i, 0, 0, 0});
+        for (int k = 0; planes && k < tiles * parts; ++k) b.plane.push_back({i, k, tiles * parts, 0});
         for (int k = 0; k < tiles; ++k) b.end.push_back({i, k, tiles, 0});
     }
 }
@@ -2735,7 +2740,7 @@ qieo_status build_col_group(qieo_batch *bt, qieo_batch::ColGroup &g)
 {
     qieo_status st = column_batch_grid(g.members[0], g.plan);
     if (st != QIEO_OK) return st;
-    plan_column_batch(g.members, g.members[0]->sm_count, g.plan);
+    plan_column_batch(g.members, g.members[0]->sm_count, true, g.plan);
     size_t off[kColumnBatchParts], bytes[kColumnBatchParts];
     const void *src[kColumnBatchParts];
     const size_t total = column_batch_layout(g.plan, 0, off, src, bytes);
@@ -3168,11 +3173,30 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
         qieo::BatchArgs args;
     };
     std::vector<Launch> launches;
+    std::vector<ColumnBatch> columns;             // the solves in the column form, by item form
+    for (int form = 0; form < 3; ++form) {
+        std::vector<qieo_instance *> grp;
+        for (qieo_instance *q : members)
+            if (use_column(q) && q->col_form == form) grp.push_back(q);
+        if (grp.empty()) continue;
+        columns.emplace_back();
+        ColumnBatch &b = columns.back();
+        b.form = form;
+        qieo_status st = column_batch_grid(grp[0], b);
+        if (st != QIEO_OK) return st;
+        plan_column_batch(grp, S->sm_count, false, b);
+        size_t off[kColumnBatchParts], bytes[kColumnBatchParts];
+        const void *src[kColumnBatchParts];
+        used = column_batch_layout(b, used, off, src, bytes);
+        if (used > kWorkListBytes) return fail(QIEO_ERR_INVALID, "too many resident solves for one work list");
+        for (int i = 0; i < kColumnBatchParts; ++i) std::memcpy(host + off[i], src[i], bytes[i]);
+        place_column_batch(b, dev, off);
+    }
     for (int narrow = 0; narrow < 2; ++narrow) {
         for (int rule = 0; rule < 2; ++rule) {
             std::vector<qieo_instance *> grp;
             for (qieo_instance *q : members)
-                if (q->narrow == narrow && q->rule == rule) grp.push_back(q);
+                if (!use_column(q) && q->narrow == narrow && q->rule == rule) grp.push_back(q);
             if (grp.empty()) continue;
             const int grid = S->bps[narrow] * S->sm_count;
             std::vector<qieo::BatchSeg> segs;
@@ -3208,6 +3232,10 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
         }
     }
     CUDA_TRY(cudaMemcpyAsync(dev, host, used, cudaMemcpyHostToDevice, S->stream));
+    for (const ColumnBatch &b : columns) {
+        qieo_status st = launch_column_batch(b, G, S->stream);
+        if (st != QIEO_OK) return st;
+    }
     for (int32_t gen = 0; gen < G; ++gen) {
         for (const Launch &L : launches) {
             cudaLaunchAttribute attr[1];
@@ -3228,7 +3256,7 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
         else qieo::batch_cip_kernel<0><<<L.grid, qieo::kThreads, 0, S->stream>>>(L.args);
         CUDA_TRY(cudaGetLastError());
     }
-    *launched = (int64_t)launches.size() * (G + 1);
+    *launched = (int64_t)launches.size() * (G + 1) + 3 * (int64_t)columns.size();
     if (!watch.empty()) {   // stop states of the solves with the convergence test, to the host
         const size_t nw = watch.size();
         const size_t p_off = used, o_off = align_up(p_off + nw * sizeof(int32_t *), 256);

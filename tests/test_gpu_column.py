@@ -208,3 +208,23 @@ def test_batch_whose_members_change_form():
     assert (bf, bg, bc) == tuple(int(v) for v in ref.best) and np.array_equal(bits, ref.best_x)
     for I in insts:
         I.close()
+
+
+@pytest.mark.parametrize("items,D", [("byte", 100), ("mid", 12), ("wide", 40)])
+def test_served_column_form(items, D):
+    """A server's solves: populations too small to hold the form's words where their state would
+    lie (these run row by row), larger ones, and one that stops by convergence."""
+    specs = [(1, 1), (300, 4), (90, 250), (2500, 60), (4100, 128), (33, 400)]
+    with Q.Server(gens_per_step=7) as srv:
+        ids = [srv.submit(_problem(ng, items), np_, 40, seed=ng, inst=2, D=D, lam=2) for ng, np_ in specs]
+        stops = srv.submit(W.knapsack(200, 3), 300, 400, seed=3, flags=Q.QIEO_FLAG_CONVERGE)
+        for rid, (ng, np_) in zip(ids, specs):
+            res, bits = srv.poll(rid, wait_ms=60000)
+            st = O.run(_problem(ng, items), np_, 40, seed=ng, inst=2, D=D, lam=2)
+            assert res.state == Q.QIEO_SOLVE_DONE and res.generations_run == 40
+            assert (res.fitness, res.generation, res.chromosome) == tuple(int(v) for v in st.best)
+            assert np.array_equal(bits, st.best_x)
+        res, bits = srv.poll(stops, wait_ms=60000)
+        ref = O.run(W.knapsack(200, 3), 300, 400, seed=3, window=20)
+        assert res.converged == 1 and res.generations_run == int(ref.t[0])
+        assert np.array_equal(bits, ref.best_x)
