@@ -25,7 +25,6 @@
 #include <map>
 #include <memory>
 #include <mutex>
-#include <queue>
 #include <unordered_map>
 #include <tuple>
 #include <new>
@@ -80,6 +79,7 @@ int pow2_ceil(int x)
 namespace qieo_internal {
 // Lets the library's other translation units report through qieo_last_error().
 void set_last_error(const char *msg) { g_last_error = msg; }
+void fill_thresholds(int32_t D, uint32_t *thr);   // qieo_noalloc.cu
 }  // namespace qieo_internal
 
 namespace {
@@ -365,10 +365,10 @@ qieo_status pinned_scratch(size_t bytes, char **out)
     };
     thread_local Scratch s;
     if (s.n < bytes) {
+        const size_t n = std::max<size_t>({bytes, 2 * s.n, 4096});   // (a new one takes 100 us)
         if (s.p) cudaFreeHost(s.p);
         s.p = nullptr;
         s.n = 0;
-        const size_t n = std::max<size_t>(bytes, 4096);
         CUDA_TRY(cudaMallocHost(&s.p, n));
         s.n = n;
     }
@@ -777,32 +777,6 @@ qieo_status wait_stream(cudaStream_t s)
         else std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 20 : 200));
     }
 }
-
-// Threshold table T[n] = round(sin^2(n pi / D) 2^32), evaluated as 2^31 (1 - cos(2 n pi/D))
-// in extended precision for n <= K and mirrored (T[2K-n] = 2^32 - T[n]) above.
-void build_thresholds(int32_t D, std::vector<uint64_t> &T)
-{
-    const int32_t K = D / 4;
-    T.assign((size_t)(2 * K + 1), 0);
-    const long double pi = acosl(-1.0L);
-    for (int32_t n = 0; n <= K; ++n) {
-        const long double c = cosl(2.0L * pi * (long double)n / (long double)D);
-        const long double val = 2147483648.0L * (1.0L - c);
-        T[(size_t)n] = (uint64_t)llroundl(val);
-    }
-    T[0] = 0;
-    T[(size_t)K] = 1ull << 31;
-    for (int32_t n = K + 1; n <= 2 * K; ++n) T[(size_t)n] = (1ull << 32) - T[(size_t)(2 * K - n)];
-}
-
-}  // namespace
-
-namespace qieo_internal {
-// The threshold table for the library's other translation units.
-void build_thresholds(int32_t D, std::vector<uint64_t> &T) { ::build_thresholds(D, T); }
-}  // namespace qieo_internal
-
-namespace {
 
 // Device memory of the column form: the state between runs, the two parities, the recorded best
 // alleles and the two lists (16 B a vector each), then the counts, the control words and the
@@ -1390,6 +1364,10 @@ struct Placement {
     void *block;
     size_t bytes;
     int32_t hist_cap;
+    // where the items are uploaded, and an event that orders it before the instance's stream (which a
+    // copy from pageable memory would otherwise wait for)
+    cudaStream_t upload;
+    cudaEvent_t uploaded;
 };
 
 qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
@@ -1566,10 +1544,8 @@ qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
             q->tile_sums[(size_t)2 * (j / (8 * qieo::kThreads)) + 1] += (uint32_t)pr->values[j];
         }
     }
-    std::vector<uint64_t> T;
-    build_thresholds(q->D, T);
-    std::vector<uint32_t> T32(T.size());
-    for (size_t i = 0; i < T.size(); ++i) T32[i] = (uint32_t)(T[i] & 0xffffffffull);
+    std::vector<uint32_t> T32((size_t)(2 * q->K + 1));
+    qieo_internal::fill_thresholds(q->D, T32.data());
 
     // One copy for the items (both layouts) and the thresholds: the parts between them are
     // sent as zeros and set by the generation-0 initialisation that follows on the stream.
@@ -1579,7 +1555,9 @@ qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
         std::memcpy(stage.data() + (off[2] - lo), packed.data(), packed.size() * 4);
         std::memcpy(stage.data() + (off[3] - lo), wide.data(), wide.size() * 4);
         std::memcpy(stage.data() + (off[13] - lo), T32.data(), T32.size() * 4);
-        ce = cudaMemcpyAsync(b + lo, stage.data(), stage.size(), cudaMemcpyHostToDevice, q->stream);
+        ce = cudaMemcpyAsync(b + lo, stage.data(), stage.size(), cudaMemcpyHostToDevice, ext ? ext->upload : q->stream);
+        if (ext && ce == cudaSuccess) ce = cudaEventRecord(ext->uploaded, ext->upload);
+        if (ext && ce == cudaSuccess) ce = cudaStreamWaitEvent(q->stream, ext->uploaded, 0);
         if (ce != cudaSuccess) return bail(fail(QIEO_ERR_CUDA, "upload: %s", cudaGetErrorString(ce)));
     }
 
@@ -2330,8 +2308,11 @@ double column_member_time(const qieo_instance *q, int s)
 // it needs, before all else on them, and the others follow, longest first, each on the block with
 // the least to do; the time is the smallest for which that works out
 // (a bisection).
-void plan_column_batch(const std::vector<qieo_instance *> &members, int sms, bool planes, ColumnBatch &b)
+// gens: the most generations of each member (empty: no limit).
+void plan_column_batch(const std::vector<qieo_instance *> &members, const std::vector<int32_t> &gens, int sms,
+                       bool planes, ColumnBatch &b)
 {
+    const auto gens_of = [&](int i) { return gens.empty() ? INT32_MAX : gens[(size_t)i]; };
     const int n = (int)members.size(), grid = b.grid;
     b.members.clear();
     std::vector<double> alone((size_t)n);
@@ -2349,57 +2330,61 @@ void plan_column_batch(const std::vector<qieo_instance *> &members, int sms, boo
     for (int i = 0; i < n; ++i) order[(size_t)i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return alone[(size_t)x] > alone[(size_t)y]; });
     typedef std::pair<double, int> Load;             // a block's time, the block
-    std::vector<std::vector<qieo::ColTask>> best, lists;
+    struct Place {
+        int at, blocks;
+    };
+    std::vector<Place> best, place((size_t)n);       // per member
+    std::vector<Load> loads;                         // a heap, the least load first
+    const auto later = [](const Load &x, const Load &y) { return x > y; };
     double hi = total / grid + longest;              // (every member on one block)
     for (int round = 0; round < 14; ++round) {
         const double t = round == 0 ? hi : 0.5 * (lo + hi);
-        lists.assign((size_t)grid, {});
         int used = 0;
         bool fits = true;
-        std::vector<int> singles;
-        std::priority_queue<Load, std::vector<Load>, std::greater<Load>> blocks;
-        for (int i : order) {
-            if (alone[(size_t)i] <= t) {
-                singles.push_back(i);
-                continue;
-            }
-            int need = std::max(2, (int)((alone[(size_t)i] - kBatchChainUs) / std::max(t - kBatchChainUs, 0.1)));
-            while (need <= grid - used && column_member_time(members[(size_t)i], need) > t) ++need;
-            if (need > grid - used) {
-                fits = false;
-                break;
-            }
-            const double each = column_member_time(members[(size_t)i], need);
-            for (int k = 0; k < need; ++k) {
-                lists[(size_t)(used + k)].push_back({i, k, need, 0});
-                blocks.push({each, used + k});
-            }
+        size_t k = 0;
+        loads.clear();
+        for (; k < order.size() && alone[(size_t)order[k]] > t; ++k) {
+            const qieo_instance *q = members[(size_t)order[k]];
+            int need = std::max(2, (int)((alone[(size_t)order[k]] - kBatchChainUs) / std::max(t - kBatchChainUs, 0.1)));
+            while (need <= grid - used && column_member_time(q, need) > t) ++need;
+            fits = need <= grid - used;
+            if (!fits) break;
+            loads.insert(loads.end(), (size_t)need, Load(column_member_time(q, need), 0));
+            place[(size_t)order[k]] = {used, need};
             used += need;
         }
-        for (int k = used; k < grid; ++k) blocks.push({0.0, k});
-        for (int i : singles) {
-            if (!fits) break;
-            Load l = blocks.top();
-            blocks.pop();
-            l.first += alone[(size_t)i];
-            // (at the first bound this always fits: the least loaded block has at most total / grid)
-            fits = l.first <= t || round == 0;
-            lists[(size_t)l.second].push_back({i, 0, 1, 0});
-            blocks.push(l);
+        if (fits) {
+            loads.resize((size_t)grid, Load(0.0, 0));
+            for (int i = 0; i < grid; ++i) loads[(size_t)i].second = i;
+            std::make_heap(loads.begin(), loads.end(), later);
+            for (; fits && k < order.size(); ++k) {
+                std::pop_heap(loads.begin(), loads.end(), later);
+                Load &l = loads.back();
+                l.first += alone[(size_t)order[k]];
+                // (at the first bound this always fits: the least loaded block has at most total / grid)
+                fits = l.first <= t || round == 0;
+                place[(size_t)order[k]] = {l.second, 1};
+                std::push_heap(loads.begin(), loads.end(), later);
+            }
         }
         if (fits) {
-            best = lists;
+            best = place;
             hi = t;
         } else {
             lo = t;
         }
         if (hi - lo < 0.02 * hi) break;
     }
-    b.tasks.clear();
-    b.first.assign(1, 0);
-    for (const auto &l : best) {
-        b.tasks.insert(b.tasks.end(), l.begin(), l.end());
-        b.first.push_back((int32_t)b.tasks.size());
+    // the blocks' lists, each in the members' order
+    b.first.assign((size_t)grid + 1, 0);
+    for (const Place &p : best)
+        for (int k = 0; k < p.blocks; ++k) b.first[(size_t)(p.at + k) + 1] += 1;
+    for (int i = 0; i < grid; ++i) b.first[(size_t)i + 1] += b.first[(size_t)i];
+    b.tasks.resize((size_t)b.first[(size_t)grid]);
+    std::vector<int32_t> next(b.first.begin(), b.first.end() - 1);
+    for (int i : order) {
+        const Place p = best[(size_t)i];
+        for (int k = 0; k < p.blocks; ++k) b.tasks[(size_t)next[(size_t)(p.at + k)]++] = {i, k, p.blocks, gens_of(i)};
     }
     b.plane.clear();
     b.end.clear();
@@ -2740,7 +2725,7 @@ qieo_status build_col_group(qieo_batch *bt, qieo_batch::ColGroup &g)
 {
     qieo_status st = column_batch_grid(g.members[0], g.plan);
     if (st != QIEO_OK) return st;
-    plan_column_batch(g.members, g.members[0]->sm_count, true, g.plan);
+    plan_column_batch(g.members, {}, g.members[0]->sm_count, true, g.plan);
     size_t off[kColumnBatchParts], bytes[kColumnBatchParts];
     const void *src[kColumnBatchParts];
     const size_t total = column_batch_layout(g.plan, 0, off, src, bytes);
@@ -3107,6 +3092,9 @@ struct StepRecord {
     const int32_t *stop_host = nullptr;        // ... and their stop states after the step
 };
 
+// Solves admitted between two looks at the steps: an admission takes the host about 50 us, and the GPU
+// starts on the first ones meanwhile.
+constexpr size_t kAdmitAtOnce = 16;
 constexpr size_t kWorkListBytes = 16u << 20;   // per region: params, segments, block starts
 
 }  // namespace
@@ -3115,6 +3103,7 @@ struct qieo_server {
     qieo_server_config cfg{};
     int device = 0, sm_count = 0;
     cudaStream_t stream = nullptr, copy_stream = nullptr;
+    cudaEvent_t uploaded = nullptr;      // the last admitted solve's items have arrived
     char *arena = nullptr;
     ArenaAlloc alloc;
     char *wl_dev[2] = {nullptr, nullptr};
@@ -3152,9 +3141,11 @@ void destroy_instance_nosync(qieo_instance *q)
     delete q;
 }
 
-// Enqueues `G` generations (+ the final rotation) of every member on the server stream
-// with the batched kernel; the work list goes through the next double-buffered region.
-qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance *> &members, int32_t G,
+// Enqueues `G` generations (+ the final rotation) of every member on the server stream, for members in
+// the column form the remaining ones if fewer, with the batched kernels; the work list goes
+// through the next double-buffered region.
+qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance *> &members,
+                                const std::vector<int32_t> &remaining, int32_t G,
                                 int64_t *launched, const std::vector<qieo_instance *> &watch,
                                 const int32_t **stop_host)
 {
@@ -3176,15 +3167,19 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
     std::vector<ColumnBatch> columns;             // the solves in the column form, by item form
     for (int form = 0; form < 3; ++form) {
         std::vector<qieo_instance *> grp;
-        for (qieo_instance *q : members)
-            if (use_column(q) && q->col_form == form) grp.push_back(q);
+        std::vector<int32_t> gens;
+        for (size_t i = 0; i < members.size(); ++i)
+            if (use_column(members[i]) && members[i]->col_form == form) {
+                grp.push_back(members[i]);
+                gens.push_back(remaining[i]);
+            }
         if (grp.empty()) continue;
         columns.emplace_back();
         ColumnBatch &b = columns.back();
         b.form = form;
         qieo_status st = column_batch_grid(grp[0], b);
         if (st != QIEO_OK) return st;
-        plan_column_batch(grp, S->sm_count, false, b);
+        plan_column_batch(grp, gens, S->sm_count, false, b);
         size_t off[kColumnBatchParts], bytes[kColumnBatchParts];
         const void *src[kColumnBatchParts];
         used = column_batch_layout(b, used, off, src, bytes);
@@ -3305,18 +3300,35 @@ void retire_oldest_step(qieo_server *S)
             else rec.finishing.push_back(R);
         }
     }
+    // All their results through a pinned buffer, one wait (a copy to pageable memory is a wait of its
+    // own, about 12 us): the record, the generations and the row of each.
+    int32_t copy_st = step_st;
+    char *pin = nullptr;
+    size_t bytes = 0;
+    for (SolveRequest *R : rec.finishing) bytes += 64 + (size_t)R->inst->xstride;
+    if (copy_st == QIEO_OK && bytes != 0) {
+        copy_st = pinned_scratch(bytes, &pin);
+        bool ok = copy_st == QIEO_OK;
+        char *at = pin;
+        for (size_t i = 0; ok && i < rec.finishing.size(); ++i) {
+            qieo_instance *q = rec.finishing[i]->inst;
+            ok = cudaMemcpyAsync(at, q->gp.best, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess &&
+                 cudaMemcpyAsync(at + 24, q->gp.gen, sizeof(int32_t), cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess &&
+                 cudaMemcpyAsync(at + 64, q->gp.best_row, (size_t)q->xstride, cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess;
+            at += 64 + q->xstride;
+        }
+        // (also after a failure: nothing may still write the buffer)
+        if (cudaStreamSynchronize(S->copy_stream) != cudaSuccess) ok = false;
+        if (!ok && copy_st == QIEO_OK) copy_st = QIEO_ERR_CUDA;
+    }
     for (SolveRequest *R : rec.finishing) {
         qieo_instance *q = R->inst;
-        int32_t st = step_st;
+        const int32_t st = copy_st;
         if (st == QIEO_OK) {
-            R->best_row.resize((size_t)q->xstride);
-            if (cudaMemcpyAsync(R->best, q->gp.best, sizeof R->best, cudaMemcpyDeviceToHost, S->copy_stream) != cudaSuccess ||
-                cudaMemcpyAsync(&R->gens_run, q->gp.gen, sizeof R->gens_run, cudaMemcpyDeviceToHost,
-                                S->copy_stream) != cudaSuccess ||
-                cudaMemcpyAsync(R->best_row.data(), q->gp.best_row, R->best_row.size(), cudaMemcpyDeviceToHost,
-                                S->copy_stream) != cudaSuccess ||
-                cudaStreamSynchronize(S->copy_stream) != cudaSuccess)
-                st = QIEO_ERR_CUDA;
+            std::memcpy(R->best, pin, sizeof R->best);
+            std::memcpy(&R->gens_run, pin + 24, sizeof R->gens_run);
+            R->best_row.assign(pin + 64, pin + 64 + q->xstride);
+            pin += 64 + q->xstride;
         }
         destroy_instance_nosync(q);
         std::lock_guard<std::mutex> lock(S->mu);
@@ -3339,7 +3351,8 @@ void server_loop(qieo_server *S)
         {
             std::unique_lock<std::mutex> lock(S->mu);
             while (!S->queue.empty() &&
-                   (int64_t)(S->active.size() + admit.size()) < (int64_t)S->cfg.max_active) {
+                   (int64_t)(S->active.size() + admit.size()) < (int64_t)S->cfg.max_active &&
+                   admit.size() < kAdmitAtOnce) {
                 SolveRequest *R = S->queue.front();
                 size_t off = 0;
                 if (!S->alloc.alloc(R->bytes, &off)) break;
@@ -3358,7 +3371,7 @@ void server_loop(qieo_server *S)
             pa.stream = S->stream;
             pa.flags &= QIEO_FLAG_CONVERGE;
             pa.elite_on_host = 0;
-            Placement pl{S->arena + R->off, R->bytes, R->gens};
+            Placement pl{S->arena + R->off, R->bytes, R->gens, S->copy_stream, S->uploaded};
             qieo_instance *q = nullptr;
             const qieo_status st = create_instance_impl(&R->prob, &pa, &pl, false, &q);
             std::lock_guard<std::mutex> lock(S->mu);
@@ -3382,10 +3395,20 @@ void server_loop(qieo_server *S)
         if (!S->active.empty() && S->inflight.size() < 2) {
             int32_t G = S->cfg.gens_per_step;
             std::vector<qieo_instance *> members;
+            std::vector<int32_t> remaining;
+            bool all_column = true;
+            int32_t longest = 0;
             for (SolveRequest *R : S->active) {
-                G = std::min(G, R->remaining);
+                // (the row-by-row kernels run the same generations for all their members)
+                if (!use_column(R->inst)) {
+                    G = std::min(G, R->remaining);
+                    all_column = false;
+                }
+                longest = std::max(longest, R->remaining);
                 members.push_back(R->inst);
+                remaining.push_back(R->remaining);
             }
+            if (all_column) G = std::min(G, longest);
             StepRecord rec;
             std::vector<qieo_instance *> watch;
             for (SolveRequest *R : S->active)
@@ -3394,7 +3417,7 @@ void server_loop(qieo_server *S)
                     watch.push_back(R->inst);
                 }
             int64_t launched = 0;
-            qieo_status st = enqueue_server_step(S, members, G, &launched, watch, &rec.stop_host);
+            qieo_status st = enqueue_server_step(S, members, remaining, G, &launched, watch, &rec.stop_host);
             if (st == QIEO_OK) {
                 if (S->spare_events.empty()) {
                     cudaEvent_t ev = nullptr;
@@ -3416,8 +3439,9 @@ void server_loop(qieo_server *S)
                     R->t_done = server_now(S);
                     continue;
                 }
-                R->remaining -= G;
-                R->inst->t += G;
+                const int32_t ran = std::min(G, R->remaining);
+                R->remaining -= ran;
+                R->inst->t += ran;
                 if (R->remaining == 0) rec.finishing.push_back(R);
                 else still.push_back(R);
             }
@@ -3429,7 +3453,8 @@ void server_loop(qieo_server *S)
             } else {
                 S->cv_done.notify_all();
             }
-        } else if (!S->inflight.empty()) {
+        } else if (!S->inflight.empty() &&
+                   (admit.size() < kAdmitAtOnce || cudaEventQuery(S->inflight.front().done) != cudaErrorNotReady)) {
             retire_oldest_step(S);
         }
     }
@@ -3460,6 +3485,7 @@ qieo_status qieo_server_create(const qieo_server_config *config, qieo_server **o
     if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&S->sm_count, cudaDevAttrMultiProcessorCount, S->device);
     if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
     if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&S->copy_stream, cudaStreamNonBlocking);
+    if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&S->uploaded, cudaEventDisableTiming);
     if (ce != cudaSuccess) return bail(fail(QIEO_ERR_CUDA, "server setup: %s", cudaGetErrorString(ce)));
     if (cfg.memory_bytes == 0) {
         size_t free_b = 0, total_b = 0;
@@ -3614,6 +3640,7 @@ qieo_status qieo_server_destroy(qieo_server *S)
     if (S->arena) cudaFree(S->arena);
     if (S->stream) cudaStreamDestroy(S->stream);
     if (S->copy_stream) cudaStreamDestroy(S->copy_stream);
+    if (S->uploaded) cudaEventDestroy(S->uploaded);
     delete S;
     return QIEO_OK;
 }

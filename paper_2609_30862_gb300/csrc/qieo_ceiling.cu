@@ -27,7 +27,7 @@
 
 namespace qieo_internal {
 void set_last_error(const char *msg);                           // qieo_api.cu
-void build_thresholds(int32_t D, std::vector<uint64_t> &T);   // qieo_api.cu
+void fill_thresholds(int32_t D, uint32_t *thr);               // qieo_noalloc.cu
 }
 
 namespace {
@@ -150,10 +150,8 @@ qieo_status qieo_measure_integer_ceiling(int32_t reps, qieo_integer_ceiling *out
     const int grid = std::max(1, sms) * kBlocksPerSm;
     const int32_t passes = 2048;
 
-    std::vector<uint64_t> T;
-    qieo_internal::build_thresholds(kD, T);
-    std::vector<uint32_t> thr(T.size());
-    for (size_t i = 0; i < T.size(); ++i) thr[i] = (uint32_t)T[i];   // T[2K] = 2^32 -> 0
+    std::vector<uint32_t> thr((size_t)(2 * (kD / 4) + 1));
+    qieo_internal::fill_thresholds(kD, thr.data());
 
     CeilingParams p{};
     p.passes = passes;

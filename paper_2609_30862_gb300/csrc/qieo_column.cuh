@@ -1627,7 +1627,7 @@ struct ColMember {
 struct ColTask {
     int32_t member;
     int32_t block, blocks;        // of the member's blocks
-    int32_t pad;
+    int32_t gens;                 // most generations of this run
 };
 
 // A member's words in shared memory (whole block).
@@ -1651,7 +1651,7 @@ __global__ void __launch_bounds__(kThreads, 2) column_batch_kernel(const ColMemb
     for (int i = first[blockIdx.x]; i < first[blockIdx.x + 1]; ++i) {
         const ColTask k = tasks[i];
         load_member(s_m, members + k.member);
-        column_run<kForm, true>(s_m.p, s_m.c, G, k.block, k.blocks, sh);
+        column_run<kForm, true>(s_m.p, s_m.c, min(G, k.gens), k.block, k.blocks, sh);
     }
 }
 

@@ -593,6 +593,11 @@ qieo_status launch_noalloc(const qieo_problem &problem, const qieo_params &param
 
 }  // namespace
 
+namespace qieo_internal {
+// The threshold words for the library's other translation units ([2 (D / 4) + 1]).
+void fill_thresholds(int32_t D, uint32_t *thr) { ::fill_thresholds(D, thr); }
+}  // namespace qieo_internal
+
 extern "C" qieo_status qieo_generation_noalloc(const qieo_problem *problem, const qieo_params *params,
                                                int32_t t, int16_t *k, uint8_t *x, int64_t *fitness,
                                                int32_t *elite)
