@@ -821,6 +821,13 @@ qieo_status configure_column(qieo_instance *q)
     const size_t rows = align_up(sv * 16, 256);
     qieo::ColParams &c = q->cp;
     c.one = 1u;
+    {
+        // (a list is cut into less than twice as many tiles as it fills)
+        const int64_t tiles = 2 * (((int64_t)sv + qieo::kThreads - 1) / qieo::kThreads);
+        int bits = 1;
+        while (bits < 31 && std::max(q->sum_w, q->sum_v) >> bits) ++bits;
+        c.sum_bits = q->col_form == 1 && std::max(q->sum_w, q->sum_v) >> bits == 0 && tiles < (int64_t)1 << std::min(62, 64 - 2 * bits) ? bits : 0;
+    }
     c.canon = reinterpret_cast<uint2 *>(b);
     c.rows = reinterpret_cast<uint2 *>(b + rows);
     c.best_nib = reinterpret_cast<int2 *>(b + 3 * rows);
