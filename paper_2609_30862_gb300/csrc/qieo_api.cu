@@ -286,7 +286,7 @@ ResidentFn resident_fn(const qieo_instance *q)
 // where a flag asks for one of the row-by-row forms.
 bool column_capable(const qieo_instance *q)
 {
-    return q->rule == 0 && q->key_ok && !q->state8 && !q->host_de && !q->row_block &&
+    return q->rule == 0 && q->key_ok && !q->state8 && !q->host_de &&
            !(q->flags & (QIEO_FLAG_UNFUSED | QIEO_FLAG_COOPERATIVE | QIEO_FLAG_REGISTER_PREFETCH |
                          QIEO_FLAG_PER_GENERATION | QIEO_FLAG_STREAMED | QIEO_FLAG_SIXTEEN |
                          QIEO_FLAG_NO_FIXED_WORDS | QIEO_FLAG_SPARSE_ALWAYS | QIEO_FLAG_STATE_I8));
@@ -1073,6 +1073,26 @@ qieo_status ensure_column(qieo_instance *q)
     CUDA_TRY(launch_column_end(q, 1));
     q->col_valid = true;
     return QIEO_OK;
+}
+
+typedef void (*ColumnObserveFn)(qieo::GenParams, qieo::ColParams, int32_t, int32_t);
+ColumnObserveFn column_observe_fn(int form)
+{
+    return form == 0 ? &qieo::column_observe_kernel<0>
+                     : form == 1 ? &qieo::column_observe_kernel<1> : &qieo::column_observe_kernel<2>;
+}
+
+// One generation of a row block: a block takes a tile and as many rows as make one wave of two
+// blocks per SM.
+cudaError_t launch_column_observe(qieo_instance *q, int32_t t)
+{
+    const int64_t ntile = plane_tiles(q), rpp = ntile > 1 ? 1 : qieo::kThreads / pow2_ceil(q->svec);
+    const int64_t nu = (q->np + rpp - 1) / rpp, parts = std::max<int64_t>(1, std::min(nu, 2 * (int64_t)q->sm_count / ntile));
+    const int64_t part_rows = (nu + parts - 1) / parts * rpp;
+    const int64_t blocks = ntile * ((q->np + part_rows - 1) / part_rows);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = launch_config(q, dim3((unsigned)blocks), 0, attr);
+    return cudaLaunchKernelEx(&cfg, column_observe_fn(q->col_form), q->gp, q->cp, t, (int32_t)part_rows);
 }
 
 // A run in the column form: one cooperative launch, the allele plane, the state between runs.
@@ -1998,7 +2018,7 @@ qieo_status qieo_create_row_block(const qieo_problem *problem, const qieo_params
         qieo_destroy_instance(q);
         return st;
     }
-    cudaError_t ce = cudaMallocAsync(&q->ext_elite, (size_t)q->xstride, q->stream);
+    cudaError_t ce = cudaMallocAsync(&q->ext_elite, (size_t)q->svec * 8 + 16, q->stream);   // (packed or bytes)
     if (ce != cudaSuccess) {
         qieo_destroy_instance(q);
         return fail(QIEO_ERR_OOM, "elite row buffer: %s", cudaGetErrorString(ce));
@@ -2023,18 +2043,30 @@ qieo_status qieo_rows_observe(qieo_instance *q, int32_t t, int64_t *best_fitness
     if (st != QIEO_OK) return st;
     st = wait_stream(q->stream);   // the pinned buffer may still feed an earlier copy
     if (st != QIEO_OK) return st;
-    const int32_t next = t + 1;
-    std::memcpy(h, &t, sizeof t);
-    std::memcpy(h + 4, &next, sizeof next);
-    CUDA_TRY(cudaMemcpyAsync(q->gp.gen, h, sizeof t, cudaMemcpyHostToDevice, q->stream));
-    CUDA_TRY(cudaMemsetAsync(q->gp.keys + (t % 3), 0, sizeof(unsigned long long), q->stream));
-    CUDA_TRY(cudaMemsetAsync(q->gp.qctr + (t % 3), 0, sizeof(unsigned int), q->stream));
-    CUDA_TRY(launch_gen(q, 0, 1, 0));
-    // the generation counter then names the next generation, as after qieo_run
-    CUDA_TRY(cudaMemcpyAsync(q->gp.gen, h + 4, sizeof next, cudaMemcpyHostToDevice, q->stream));
-    CUDA_TRY(cudaMemcpyAsync(h + 8, q->gp.keys + (t % 3), sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                             q->stream));
-    st = wait_checked(q);
+    if (use_column(q)) {           // (no wait in these kernels can run out)
+        st = ensure_column(q);
+        if (st != QIEO_OK) return st;
+        CUDA_TRY(cudaMemsetAsync(q->gp.keys + (t % 3), 0, sizeof(unsigned long long), q->stream));
+        CUDA_TRY(launch_column_observe(q, t));
+        CUDA_TRY(cudaMemcpyAsync(h + 8, q->gp.keys + (t % 3), sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                 q->stream));
+        st = wait_stream(q->stream);
+    } else {
+        if (q->col_mem) st = ensure_state(q);
+        if (st != QIEO_OK) return st;
+        const int32_t next = t + 1;
+        std::memcpy(h, &t, sizeof t);
+        std::memcpy(h + 4, &next, sizeof next);
+        CUDA_TRY(cudaMemcpyAsync(q->gp.gen, h, sizeof t, cudaMemcpyHostToDevice, q->stream));
+        CUDA_TRY(cudaMemsetAsync(q->gp.keys + (t % 3), 0, sizeof(unsigned long long), q->stream));
+        CUDA_TRY(cudaMemsetAsync(q->gp.qctr + (t % 3), 0, sizeof(unsigned int), q->stream));
+        CUDA_TRY(launch_gen(q, 0, 1, 0));
+        // the generation counter then names the next generation, as after qieo_run
+        CUDA_TRY(cudaMemcpyAsync(q->gp.gen, h + 4, sizeof next, cudaMemcpyHostToDevice, q->stream));
+        CUDA_TRY(cudaMemcpyAsync(h + 8, q->gp.keys + (t % 3), sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                 q->stream));
+        st = wait_checked(q);
+    }
     if (st != QIEO_OK) return st;
     unsigned long long key = 0;
     std::memcpy(&key, h + 8, sizeof key);
@@ -2058,14 +2090,36 @@ qieo_status qieo_rows_rotate(qieo_instance *q, const uint8_t *elite_bits)
     st = set_device(q);
     if (st != QIEO_OK) return st;
     char *h = nullptr;
-    st = pinned_scratch((size_t)q->xstride, &h);
+    st = pinned_scratch((size_t)q->svec * 8, &h);
     if (st != QIEO_OK) return st;
     st = wait_stream(q->stream);
     if (st != QIEO_OK) return st;
+    uint8_t any = use_column(q) ? 0 : 2;
+    for (int32_t j = 0; any < 2 && j < q->ng; j += 256) {
+        for (int32_t i = j, e = std::min(j + 256, q->ng); i < e; ++i) any |= elite_bits[i];
+    }
+    if (any < 2) {                 // the column form; an invalid row is reported below
+        st = ensure_column(q);
+        if (st != QIEO_OK) return st;
+        const size_t n = (size_t)q->svec * 8;
+        std::memcpy(h, elite_bits, (size_t)q->ng);
+        std::memset(h + q->ng, 0, n - (size_t)q->ng);
+        CUDA_TRY(cudaMemcpyAsync(q->ext_elite, h, n, cudaMemcpyHostToDevice, q->stream));
+        qieo::column_rotate_kernel<<<(q->svec + qieo::kThreads - 1) / qieo::kThreads, qieo::kThreads, 0, q->stream>>>(
+            q->gp, q->cp, reinterpret_cast<const uint2 *>(q->ext_elite));
+        CUDA_TRY(cudaGetLastError());
+        q->state_valid = false;
+        return wait_stream(q->stream);
+    }
     std::memset(h, 0, (size_t)q->xstride);
     for (int32_t j = 0; j < q->ng; ++j) {
         if (elite_bits[j] > 1) return fail(QIEO_ERR_INVALID, "elite_bits[%d] = %d is not 0 or 1", j, elite_bits[j]);
         h[j >> 3] = (char)((unsigned char)h[j >> 3] | (unsigned char)(elite_bits[j] << (j & 7)));
+    }
+    if (q->col_mem) {
+        st = ensure_state(q);
+        if (st != QIEO_OK) return st;
+        q->col_valid = false;
     }
     CUDA_TRY(cudaMemcpyAsync(q->ext_elite, h, (size_t)q->xstride, cudaMemcpyHostToDevice, q->stream));
     const size_t total = (size_t)q->np * q->svec;

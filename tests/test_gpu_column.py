@@ -228,3 +228,43 @@ def test_served_column_form(items, D):
         ref = O.run(W.knapsack(200, 3), 300, 400, seed=3, window=20)
         assert res.converged == 1 and res.generations_run == int(ref.t[0])
         assert np.array_equal(bits, ref.best_x)
+
+
+@pytest.mark.parametrize("ng,np_,D,items,start", [
+    (1, 1, 4, "byte", None), (9, 35, 12, "byte", None), (257, 700, 100, "mid", None), (2100, 300, 40, "byte", None),
+    (20003, 70, 100, "byte", None), (100, 90, 100, "wide", None), (4100, 700, 20, "mid", "equal"),
+    (1500, 40, 100, "byte", "mixed"),
+])
+def test_row_blocks(ng, np_, D, items, start):
+    """A population in two row blocks, the elite exchanged here, from the start, from a checkpoint with
+    equal rows and from one whose rows differ (which runs row by row): the oracle's unsharded run."""
+    prob, cut = _problem(ng, items), (np_ + 2) // 3
+    k0 = np.zeros((np_, ng), dtype=np.int16)
+    if start:
+        k0[:] = np.random.default_rng(4).integers(-(D // 4), D // 4 + 1, size=(1 if start == "equal" else np_, ng))
+    st = O.State(np_, ng)
+    st.k[:] = k0
+    O.run(prob, np_, 40, seed=ng, inst=3, D=D, lam=2, state=st)
+    blocks = [Q.Instance(prob, b - a, seed=ng, inst=3, D=D, lam=2, row0=a) for a, b in ((0, cut), (cut, np_)) if b > a]
+    rows0 = [0, cut]
+    for solve in range(2):
+        for I, r0 in zip(blocks, rows0):
+            I.reset()
+            if start:
+                load_state(I, k0[r0:r0 + I.np_], D)
+        he, hf = [], []
+        for t in range(40):
+            found = [I.rows_observe(t) for I in blocks]
+            f, row = max(((f, -c) for f, c in found))
+            owner = 1 if len(blocks) > 1 and -row >= cut else 0
+            elite = blocks[owner].allele_row(-row - rows0[owner])
+            for I in blocks:
+                I.rows_rotate(elite)
+            he.append(-row)
+            hf.append(f)
+        assert np.array_equal(he, st.hist_e) and np.array_equal(hf, st.hist_f)
+        assert np.array_equal(np.concatenate([I.state()[0] for I in blocks]), st.k)
+        assert np.array_equal(np.concatenate([I.fitness() for I in blocks]), st.f)
+        assert np.array_equal(np.concatenate([I.alleles() for I in blocks]), st.x)
+    for I in blocks:
+        I.close()
