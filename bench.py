@@ -131,7 +131,7 @@ def profile_traffic(kernel: str, workload: str):
 def kernel_source_hash() -> str:
     import hashlib
     hs = hashlib.sha256()
-    for name in ("qieo_device.cuh", "qieo_kernels.cuh", "qieo_api.cu"):
+    for name in ("qieo_device.cuh", "qieo_kernels.cuh", "qieo_column.cuh", "qieo_api.cu"):
         with open(os.path.join(ROOT, "paper_2609_30862_gb300", "csrc", name), "rb") as fh:
             hs.update(fh.read())
     return hs.hexdigest()[:16]
@@ -785,10 +785,11 @@ def run_batched(a):
                  "t_int_us": t_int * 1e6,
                  "state_in_l2": state_bytes < L2_BYTES,
                  "traffic": profile_traffic("batch_generation_kernel" if a.per_generation
-                                            else "batch_run_kernel", "c4"),
+                                            else "column_batch_kernel", "c4"),
                  "kernel": ("batch_generation_kernel (one launch per generation for all members)"
                             if a.per_generation else
-                            "batch_run_kernel (one persistent launch per run for all members)"),
+                            "column_batch_kernel (one cooperative launch per run for all members; one row "
+                            "of angle indices a member, no state streamed: the 4 B figures do not apply)"),
                  "us_per_generation": launch_s * 1e6,
                  "traffic_per": "generation (the persistent launch divided by its generations)"})
     if roof["traffic"]:
@@ -811,8 +812,8 @@ def run_batched(a):
         "e2e": {"value": e2e_value, "unit": "solves/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "what": "256 x qieo_create_instance from host arrays + qieo_create_batch + qieo_batch_run + "
                         "256 x qieo_get_best + destroy, per step"},
-        # per step: n resets, then G + 1 batched launches, or the first generation's launch, one
-        # persistent launch for the others and the final CIP
+        # per step: n resets, then G + 1 batched launches, or the column form's run, allele planes
+        # and end
         "gpu_launches": a.steps * (n + (G + 1 if a.per_generation else 3)),
         "clocks": clocks,
         "one_launch_per_instance": {"value": world * n * single_steps / ts, "unit": "solves/s",
@@ -942,7 +943,7 @@ def run_served(a):
                         "alleles), wall clock over the stream; bytes are per request"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                      "frac": achieved / hbm_peak, "peak_source": "%s hbm_gbs" % peak_src,
-                     "traffic": None, "kernel": "batch_generation_kernel (server steps)",
+                     "traffic": None, "kernel": "column_batch_kernel (server steps)",
                      "note": "4 B per served gene-update over the stream's span, idle gaps between "
                              "arrivals included"},
         "gpu_launches": stats["kernel_launches"],

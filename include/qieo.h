@@ -160,7 +160,14 @@ qieo_status qieo_reset(qieo_instance *inst);
 
 /* Runs `generations` >= 0 generations from the current one (Fig. 1: QIP, Evaluation,
  * DetermineElite, CIP, per generation; the CIP of the last generation is applied before
- * returning, so run(a) followed by run(b) equals run(a + b)). Each generation is one kernel
+ * returning, so run(a) followed by run(b) equals run(a + b)).
+ * Rule R1 from equal rows (every run from generation 0 on) is the column form: R1 steps all
+ * qubits of a gene alike, so one row of angle indices is the population's state, and a run
+ * is one or two cooperative launches whose blocks wait, bounded, for one another between
+ * generations. Not with elite_on_host, byte state, a fitness that does not fit the packed
+ * elite key, or QIEO_FLAG_UNFUSED, _COOPERATIVE, _REGISTER_PREFETCH, _PER_GENERATION,
+ * _STREAMED, _SIXTEEN, _NO_FIXED_WORDS or _SPARSE_ALWAYS. Results do not depend on it.
+ * Otherwise each generation is one kernel
  * launch, chained to the next by programmatic dependent launch and replayed from a CUDA
  * graph when a run length repeats; instances of at most 2^22 genes (or any instance with
  * QIEO_FLAG_COOPERATIVE) run the whole run as one cooperative launch whose blocks meet at
@@ -206,7 +213,7 @@ qieo_status qieo_get_elite_history(qieo_instance *inst, int32_t first, int32_t n
  * that drew (ran QIP, Sec. III-B, with a Philox draw per qubit, after their CIP); the rest
  * were fixed (every qubit at theta = 0 or pi/2, |alpha|^2 or |beta|^2 = 1, Sec. I), so
  * their alleles were known without a draw (the fixed-allele pass of the dense form, the
- * stable vectors of the sparse form). np * ceil(ng / 8) means every vector drew; generations
+ * stable vectors of the sparse form, the dropped quads of the column form). np * ceil(ng / 8) means every vector drew; generations
  * run in a batch, or restored by a checkpoint load, report that value (they are not counted).
  * QIEO_ERR_INVALID for an instance without the words, out NULL or a range outside [0, t). */
 qieo_status qieo_get_drawn_vectors(qieo_instance *inst, int32_t first, int32_t n, int64_t *out);
@@ -214,7 +221,8 @@ qieo_status qieo_get_drawn_vectors(qieo_instance *inst, int32_t first, int32_t n
 /* The observation thresholds T[0 .. 2K] the device uses (2K+1 uint64). */
 qieo_status qieo_get_threshold_table(qieo_instance *inst, uint64_t *t_out);
 
-/* Launch shape of the fused generation kernel. Results do not depend on it (all sums are
+/* Launch shape of the fused generation kernel, for the runs that are not in the column form
+ * (see qieo_run; that form cuts its work by the genes that still draw). Results do not depend on it (all sums are
  * exact integers and every draw is keyed by gene, chromosome and generation). A row is cut
  * into tiles of lanes_per_row * warps_per_row vectors of 8 genes; a persistent grid of
  * grid_ctas blocks covers the ntile * np tile-rows, in equal contiguous shares when a share
@@ -354,12 +362,14 @@ qieo_status qieo_get_convergence(qieo_instance *inst, int32_t *stopped, int32_t 
 /* A batch: many instances advanced together (batching of independent QIEO solves; the
  * paper runs one problem at a time). The instances keep their own state, records and
  * generation counters; qieo_batch_run(b, G) is equivalent to qieo_run(inst, G) on every
- * member, bit for bit. The work of a generation (every member's tiles of rows) is cut into
+ * member, bit for bit. Members in the column form (see qieo_run) run all their generations in
+ * one cooperative launch per item-sum form, each on its own blocks. For the others, and for
+ * all members when one has QIEO_FLAG_PER_GENERATION, the work of a generation (every member's tiles of rows) is cut into
  * segments balanced over a grid of one block per resident slot; members are grouped by
  * item-sum form and rotation rule. By default a run is one persistent cooperative launch
  * per group for all its generations: blocks take (generation, segment) items from one queue
  * in order, and a segment of an instance's next generation waits (bounded) only for that
- * instance's previous generation to close, not for the other members. When a member uses
+ * instance's previous generation to close, not for the other members. When one of these uses
  * QIEO_FLAG_CONVERGE or QIEO_FLAG_PER_GENERATION, a run is instead one launch per group and
  * generation (replayed from a CUDA graph when a run length repeats). A wait that runs out
  * sets the member's error word (QIEO_ERR_TIMEOUT from its next checked call). Members must
@@ -396,8 +406,8 @@ qieo_status qieo_autotune(qieo_instance *inst, int32_t trial_generations,
  * A server reserves one device arena for resident populations and runs a worker thread:
  * submitted requests queue in arrival order and are admitted, as arena memory and the
  * active-solve limit allow, into the set of resident solves; every scheduling step runs
- * gens_per_step generations of all resident solves with the batched kernel (one launch per
- * generation), and a solve that reaches its generation count leaves, freeing its memory
+ * gens_per_step generations of all resident solves (fewer where one ends before) with the
+ * batched kernels, and a solve that reaches its generation count leaves, freeing its memory
  * for the next arrivals. Each result is bit-identical to qieo_run on the same problem and
  * params alone. */
 typedef struct qieo_server qieo_server;
@@ -442,8 +452,8 @@ qieo_status qieo_server_poll(qieo_server *server, int64_t id, int32_t wait_ms, u
                              qieo_solve_result *result);
 
 /* Counters of a server since its creation. kernel_launches counts every kernel the server
- * put on the GPU (one initialisation per admitted solve; per step and group of members,
- * one batched launch per generation plus the final rotation). */
+ * put on the GPU (one initialisation per admitted solve; per step and group of members, three
+ * launches in the column form, otherwise one per generation plus the final rotation). */
 typedef struct {
     int64_t submitted, admitted, completed, steps, kernel_launches;
     int32_t queued, active;   /* now */

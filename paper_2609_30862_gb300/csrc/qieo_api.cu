@@ -2337,6 +2337,17 @@ ColumnBatchFn column_batch_fn(int form)
                      : form == 1 ? &qieo::column_batch_kernel<1> : &qieo::column_batch_kernel<2>;
 }
 
+// What the batched kernels read of a member (the draws of generations run in a batch are not counted).
+qieo::ColMember column_member(const qieo_instance *q)
+{
+    qieo::ColMember m;
+    std::memset(&m, 0, sizeof m);                   // (compared by bytes)
+    m.p = q->gp;
+    m.c = q->cp;
+    m.p.hist_d = nullptr;
+    return m;
+}
+
 // Time of a generation of a member on s blocks, us: the chain from one generation's elite to the
 // next (2 to 4 us) and the passes of the block with the longest share (see column_geometry,
 // column_home). A pass takes 0.38 us with two blocks on the SM, and the list shortens during a
@@ -2379,10 +2390,7 @@ void plan_column_batch(const std::vector<qieo_instance *> &members, const std::v
     std::vector<double> alone((size_t)n);
     double lo = 0.0, total = 0.0, longest = 0.0;
     for (int i = 0; i < n; ++i) {
-        qieo::ColMember m{};
-        m.p = members[(size_t)i]->gp;
-        m.c = members[(size_t)i]->cp;
-        b.members.push_back(m);
+        b.members.push_back(column_member(members[(size_t)i]));
         alone[(size_t)i] = column_member_time(members[(size_t)i], 1);
         total += alone[(size_t)i];
         longest = std::max(longest, alone[(size_t)i]);
@@ -2802,9 +2810,7 @@ qieo_status upload_col_group(qieo_batch *bt, qieo_batch::ColGroup &g)
 {
     bool same = true;
     for (size_t i = 0; i < g.members.size(); ++i) {
-        qieo::ColMember m{};
-        m.p = g.members[i]->gp;
-        m.c = g.members[i]->cp;
+        const qieo::ColMember m = column_member(g.members[i]);
         if (std::memcmp(&m, &g.plan.members[i], sizeof m) == 0) continue;
         g.plan.members[i] = m;
         same = false;

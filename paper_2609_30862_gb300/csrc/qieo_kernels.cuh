@@ -11,11 +11,12 @@
 // The CIP of generation t is applied at the top of generation t+1 because the elite is a
 // grid-wide result, and once more after the last generation of a run.
 //
-// Two drivers of the same generation body:
+// This file holds the row-by-row forms, which rotate and draw every qubit of every row: rule R2,
+// populations whose rows differ, and runs whose flags ask for one. (Rule R1 from equal rows runs
+// in the column form, qieo_column.cuh.) Drivers of the same generation body:
 //   run_kernel         one cooperative launch per run: all generations, a bounded grid
-//                      barrier between them, and the final CIP (default path);
-//   generation_kernel  one launch per generation (host DetermineElite variant, and runs
-//                      that cannot be launched cooperatively), with cip_kernel at the end.
+//                      barrier between them, and the final CIP (at most 2^22 genes);
+//   generation_kernel  one launch per generation, with cip_kernel at the end.
 //
 // Data layout in device memory (row c = chromosome c, gene-fastest, Sec. V-D):
 //   state  uint16 4n, n = k + K in [0, 2K] (scaled by 4 so that it is the byte offset of

@@ -179,8 +179,8 @@ __device__ __forceinline__ long long warp_sum(long long s)
 // bytes are shifted by its misalignment with the neighbouring lane's, and only the first and
 // the last lane of the tile store partial words. A thread per 8 genes with element accesses
 // and two atomics each, which this replaces, spent its time on 1.3 M contended atomics and
-// on single-byte stores (512 x 10,007 genes, a whole call with its rotation: 170 us, now 27 us; this
-// kernel 19 us, of which its first loads and the last block's scan are about a third).
+// on single-byte stores (512 x 10,007 genes, a whole call with its rotation: 170 us, now 27 us, 19 of
+// them in this kernel).
 constexpr int kTileGenes = 256;
 
 template <int kThr>
