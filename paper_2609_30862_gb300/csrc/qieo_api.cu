@@ -1095,9 +1095,29 @@ cudaError_t launch_column_observe(qieo_instance *q, int32_t t)
     return cudaLaunchKernelEx(&cfg, column_observe_fn(q->col_form), q->gp, q->cp, t, (int32_t)part_rows);
 }
 
+// Runs of so few generations of at most so many genes are two plain launches a generation that draw
+// every gene, fixed or not: a pair takes 7 us for a small population (64 x 100; 19 us for 1,024 x
+// 10,000), the cooperative launches, the plane and the end of a run 15 us and 1 to 2 a generation (37
+// and 10). At 2^24 genes the draws of a generation take 8 us.
+constexpr int32_t kStepRun = 3;
+constexpr int64_t kStepGenes = (int64_t)1 << 24;
+
 // A run in the column form: one cooperative launch, the allele plane, the state between runs.
 qieo_status run_column(qieo_instance *q, int32_t G)
 {
+    if (G <= kStepRun && (int64_t)q->np * q->svec * 8 <= kStepGenes &&
+        !(q->flags & (QIEO_FLAG_TIME_KERNELS | QIEO_FLAG_TIME_GENERATIONS))) {
+        qieo_status st = ensure_column(q);
+        if (st != QIEO_OK) return st;
+        for (int32_t g = 0; g < G; ++g) {
+            CUDA_TRY(launch_column_observe(q, -1));
+            cudaLaunchAttribute attr[1];
+            cudaLaunchConfig_t cfg = launch_config(q, dim3(plane_tiles(q)), 0, attr);
+            CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_step_kernel, q->gp, q->cp));
+        }
+        q->state_valid = false;
+        return QIEO_OK;
+    }
     const bool timing = (q->flags & QIEO_FLAG_TIME_KERNELS) != 0, stamps = (q->flags & QIEO_FLAG_TIME_GENERATIONS) != 0;
     qieo_status st = ensure_column(q);
     if (st != QIEO_OK) return st;
@@ -2521,10 +2541,12 @@ qieo_status launch_column_batch(const ColumnBatch &b, int32_t G, cudaStream_t st
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     CUDA_TRY(cudaLaunchKernelEx(&cfg, column_batch_fn(b.form), b.d_members, b.d_tasks, b.d_first, G));
-    qieo::column_batch_plane_kernel<<<(unsigned)b.plane.size(), qieo::kThreads, 0, stream>>>(b.d_members, b.d_plane);
-    CUDA_TRY(cudaGetLastError());
-    qieo::column_batch_end_kernel<<<(unsigned)b.end.size(), qieo::kThreads, 0, stream>>>(b.d_members, b.d_end);
-    CUDA_TRY(cudaGetLastError());
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)b.plane.size());
+    CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_batch_plane_kernel, b.d_members, b.d_plane));
+    cfg.gridDim = dim3((unsigned)b.end.size());
+    CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_batch_end_kernel, b.d_members, b.d_end));
     return QIEO_OK;
 }
 

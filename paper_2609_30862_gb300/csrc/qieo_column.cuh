@@ -1627,6 +1627,7 @@ __global__ void __launch_bounds__(kThreads) column_expand_kernel(const GenParams
 // One generation of a row block from equal rows (a population sharded by rows, whose elite is picked
 // outside): the block's alleles, fitness and best key. A block keeps one tile's thresholds and items
 // for its rows, as in a run; the angle indices stay as they are until column_rotate_kernel.
+// t < 0: generation *p.gen of an instance, which column_step_kernel closes.
 // Bound by the integer pipes and, with 50 rows a block, by its start: 1,500 rows of 20,000 genes
 // 30 us, 38 us row by row with the state read (and the rotation 2.5 us, 15 us row by row).
 template <int kForm>
@@ -1647,6 +1648,17 @@ __global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenPa
     if (tid < 2) s_fix[tid] = 0;
     grid_dependency_wait();
     __syncthreads();
+    const bool step = t < 0;
+    if (step) {
+        if (column_stopped(p, c, (int)blockIdx.x)) return;
+        t = *p.gen;
+        // (no block of this launch reads the list's counts; column_step_kernel fills them again)
+        if (blockIdx.x == 0 && tid == 0) {
+            c.ctl[kCtlRan] = 1;
+            c.ctl[kCtlGen] = (int32_t)(c.head->nv + c.head->ns);
+            *c.head = ColSlot{};
+        }
+    }
     const ColGeom m = column_geometry((uint32_t)p.svec, 0u, p.np, (int)gridDim.x);
     const BlockShare b = tile_geometry(m.lanes, m.warps);
     const int tile = (int)blockIdx.x % m.ntile, part = (int)blockIdx.x / m.ntile;
@@ -1700,7 +1712,70 @@ __global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenPa
         column_flush<kForm>(p, c.sum_bits, m.ntile, s_row, n, s_fix, key, s_acc32, s_acc64);
     }
     // the generation counter then names the next generation, as after a run
-    if (blockIdx.x == 0 && tid == 0) *p.gen = t + 1;
+    if (!step && blockIdx.x == 0 && tid == 0) *p.gen = t + 1;
+    allow_dependent_launch();
+}
+
+// Closes a generation that column_observe_kernel drew for an instance: the elite from its key, CIP
+// of the one row, the best row if it improved, the list the next run starts with, and by the
+// last block the records. Runs of a few generations are these two launches each (see kStepRun): 64
+// rows of 100 genes, one generation: 7.8 us from call to call; 15.4 with the cooperative kernel, the
+// plane and the end, 9.4 in the resident form.
+__global__ void __launch_bounds__(kThreads) column_step_kernel(const GenParams p, const ColParams c)
+{
+    __shared__ uint32_t s_thr[kMaxThr];
+    __shared__ int s_last;
+    load_thresholds(p, s_thr);
+    grid_dependency_wait();
+    __syncthreads();
+    if (c.ctl[kCtlRan] == 0) return;              // (stopped by convergence)
+    const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(s_thr);
+    const uint32_t off_top = (uint32_t)(8 * p.K), k8 = off_top * 0x00010001u;
+    const int32_t t = *p.gen;
+    const unsigned long long key = p.keys[t % 3];
+    const int32_t e0 = (int32_t)(0xffffffu - (uint32_t)(key & 0xffffffull)), e = e0 >= 0 && e0 < p.np ? e0 : 0;
+    const int64_t f = (int64_t)(key >> 24) - kKeyBias;
+    const bool improved = p.best[1] < 0 || f > p.best[0];
+    const int vec = blockIdx.x * kThreads + threadIdx.x;
+    const bool act = vec < p.svec;
+    uint2 s[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+    uint32_t bits = 0u;
+    if (act) {
+        for (int h = 0; h < 2; ++h) {
+            const int q = 2 * vec + h;
+            const uint2 o = c.canon[q];
+            const Draw4 d = philox4x32_10_rk((uint32_t)q, (uint32_t)e, (uint32_t)t, 0u, p.rk0, p.rk1);
+            const uint32_t x = observe_quad(d, o, thr_bytes, off_top);
+            s[h] = step_quad(o, x, k8);
+            c.canon[q] = s[h];
+            bits |= x << (4 * h);
+        }
+        if (improved) p.best_row[vec] = (uint8_t)bits;
+    }
+    const bool fa = quad_fixed(s[0], off_top), fb = quad_fixed(s[1], off_top);
+    int64_t fw = 0, fv = 0;
+    if (act && fa) quad_sums(p, 2 * vec, s[0], fw, fv);
+    if (act && fb) quad_sums(p, 2 * vec + 1, s[1], fw, fv);
+    column_append(c.head, column_list(c, p.svec, 0), p.svec, act, true, 2 * vec, 2 * vec + 1, fa, fb, fw, fv);
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atom_add_acq_rel(reinterpret_cast<unsigned int *>(c.ctl + kCtlTicket), 1u) == gridDim.x - 1u ? 1 : 0;
+    __syncthreads();
+    if (!s_last || threadIdx.x != 0) return;
+    c.ctl[kCtlTicket] = 0;
+    if (e != e0) atomicOr(p.error, kErrEliteRange);
+    int32_t run = 0;
+    if (p.converge) {
+        const int32_t before = t > 0 ? p.conv[(t - 1) & 1] : 0;
+        run = before > 0 && f == p.hist_f[t - 1] ? before + 1 : 1;
+        if (run >= kConvergeWindow) {
+            p.conv[3] = t;
+            p.conv[2] = kStopped;
+        }
+    }
+    column_record(p, t, e, f, improved, run, (uint32_t)c.ctl[kCtlGen]);
+    *p.gen = t + 1;
+    *p.bar_gen = t + 1;
+    p.keys[0] = p.keys[1] = p.keys[2] = 0ull;
 }
 
 // CIP of a row block with equal rows toward an elite row supplied from outside: bytes of 0 or 1,
@@ -1769,6 +1844,7 @@ __global__ void __launch_bounds__(kThreads) column_batch_plane_kernel(const ColM
 {
     __shared__ ColMember s_m;
     __shared__ uint32_t s_thr[kMaxThr];
+    grid_dependency_wait();
     const ColTask k = tasks[blockIdx.x];
     load_member(s_m, members + k.member);
     load_thresholds(s_m.p, s_thr);
@@ -1780,6 +1856,7 @@ __global__ void __launch_bounds__(kThreads) column_batch_end_kernel(const ColMem
 {
     __shared__ ColMember s_m;
     __shared__ uint32_t s_thr[kMaxThr];
+    grid_dependency_wait();
     const ColTask k = tasks[blockIdx.x];
     load_member(s_m, members + k.member);
     load_thresholds(s_m.p, s_thr);

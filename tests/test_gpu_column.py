@@ -268,3 +268,31 @@ def test_row_blocks(ng, np_, D, items, start):
         assert np.array_equal(np.concatenate([I.alleles() for I in blocks]), st.x)
     for I in blocks:
         I.close()
+
+
+@pytest.mark.parametrize("ng,np_,D,items,chunks", [
+    (1, 1, 4, "byte", [1] * 6), (50, 33, 100, "byte", [1] * 90), (1023, 40, 100, "byte", [1] * 70 + [20] + [1] * 5),
+    (700, 300, 12, "wide", [1] * 20 + [3, 1]), (4100, 130, 100, "mid", [30, 1, 1, 25, 1]),
+    (40000, 400, 8, "byte", [1, 4, 1, 1]), (300, 20000, 16, "byte", [1, 7, 1]),
+])
+def test_runs_of_one_generation(ng, np_, D, items, chunks):
+    """Runs of one generation (two plain launches) between longer ones, through the points where genes
+    reach their bounds."""
+    prob, gens = _problem(ng, items), sum(chunks)
+    st = O.run(prob, np_, gens, seed=ng, inst=3, D=D, lam=2, kind="omp")
+    with Q.Instance(prob, np_, seed=ng, inst=3, D=D, lam=2) as I:
+        for solve in range(2):
+            for g in chunks:
+                I.run(g)
+            check(I, st, gens)
+            I.reset()
+    conv = W.knapsack(60, 21)
+    ref = O.run(conv, 17, 600, seed=21, window=20)
+    n = int(ref.t[0])
+    with Q.Instance(conv, 17, seed=21, flags=Q.QIEO_FLAG_CONVERGE) as I:
+        for _ in range(n + 7):
+            I.run(1)
+        k, t = I.state()
+        assert ref.stopped and t == n and np.array_equal(k, ref.k)
+        assert np.array_equal(I.history(0, n)[0], ref.hist_e)
+        assert np.array_equal(I.best()[0], ref.best_x) and I.convergence() == (True, 20)
