@@ -792,10 +792,15 @@ qieo_status configure_column(qieo_instance *q)
 {
     if (!q->col_mem) return QIEO_OK;
     const size_t sv = (size_t)q->svec;
-    // packed sums as in the row-by-row forms (items in [0, 255], row sums below 2^26, at most
-    // 4,095 tiles of 256 vectors); items in [0, 2^20) keep a tile-row's sum below 2^31
+    // Most tiles that column_home cuts a list of this population into, on any of the grids (up to three
+    // blocks per SM; a batch's member may have fewer): a list that fills n tiles gets whole
+    // turns of the blocks, fewer than n + min(n, blocks).
+    const int64_t tiles = ((int64_t)sv + qieo::kThreads - 1) / qieo::kThreads;
+    const int64_t cut = tiles + std::min<int64_t>(tiles, 3 * (int64_t)q->sm_count) - 1;
+    // packed sums as in the row-by-row forms (items in [0, 255], row sums below 2^26, a tile
+    // count of 12 bits); items in [0, 2^20) keep a tile-row's sum below 2^31
     const bool wide = (q->flags & QIEO_FLAG_FORCE_WIDE) != 0;
-    if (!wide && q->narrow_items && q->sum_w < (1ll << 26) && q->sum_v < (1ll << 26) && sv <= (size_t)4095 * qieo::kThreads)
+    if (!wide && q->narrow_items && q->sum_w < (1ll << 26) && q->sum_v < (1ll << 26) && cut <= 4095)
         q->col_form = 0;
     else
         q->col_form = !wide && q->small_items ? 1 : 2;
@@ -822,11 +827,9 @@ qieo_status configure_column(qieo_instance *q)
     qieo::ColParams &c = q->cp;
     c.one = 1u;
     {
-        // (a list is cut into less than twice as many tiles as it fills)
-        const int64_t tiles = 2 * (((int64_t)sv + qieo::kThreads - 1) / qieo::kThreads);
         int bits = 1;
         while (bits < 31 && std::max(q->sum_w, q->sum_v) >> bits) ++bits;
-        c.sum_bits = q->col_form == 1 && std::max(q->sum_w, q->sum_v) >> bits == 0 && tiles < (int64_t)1 << std::min(62, 64 - 2 * bits) ? bits : 0;
+        c.sum_bits = q->col_form == 1 && std::max(q->sum_w, q->sum_v) >> bits == 0 && cut < (int64_t)1 << std::min(62, 64 - 2 * bits) ? bits : 0;
     }
     c.canon = reinterpret_cast<uint2 *>(b);
     c.rows = reinterpret_cast<uint2 *>(b + rows);

@@ -296,3 +296,26 @@ def test_runs_of_one_generation(ng, np_, D, items, chunks):
         assert ref.stopped and t == n and np.array_equal(k, ref.k)
         assert np.array_equal(I.history(0, n)[0], ref.hist_e)
         assert np.array_equal(I.best()[0], ref.best_x) and I.convergence() == (True, 20)
+
+
+def _few_bits(ng):
+    """Items of three bits: with millions of genes a row's sums still fit the packed row word."""
+    r = np.random.RandomState(ng)
+    w, v = r.randint(0, 8, ng), r.randint(0, 8, ng)
+    return W.custom_problem(w, v, int(w.sum()) // 2)
+
+
+@pytest.mark.parametrize("ng,np_,items", [(640_001, 3, "byte"), (1_000_003, 2, "wide"), (8_190_001, 3, "bits")])
+def test_more_tiles_than_blocks(ng, np_, items):
+    """Lists that a grid covers in several turns, cut into more tiles than they fill; 8,190,001 genes
+    fill 4,000 tiles, whose cut no longer fits the 12-bit count of a packed row word. Alone, and as a
+    member of a batch (fewer blocks each)."""
+    prob = _few_bits(ng) if items == "bits" else _problem(ng, items)
+    st = O.run(prob, np_, 6, seed=ng, inst=3, lam=2, kind="omp")
+    with Q.Instance(prob, np_, seed=ng, inst=3, lam=2) as I, Q.Instance(prob, np_, seed=9, inst=1, lam=2) as J:
+        I.run(6)
+        check(I, st, 6)
+        I.reset()
+        with Q.Batch([I, J]) as b:
+            b.run(6)
+        check(I, st, 6)
