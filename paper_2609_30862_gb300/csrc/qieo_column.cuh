@@ -930,6 +930,12 @@ __device__ __forceinline__ bool column_stopped(const GenParams &p, const ColPara
     return true;
 }
 
+// Whether an earlier wait of the instance ran out (one thread; its block shares the answer, since
+// another block may set the word meanwhile). The words of such a run are not those of any
+// generation, so nothing runs on them until a reset: column_begin has left kCtlRan 0, and the
+// launches that follow change neither the records nor the generation counter.
+__device__ __forceinline__ bool column_failed(const GenParams &p) { return ld_acquire(p.error) != 0; }
+
 __device__ __forceinline__ void column_begin(const GenParams &p, const ColParams &c, int32_t t0, bool draws)
 {
     c.ctl[kCtlRan] = 0;
@@ -991,6 +997,7 @@ __device__ __forceinline__ void column_run(const GenParams &p, const ColParams &
         sh.fix[1] = (int64_t)c.head->fv;
         sh.slot = ColSlot{};
         sh.debt = 0.0f;
+        sh.ok = column_failed(p) ? 0 : 1;
     }
     const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(sh.thr);
     const uint32_t off_top = (uint32_t)(8 * p.K), k8 = off_top * 0x00010001u;
@@ -1014,6 +1021,7 @@ __device__ __forceinline__ void column_run(const GenParams &p, const ColParams &
     int32_t g = 0, e = 0;
     bool improved = false, stop = false;
     __syncthreads();
+    if (!sh.ok) return;
 
     for (; !kMember || m.items != 0; ++g) {
         const int32_t t = t0 + g;
@@ -1194,6 +1202,7 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
         s_fix[1] = (int64_t)from->fv;
         s_slot = ColSlot{};
         for (int i = 0; i < 4; ++i) s_sync[i] = ColSync{};
+        s_ok = column_failed(p) ? 0 : 1;          // (column_run_kernel's wait, among others)
     }
     int32_t g = phase ? c.ctl[kCtlGen] : 0, e = phase ? c.ctl[kCtlElite] : 0;
     int cur = phase ? c.ctl[kCtlCur] : 0;
@@ -1252,6 +1261,7 @@ __global__ void __launch_bounds__(kThreads, 2) column_small_kernel(const GenPara
     bool have = true;                             // generation t0 + g - 1's elite is known
     int q = 0;                                    // the pass of the pair below
     __syncthreads();
+    if (!s_ok) return;
     if (m.items != 0) load(g == 0 ? c.canon : column_parity(c, p.svec, t0 + g + 1));
 
     while (m.items != 0) {
@@ -1651,6 +1661,10 @@ __global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenPa
     const bool step = t < 0;
     if (step) {
         if (column_stopped(p, c, (int)blockIdx.x)) return;
+        if (*p.error != 0) {                      // (no launch before this one is still running)
+            if (blockIdx.x == 0 && tid == 0) c.ctl[kCtlRan] = 0;
+            return;
+        }
         t = *p.gen;
         // (no block of this launch reads the list's counts; column_step_kernel fills them again)
         if (blockIdx.x == 0 && tid == 0) {

@@ -319,3 +319,27 @@ def test_more_tiles_than_blocks(ng, np_, items):
         with Q.Batch([I, J]) as b:
             b.run(6)
         check(I, st, 6)
+
+
+@pytest.mark.parametrize("ng,np_", [(400, 300), (2000, 300), (5000, 100), (20000, 1000)])
+def test_timed_out_run_is_reported_until_the_reset(ng, np_):
+    """Blocks that meet at the grid barrier, in column_small_kernel and (20,000 x 1,000, long shares
+    from a queue, with column_small_kernel launched behind it) in column_run_kernel: a 1 ns bound
+    runs out and is reported; later runs, of one generation or many, do nothing to the population
+    until the reset, after which a run is right again."""
+    prob = W.knapsack(ng, 16)
+    with Q.Instance(prob, np_, seed=16) as I:
+        I.set_wait_timeout(1)
+        I.run(30)
+        with pytest.raises(Q.QieoError) as e:
+            I.synchronize()
+        assert e.value.status == Q.QIEO_ERR_TIMEOUT
+        I.set_wait_timeout(10 * 10**9)
+        for g in (1, 30):
+            I.run(g)
+            with pytest.raises(Q.QieoError) as e:
+                I.best()
+            assert e.value.status == Q.QIEO_ERR_TIMEOUT
+        I.reset()
+        I.run(30)
+        check(I, O.run(prob, np_, 30, seed=16, kind="omp"), 30)
