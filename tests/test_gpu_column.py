@@ -343,3 +343,22 @@ def test_timed_out_run_is_reported_until_the_reset(ng, np_):
         I.reset()
         I.run(30)
         check(I, O.run(prob, np_, 30, seed=16, kind="omp"), 30)
+
+
+def test_row_by_row_batch_wait_that_runs_out_is_reported():
+    """Members of rule R2 run row by row: batch_run_kernel's bounded wait for a member's previous
+    generation. The member whose bound is 1 ns reports the timeout, the other is unaffected."""
+    probs = [W.knapsack(3000, 41), W.knapsack(2500, 42)]
+    with Q.Instance(probs[0], 120, seed=41, rule=1) as a, Q.Instance(probs[1], 90, seed=42, rule=1) as b:
+        a.set_wait_timeout(1)
+        with Q.Batch([a, b]) as bt:
+            bt.run(6)
+        with pytest.raises(Q.QieoError) as e:
+            a.synchronize()
+        assert e.value.status == Q.QIEO_ERR_TIMEOUT
+        check(b, O.run(probs[1], 90, 6, seed=42, rule=1), 6)
+        a.set_wait_timeout(10 * 10**9)
+        a.reset()
+        with Q.Batch([a]) as bt:
+            bt.run(6)
+        check(a, O.run(probs[0], 120, 6, seed=41, rule=1), 6)
