@@ -426,7 +426,8 @@ typedef struct {
 
 typedef struct {
     int32_t state;            /* QIEO_SOLVE_* */
-    int32_t status;           /* qieo_status of a failed solve */
+    int32_t status;           /* qieo_status of a failed solve (QIEO_ERR_TIMEOUT: one of its waits
+                               * between blocks ran out; other solves are not affected) */
     int64_t fitness;          /* best-so-far record of the solve (see qieo_get_best) */
     int32_t generation, chromosome;
     double submit_s, admit_s, done_s;   /* seconds on the server's clock */
@@ -462,6 +463,10 @@ typedef struct {
 } qieo_server_stats;
 
 qieo_status qieo_server_get_stats(qieo_server *server, qieo_server_stats *out);
+
+/* Bound of one wait between the blocks of a solve (see qieo_set_wait_timeout), for the solves
+ * submitted from now on, in nanoseconds (default 10 s; >= 1). */
+qieo_status qieo_server_set_wait_timeout(qieo_server *server, int64_t ns);
 
 /* Cancels a request that is still queued (QIEO_ERR_BUSY once it runs). */
 qieo_status qieo_server_cancel(qieo_server *server, int64_t id);

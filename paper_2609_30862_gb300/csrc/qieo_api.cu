@@ -1314,6 +1314,12 @@ qieo_status run_unfused(qieo_instance *q, int32_t G)
     return QIEO_OK;
 }
 
+// What an instance's error word says.
+qieo_status error_status(int32_t err)
+{
+    return err & qieo::kErrBarrierTimeout ? QIEO_ERR_TIMEOUT : err & qieo::kErrEliteRange ? QIEO_ERR_CUDA : QIEO_OK;
+}
+
 // Waits for the instance's stream and reports a device-side wait that ran out.
 qieo_status wait_checked(qieo_instance *q)
 {
@@ -3175,6 +3181,7 @@ struct SolveRequest {
     int64_t best[3] = {0, -1, -1};
     std::vector<uint8_t> best_row;
     int32_t gens_run = 0, converged = 0;
+    int64_t wait_ns = (int64_t)kDefaultBarrierWaitNs;
 };
 
 struct StepRecord {
@@ -3215,6 +3222,7 @@ struct qieo_server {
     int bps[2] = {1, 1};                 // batch kernel blocks per SM: [wide, narrow]
     int64_t n_submitted = 0, n_admitted = 0, n_completed = 0, n_steps = 0, n_launches = 0;
     int32_t max_active_seen = 0;
+    int64_t wait_ns = (int64_t)kDefaultBarrierWaitNs;   // of solves submitted from now on
 };
 
 namespace {
@@ -3393,21 +3401,26 @@ void retire_oldest_step(qieo_server *S)
         }
     }
     // All their results through a pinned buffer, one wait (a copy to pageable memory is a wait of its
-    // own, about 12 us): the record, the generations and the row of each.
+    // own, about 12 us): the record and the generations (parts of the block that follow one another),
+    // the error word and the row of each.
+    constexpr size_t kRowAt = 512;
     int32_t copy_st = step_st;
     char *pin = nullptr;
     size_t bytes = 0;
-    for (SolveRequest *R : rec.finishing) bytes += 64 + (size_t)R->inst->xstride;
+    const auto gen_at = [](const qieo_instance *q) {
+        return (size_t)(reinterpret_cast<char *>(q->gp.gen) - reinterpret_cast<char *>(q->gp.best));
+    };
+    for (SolveRequest *R : rec.finishing) bytes += kRowAt + (size_t)R->inst->xstride;
     if (copy_st == QIEO_OK && bytes != 0) {
         copy_st = pinned_scratch(bytes, &pin);
         bool ok = copy_st == QIEO_OK;
         char *at = pin;
         for (size_t i = 0; ok && i < rec.finishing.size(); ++i) {
             qieo_instance *q = rec.finishing[i]->inst;
-            ok = cudaMemcpyAsync(at, q->gp.best, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess &&
-                 cudaMemcpyAsync(at + 24, q->gp.gen, sizeof(int32_t), cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess &&
-                 cudaMemcpyAsync(at + 64, q->gp.best_row, (size_t)q->xstride, cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess;
-            at += 64 + q->xstride;
+            ok = cudaMemcpyAsync(at, q->gp.best, gen_at(q) + sizeof(int32_t), cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess &&
+                 cudaMemcpyAsync(at + kRowAt - 8, q->gp.error, sizeof(int32_t), cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess &&
+                 cudaMemcpyAsync(at + kRowAt, q->gp.best_row, (size_t)q->xstride, cudaMemcpyDeviceToHost, S->copy_stream) == cudaSuccess;
+            at += kRowAt + q->xstride;
         }
         // (also after a failure: nothing may still write the buffer)
         if (cudaStreamSynchronize(S->copy_stream) != cudaSuccess) ok = false;
@@ -3415,17 +3428,23 @@ void retire_oldest_step(qieo_server *S)
     }
     for (SolveRequest *R : rec.finishing) {
         qieo_instance *q = R->inst;
-        const int32_t st = copy_st;
-        if (st == QIEO_OK) {
-            std::memcpy(R->best, pin, sizeof R->best);
-            std::memcpy(&R->gens_run, pin + 24, sizeof R->gens_run);
-            R->best_row.assign(pin + 64, pin + 64 + q->xstride);
-            pin += 64 + q->xstride;
+        int32_t st = copy_st;
+        if (copy_st == QIEO_OK) {
+            // A wait of this solve that ran out fails it alone; its step is over.
+            int32_t err = 0;
+            std::memcpy(&err, pin + kRowAt - 8, sizeof err);
+            st = error_status(err);
+            if (st == QIEO_OK) {
+                std::memcpy(R->best, pin, sizeof R->best);
+                std::memcpy(&R->gens_run, pin + gen_at(q), sizeof R->gens_run);
+                R->best_row.assign(pin + kRowAt, pin + kRowAt + q->xstride);
+            }
+            pin += kRowAt + q->xstride;
         }
         destroy_instance_nosync(q);
         std::lock_guard<std::mutex> lock(S->mu);
         R->inst = nullptr;
-        if (st == QIEO_OK) S->alloc.release(R->off, R->bytes);   // a failed step keeps its memory
+        if (copy_st == QIEO_OK) S->alloc.release(R->off, R->bytes);   // a failed step keeps its memory
         R->status = st;
         R->state = st == QIEO_OK ? QIEO_SOLVE_DONE : QIEO_SOLVE_FAILED;
         R->t_done = server_now(S);
@@ -3470,6 +3489,7 @@ void server_loop(qieo_server *S)
             R->t_admit = server_now(S);
             if (st == QIEO_OK) {
                 R->inst = q;
+                q->gp.wait_ns = (uint64_t)R->wait_ns;
                 R->remaining = R->gens;
                 R->state = QIEO_SOLVE_RUNNING;
                 S->active.push_back(R);
@@ -3642,6 +3662,7 @@ qieo_status qieo_server_submit(qieo_server *S, const qieo_problem *pr, const qie
     R->bytes = bytes;
     std::lock_guard<std::mutex> lock(S->mu);
     if (S->stop) return fail(QIEO_ERR_INVALID, "server is stopping");
+    R->wait_ns = S->wait_ns;
     R->id = S->next_id++;
     R->t_submit = server_now(S);
     S->n_submitted += 1;
@@ -3690,6 +3711,15 @@ qieo_status qieo_server_get_stats(qieo_server *S, qieo_server_stats *out)
     out->active = (int32_t)S->active.size();
     out->max_active = S->max_active_seen;
     out->reserved = 0;
+    return QIEO_OK;
+}
+
+qieo_status qieo_server_set_wait_timeout(qieo_server *S, int64_t ns)
+{
+    if (!S) return fail(QIEO_ERR_INVALID, "server is NULL");
+    if (ns < 1) return fail(QIEO_ERR_INVALID, "wait timeout must be >= 1 ns");
+    std::lock_guard<std::mutex> lock(S->mu);
+    S->wait_ns = ns;
     return QIEO_OK;
 }
 

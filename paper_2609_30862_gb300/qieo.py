@@ -55,7 +55,8 @@ EXPORTS = (
     "qieo_checkpoint_save", "qieo_checkpoint_load", "qieo_philox",
     "qieo_generation_noalloc", "qieo_create_batch", "qieo_batch_run", "qieo_destroy_batch",
     "qieo_run_batch", "qieo_autotune", "qieo_server_create", "qieo_server_submit", "qieo_server_poll",
-    "qieo_server_get_stats", "qieo_server_cancel", "qieo_server_destroy", "qieo_last_error",
+    "qieo_server_get_stats", "qieo_server_set_wait_timeout", "qieo_server_cancel", "qieo_server_destroy",
+    "qieo_last_error",
 )
 
 QIEO_SOLVE_QUEUED = 0
@@ -138,6 +139,7 @@ def load(build_if_missing: bool = True) -> C.CDLL:
         "qieo_reset": ([P], C.c_int),
         "qieo_run": ([P, i32], C.c_int),
         "qieo_set_wait_timeout": ([P, i64], C.c_int),
+        "qieo_server_set_wait_timeout": ([P, i64], C.c_int),
         "qieo_synchronize": ([P], C.c_int),
         "qieo_get_best": ([P, P, P, P, P], C.c_int),
         "qieo_get_state": ([P, P, P], C.c_int),
@@ -438,6 +440,10 @@ def qieo_server_get_stats(h) -> qieo_server_stats:
     return st
 
 
+def qieo_server_set_wait_timeout(h, ns: int) -> None:
+    _check(load().qieo_server_set_wait_timeout(h, int(ns)))
+
+
 def qieo_server_cancel(h, rid: int) -> None:
     _check(load().qieo_server_cancel(h, int(rid)))
 
@@ -466,6 +472,9 @@ class Server:
 
     def poll(self, rid: int, wait_ms: int = 0):
         return qieo_server_poll(self.h, rid, wait_ms, self.ng.get(rid, 0))
+
+    def set_wait_timeout(self, ns: int) -> None:
+        qieo_server_set_wait_timeout(self.h, ns)
 
     def cancel(self, rid: int) -> None:
         qieo_server_cancel(self.h, rid)

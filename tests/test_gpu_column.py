@@ -362,3 +362,25 @@ def test_row_by_row_batch_wait_that_runs_out_is_reported():
         with Q.Batch([a]) as bt:
             bt.run(6)
         check(a, O.run(probs[0], 120, 6, seed=41, rule=1), 6)
+
+
+def test_served_solve_whose_wait_runs_out_fails_alone():
+    """A served solve on several blocks whose waits are bounded by 1 ns is reported as failed with the
+    timeout; solves beside it, and one that needs the arena memory it leaves, are right."""
+    prob, small = W.knapsack(20000, 5), W.knapsack(300, 6)
+    with Q.Server(memory_bytes=64 << 20, gens_per_step=7) as srv:
+        before = srv.submit(small, 40, 60, seed=1)
+        srv.set_wait_timeout(1)
+        bad = [srv.submit(prob, 500, 60, seed=2), srv.submit(prob, 500, 60, seed=2, flags=Q.QIEO_FLAG_CONVERGE)]
+        srv.set_wait_timeout(10 * 10**9)
+        after = srv.submit(prob, 500, 60, seed=3)
+        for rid in bad:
+            res, _ = srv.poll(rid, wait_ms=60000)
+            assert (res.state, res.status) == (Q.QIEO_SOLVE_FAILED, Q.QIEO_ERR_TIMEOUT)
+        for rid, p, n, seed in ((before, small, 40, 1), (after, prob, 500, 3)):
+            res, bits = srv.poll(rid, wait_ms=60000)
+            ref = O.run(p, n, 60, seed=seed, kind="omp")
+            assert res.state == Q.QIEO_SOLVE_DONE
+            assert (res.fitness, res.generation, res.chromosome) == tuple(int(v) for v in ref.best)
+            assert np.array_equal(bits, ref.best_x)
+        assert srv.stats()["completed"] == 2
