@@ -41,6 +41,16 @@ def stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps())
 
 
+def objects() -> list[str]:
+    """The object of every translation unit, in the order of sources()."""
+    return [os.path.join(BUILD, os.path.basename(src)[:-3] + ".o") for src in sources()]
+
+
+def link(out: str, *more: str) -> None:
+    """Link the objects, and whatever else is given, into a shared library."""
+    subprocess.check_call([nvcc(), "-gencode", GENCODE, "-shared", *objects(), *more, "-o", out])
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every translation unit to an object in parallel, then link the library."""
     if not force and not stale():
@@ -51,22 +61,18 @@ def build(force: bool = False, verbose: bool = False) -> str:
     common = [nvcc(), "-gencode", GENCODE, "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
               *(["-Xptxas", "-v"] if verbose else [])]
-    objs = [os.path.join(BUILD, os.path.basename(src)[:-3] + ".%s.o" % tag) for src in sources()]
 
     def compile_one(pair):
         src, obj = pair
-        subprocess.check_call(common + ["-c", src, "-o", obj])
+        tmp = obj + ".tmp" + tag
+        subprocess.check_call(common + ["-c", src, "-o", tmp])
+        os.replace(tmp, obj)
 
-    try:
-        with ThreadPoolExecutor(max_workers=max(1, len(objs))) as ex:
-            list(ex.map(compile_one, zip(sources(), objs)))
-        tmp = LIB + ".tmp" + tag
-        subprocess.check_call([nvcc(), "-gencode", GENCODE, "-shared", *objs, "-o", tmp])
-        os.replace(tmp, LIB)
-    finally:
-        for obj in objs:
-            if os.path.exists(obj):
-                os.remove(obj)
+    with ThreadPoolExecutor(max_workers=max(1, len(sources()))) as ex:
+        list(ex.map(compile_one, zip(sources(), objects())))
+    tmp = LIB + ".tmp" + tag
+    link(tmp)
+    os.replace(tmp, LIB)
     return LIB
 
 

@@ -2852,22 +2852,10 @@ qieo_status upload_col_group(qieo_batch *bt, qieo_batch::ColGroup &g)
     return QIEO_OK;
 }
 
-// Groups the members: those that run in the column form by item form, the others by item width and
-// rule. A member with QIEO_FLAG_PER_GENERATION keeps the whole batch row by row. Groups are built
-// again when a member changes form (a checkpoint whose rows differ).
-qieo_status group_members(qieo_batch *bt)
+// The groups of a batch that has none: members in the column form by item form, the others by item
+// width and rule.
+qieo_status build_groups(qieo_batch *bt, const std::vector<char> &as_column)
 {
-    bool per_gen = false;
-    for (const qieo_instance *q : bt->members) per_gen = per_gen || (q->flags & QIEO_FLAG_PER_GENERATION);
-    std::vector<char> as_column;
-    for (const qieo_instance *q : bt->members) as_column.push_back(!per_gen && use_column(q) ? 1 : 0);
-    if (as_column == bt->as_column) return QIEO_OK;
-    if (!bt->as_column.empty()) {
-        qieo_status st = wait_stream(bt->stream);
-        if (st != QIEO_OK) return st;
-        free_groups(bt);
-        bt->as_column.clear();
-    }
     // One persistent launch per run unless a member asks for one launch per generation or
     // uses the convergence test.
     bt->persistent = true;
@@ -2903,6 +2891,31 @@ qieo_status group_members(qieo_batch *bt)
     for (auto &g : bt->col_groups) {
         qieo_status st = build_col_group(bt, g);
         if (st != QIEO_OK) return st;
+    }
+    return QIEO_OK;
+}
+
+// Groups the members for the forms they run in now. A member with QIEO_FLAG_PER_GENERATION keeps the
+// whole batch row by row. Groups are built again when a member changes form (a checkpoint whose
+// rows differ). An attempt that fails (device memory) leaves none, and the next one starts anew.
+qieo_status group_members(qieo_batch *bt)
+{
+    bool per_gen = false;
+    for (const qieo_instance *q : bt->members) per_gen = per_gen || (q->flags & QIEO_FLAG_PER_GENERATION);
+    std::vector<char> as_column;
+    for (const qieo_instance *q : bt->members) as_column.push_back(!per_gen && use_column(q) ? 1 : 0);
+    if (as_column == bt->as_column) return QIEO_OK;
+    if (!bt->as_column.empty()) {
+        qieo_status st = wait_stream(bt->stream);
+        if (st != QIEO_OK) return st;
+        free_groups(bt);
+        bt->as_column.clear();
+    }
+    const qieo_status st = build_groups(bt, as_column);
+    if (st != QIEO_OK) {
+        free_groups(bt);
+        cudaGetLastError();      // (reported above; not again by the next launch)
+        return st;
     }
     bt->as_column = as_column;
     return QIEO_OK;
