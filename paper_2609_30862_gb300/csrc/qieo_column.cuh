@@ -852,7 +852,7 @@ __device__ __forceinline__ bool column_rebuild(const GenParams &p, const ColPara
     return true;
 }
 
-// Records of generation t with elite e of fitness f (one thread). drew: vectors on its list.
+// Records of generation t with elite e of fitness f (one thread). drew: vectors that it drew (those on its list).
 __device__ __forceinline__ void column_record(const GenParams &p, int32_t t, int32_t e, int64_t f, bool improved,
                                               int32_t run, uint32_t drew)
 {
@@ -1667,7 +1667,6 @@ __global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenPa
         // (no block of this launch reads the list's counts; column_step_kernel fills them again)
         if (blockIdx.x == 0 && tid == 0) {
             c.ctl[kCtlRan] = 1;
-            c.ctl[kCtlGen] = (int32_t)(c.head->nv + c.head->ns);
             *c.head = ColSlot{};
         }
     }
@@ -1784,7 +1783,7 @@ __global__ void __launch_bounds__(kThreads) column_step_kernel(const GenParams p
             p.conv[2] = kStopped;
         }
     }
-    column_record(p, t, e, f, improved, run, (uint32_t)c.ctl[kCtlGen]);
+    column_record(p, t, e, f, improved, run, (uint32_t)p.svec);      // (column_observe_kernel draws every vector)
     *p.gen = t + 1;
     *p.bar_gen = t + 1;
     p.keys[0] = p.keys[1] = p.keys[2] = 0ull;

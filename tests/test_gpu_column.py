@@ -384,3 +384,18 @@ def test_served_solve_whose_wait_runs_out_fails_alone():
             assert (res.fitness, res.generation, res.chromosome) == tuple(int(v) for v in ref.best)
             assert np.array_equal(bits, ref.best_x)
         assert srv.stats()["completed"] == 2
+
+
+def test_drawn_vectors_of_short_and_long_runs():
+    """A long run counts the vectors on its list; a run of one generation draws every vector, fixed or
+    not, and says so."""
+    prob, np_ = W.knapsack(8000, 5), 2000
+    with Q.Instance(prob, np_, seed=5, D=12) as I:
+        assert I.shape().fixed_words == 1
+        I.run(60)
+        I.run(1)
+        I.run(20)
+        got = I.drawn_vectors(0, 81)
+        assert got[0] == got[60] == np_ * 1000
+        assert got[59] < np_ * 100 and got[61:].max() < np_ * 100
+        check(I, O.run(prob, np_, 81, seed=5, D=12, kind="omp"), 81)
