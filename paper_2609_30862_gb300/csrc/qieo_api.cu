@@ -1182,7 +1182,15 @@ qieo_status run_device(qieo_instance *q, int32_t G)
         qieo_status st = ensure_events(q);
         if (st != QIEO_OK) return st;
     }
-    if (use_column(q)) return run_column(q, G);
+    // A run that is being captured must not hold the conversion from the full state: each replay
+    // would start from the same one.
+    bool column = use_column(q);
+    if (column && !q->col_valid) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        CUDA_TRY(cudaStreamIsCapturing(q->stream, &capture));
+        column = capture == cudaStreamCaptureStatusNone;
+    }
+    if (column) return run_column(q, G);
     if (q->col_mem) {
         qieo_status st = ensure_state(q);
         if (st != QIEO_OK) return st;
@@ -2293,13 +2301,16 @@ qieo_status qieo_checkpoint_load(qieo_instance *q, const void *buffer, size_t by
     if (st == QIEO_OK) st = upload(q, q->gp.state, p, h.state_bytes);
     if (st != QIEO_OK) return st;
     if (q->col_mem) {   // the column form needs equal rows
+        q->state_valid = true;
+        q->col_valid = false;
+        q->fword_dirty = true;
         const size_t row = h.state_bytes / (size_t)q->np;
         bool equal = true;
         for (int32_t c = 1; c < q->np && equal; ++c) equal = std::memcmp(p, p + (size_t)c * row, row) == 0;
         q->rows_equal = equal;
-        q->state_valid = true;
-        q->col_valid = false;
-        q->fword_dirty = true;
+        // The form's words now and not in the next run, which may be captured in a graph: each of
+        // its replays would start from the checkpoint again.
+        if (use_column(q)) st = ensure_column(q);
     }
     if (st == QIEO_OK) st = clear_fword(q, q->stream);   // the words of the reset state
     if (st == QIEO_OK) st = upload(q, q->gp.conv, h.conv, sizeof h.conv);

@@ -399,3 +399,36 @@ def test_drawn_vectors_of_short_and_long_runs():
         assert got[0] == got[60] == np_ * 1000
         assert got[59] < np_ * 100 and got[61:].max() < np_ * 100
         check(I, O.run(prob, np_, 81, seed=5, D=12, kind="omp"), 81)
+
+
+@pytest.mark.parametrize("start", ["checkpoint", "batch"])
+def test_captured_run_goes_on_with_every_replay(start):
+    """A run captured right after the population came from elsewhere: a checkpoint with equal rows, or a
+    batch that ran row by row (a member asks for one launch per generation). Each replay of the
+    graph continues where the one before stopped."""
+    torch = pytest.importorskip("torch")
+    prob, np_ = W.knapsack(2603, 5), 90
+    stream = torch.cuda.Stream()
+    with Q.Instance(prob, np_, seed=5, stream=stream.cuda_stream) as I:
+        if start == "checkpoint":
+            with Q.Instance(prob, np_, seed=5) as J:
+                J.run(12)
+                I.load(J.save())
+        else:
+            with Q.Instance(prob, np_, seed=6, stream=stream.cuda_stream, flags=Q.QIEO_FLAG_PER_GENERATION) as J:
+                with Q.Batch([I, J]) as b:
+                    b.run(12)
+                J.synchronize()
+        I.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            I.run(6)
+        for _ in range(4):
+            graph.replay()
+        torch.cuda.synchronize()
+        st = O.run(prob, np_, 36, seed=5)
+        k, t = I.state()
+        assert t == 36 and np.array_equal(k, st.k)
+        bits, bf, bg, bc = I.best()
+        assert (bf, bg, bc) == tuple(int(v) for v in st.best) and np.array_equal(bits, st.best_x)
+        assert np.array_equal(I.fitness(), st.f)
