@@ -1051,14 +1051,19 @@ cudaError_t launch_column_end(qieo_instance *q, int32_t from_rows)
     return cudaLaunchKernelEx(&cfg, qieo::column_end_kernel, q->gp, q->cp, from_rows);
 }
 
+// Blocks of a launch over the full state.
+int state_blocks(const qieo_instance *q)
+{
+    const size_t total = (size_t)q->np * q->svec;
+    return (int)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)q->sm_count * 8));
+}
+
 // The full state for the row-by-row forms (and, for batches, whatever the batched kernels read).
 qieo_status ensure_state(qieo_instance *q)
 {
     if (q->state_valid) return QIEO_OK;
-    const size_t total = (size_t)q->np * q->svec;
-    const int blocks = (int)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)q->sm_count * 8));
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = launch_config(q, dim3(blocks), 0, attr);
+    cudaLaunchConfig_t cfg = launch_config(q, dim3(state_blocks(q)), 0, attr);
     CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_expand_kernel, q->gp, q->cp));
     if (q->fword_state_bytes) {    // no vector known to be fixed
         CUDA_TRY(cudaMemsetAsync(q->fword_mem, 0, q->fword_state_bytes, q->stream));
@@ -2190,6 +2195,10 @@ struct CheckpointHeader {
 
 const char kCheckpointMagic[8] = {'Q', 'I', 'E', 'O', 'C', 'K', 'P', '1'};
 
+// Rows of a checkpoint up to this many bytes are compared on the host (0.05 us a KB); a launch and its
+// answer take 20 us.
+constexpr size_t kCompareOnHost = (size_t)512 << 10;
+
 size_t state_bytes_of(const qieo_instance *q)
 {
     return (size_t)q->np * q->svec * (q->state8 ? 8 : 16);
@@ -2265,6 +2274,9 @@ qieo_status qieo_checkpoint_save(qieo_instance *q, void *buffer, size_t bytes)
     if (st == QIEO_OK && h.t > 0) st = fetch(q, p, q->hist_f, (size_t)h.t * sizeof(int64_t));
     p += (size_t)h.t * sizeof(int64_t);
     if (st != QIEO_OK) return st;
+    // (repeating one row on the host takes as long as the copy at 20 MB, 7 % longer at 160 MB)
+    if (h.state_bytes > ((size_t)32 << 20)) st = ensure_state(q);
+    if (st != QIEO_OK) return st;
     if (q->state_valid) return fetch(q, p, q->gp.state, h.state_bytes);
     const size_t row = (size_t)q->svec * sizeof(uint4);   // every row is the column form's
     st = fetch(q, p, q->cp.canon, row);
@@ -2304,10 +2316,20 @@ qieo_status qieo_checkpoint_load(qieo_instance *q, const void *buffer, size_t by
         q->state_valid = true;
         q->col_valid = false;
         q->fword_dirty = true;
-        const size_t row = h.state_bytes / (size_t)q->np;
-        bool equal = true;
-        for (int32_t c = 1; c < q->np && equal; ++c) equal = std::memcmp(p, p + (size_t)c * row, row) == 0;
-        q->rows_equal = equal;
+        int32_t differ = 0;   // (the reset cleared the word)
+        if (h.state_bytes <= kCompareOnHost) {
+            const size_t row = h.state_bytes / (size_t)q->np;
+            for (int32_t c = 1; c < q->np && !differ; ++c) differ = std::memcmp(p, p + (size_t)c * row, row) != 0;
+        } else {
+            cudaLaunchAttribute attr[1];
+            cudaLaunchConfig_t cfg = launch_config(q, dim3(state_blocks(q)), 0, attr);
+            CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_compare_kernel, q->gp, q->cp));
+            CUDA_TRY(cudaMemcpyAsync(&differ, q->cp.ctl + qieo::kCtlDiffer, sizeof differ, cudaMemcpyDeviceToHost,
+                                     q->stream));
+            st = wait_stream(q->stream);
+            if (st != QIEO_OK) return st;
+        }
+        q->rows_equal = differ == 0;
         // The form's words now and not in the next run, which may be captured in a graph: each of
         // its replays would start from the checkpoint again.
         if (use_column(q)) st = ensure_column(q);

@@ -59,6 +59,8 @@ constexpr int kCtlRebuilds = 10;  // ... the rebuilds
 constexpr int kCtlElite = 11;     // ... the last elite
 constexpr int kCtlImproved = 12;  // ... whether it improved the best
 
+constexpr int kCtlDiffer = 13;    // column_compare_kernel: a row of the full state differs from row 0
+
 constexpr int kColPosted = 64;              // most blocks that meet through posts
 
 struct ColParams {
@@ -1620,6 +1622,20 @@ __global__ void __launch_bounds__(kThreads) column_reset_kernel(const GenParams 
         column_clear_words(c);
         for (int i = 0; i < 16; ++i) c.ctl[i] = 0;
     }
+}
+
+// Whether a row of the full state differs from row 0 (a checkpoint's may). Bound by memory; a host
+// comparison of the checkpoint's 20 MB (1,024 x 10,000) took 1 ms of the load's 2.6.
+__global__ void __launch_bounds__(kThreads) column_compare_kernel(const GenParams p, const ColParams c)
+{
+    grid_dependency_wait();
+    const size_t total = (size_t)p.np * p.svec, stride = (size_t)gridDim.x * kThreads;
+    bool differ = false;
+    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < total; i += stride) {
+        const uint4 a = p.state[i], b = __ldg(p.state + i % (size_t)p.svec);
+        differ = differ || a.x != b.x || a.y != b.y || a.z != b.z || a.w != b.w;
+    }
+    if (differ) c.ctl[kCtlDiffer] = 1;
 }
 
 // The full state from the state between runs (every row equal), for the row-by-row forms.

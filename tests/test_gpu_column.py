@@ -432,3 +432,21 @@ def test_captured_run_goes_on_with_every_replay(start):
         bits, bf, bg, bc = I.best()
         assert (bf, bg, bc) == tuple(int(v) for v in st.best) and np.array_equal(bits, st.best_x)
         assert np.array_equal(I.fitness(), st.f)
+
+
+@pytest.mark.parametrize("ng,np_,row", [(4096, 64, None), (4096, 64, 63), (4104, 64, None), (4104, 64, 1), (33, 9000, 8999),
+                                        (1, 1, None), (20001, 300, None), (20001, 300, 299)])
+def test_checkpoint_rows_are_compared(ng, np_, row):
+    """A loaded population, with equal rows or with one gene of one row changed, on both sides of the
+    size (512 KB: 4,096 x 64) from which the device compares the rows."""
+    prob = W.knapsack(ng, 4)
+    k0 = np.random.default_rng(ng).integers(-25, 26, size=(1, ng)).astype(np.int16).repeat(np_, 0)
+    if row is not None:
+        k0[row, ng - 1] = 25 if k0[row, ng - 1] < 25 else -25
+    st = O.State(np_, ng)
+    st.k[:] = k0
+    O.run(prob, np_, 9, seed=4, state=st)
+    with Q.Instance(prob, np_, seed=4) as I:
+        load_state(I, k0)
+        I.run(9)
+        check(I, st, 9)
