@@ -207,6 +207,8 @@ struct qieo_instance {
     bool state_valid = false;      // the full state holds the population
     bool col_valid = false;        // cp's state between runs holds it
     bool force_rows = false;       // autotuning: time the row-by-row forms
+    bool keep_state = false;       // member of a batch that runs row by row: a reset writes the full
+                                   // state too
 };
 
 namespace {
@@ -1715,9 +1717,10 @@ qieo_status qieo_reset(qieo_instance *q)
     const int blocks = std::max(1, std::min(q->sm_count * 4, (int)std::min<size_t>((words + 255) / 256, 1 << 20)));
     q->rows_equal = true;
     if (q->col_mem && column_capable(q)) {
-        qieo::column_reset_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, q->cp, xbytes, (size_t)q->np * 2);
+        qieo::column_reset_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, q->cp, q->keep_state ? words : 0, xbytes,
+                                                                           (size_t)q->np * 2);
         q->col_valid = true;
-        q->state_valid = false;
+        q->state_valid = q->keep_state;
     } else {
         qieo::init_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, words, xbytes, (size_t)q->np * 2);
         q->col_valid = false;
@@ -2951,6 +2954,16 @@ qieo_status group_members(qieo_batch *bt)
         return st;
     }
     bt->as_column = as_column;
+    // Members that could run in the column form but do not here have their full state from now on after
+    // a reset too: made by the batch's next run, it would be made again by every replay of a graph
+    // that this run was captured in.
+    for (size_t i = 0; i < bt->members.size(); ++i) {
+        qieo_instance *q = bt->members[i];
+        if (!q->col_mem || as_column[i]) continue;
+        q->keep_state = true;
+        const qieo_status made = ensure_state(q);
+        if (made != QIEO_OK) return made;
+    }
     return QIEO_OK;
 }
 

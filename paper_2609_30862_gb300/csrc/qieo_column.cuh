@@ -1599,13 +1599,13 @@ __global__ void __launch_bounds__(kThreads) column_end_kernel(const GenParams p,
 }
 
 // Generation 0 of an instance that runs in the column form: the words every form shares, one row
-// at pi/4, every vector on the list, no recorded best row. The full state is not written
-// (column_expand_kernel makes it when another form needs it).
-__global__ void __launch_bounds__(kThreads) column_reset_kernel(const GenParams p, const ColParams c, size_t xbytes,
-                                                                size_t acc_words)
+// at pi/4, every vector on the list, no recorded best row. The full state is written if state_words
+// is not 0 (column_expand_kernel makes it otherwise, when another form needs it).
+__global__ void __launch_bounds__(kThreads) column_reset_kernel(const GenParams p, const ColParams c, size_t state_words,
+                                                                size_t xbytes, size_t acc_words)
 {
     grid_dependency_wait();
-    init_words(p, 0, xbytes, acc_words);
+    init_words(p, state_words, xbytes, acc_words);
     const uint32_t kk = (uint32_t)(4 * p.K) * 0x00010001u;
     const int i0 = blockIdx.x * kThreads + threadIdx.x, stride = (int)gridDim.x * kThreads;
     for (int vec = i0; vec < p.svec; vec += stride) {

@@ -450,3 +450,33 @@ def test_checkpoint_rows_are_compared(ng, np_, row):
         load_state(I, k0)
         I.run(9)
         check(I, st, 9)
+
+
+def test_captured_row_by_row_batch_goes_on_with_every_replay():
+    """A member that could run in the column form, in a batch that runs row by row: reset, then a captured
+    run of the batch, replayed."""
+    torch = pytest.importorskip("torch")
+    prob, np_ = W.knapsack(2603, 5), 90
+    stream = torch.cuda.Stream()
+    with Q.Instance(prob, np_, seed=5, stream=stream.cuda_stream) as I, \
+            Q.Instance(prob, np_, seed=6, stream=stream.cuda_stream, flags=Q.QIEO_FLAG_PER_GENERATION) as J:
+        with Q.Batch([I, J]) as b:
+            b.run(3)
+            I.reset()
+            J.reset()
+            I.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                b.run(6)
+            for _ in range(4):
+                graph.replay()
+            torch.cuda.synchronize()
+            for X, seed in ((I, 5), (J, 6)):
+                st = O.run(prob, np_, 24, seed=seed)
+                k, t = X.state()
+                assert t == 24 and np.array_equal(k, st.k)
+                assert np.array_equal(X.best()[0], st.best_x) and np.array_equal(X.fitness(), st.f)
+        I.run(30)                # a run of its own goes on from there
+        I.reset()
+        I.run(30)
+        check(I, O.run(prob, np_, 30, seed=5), 30)
