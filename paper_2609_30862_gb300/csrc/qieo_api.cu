@@ -3253,7 +3253,14 @@ struct StepRecord {
 // Solves admitted between two looks at the steps: an admission takes the host about 50 us, and the GPU
 // starts on the first ones meanwhile.
 constexpr size_t kAdmitAtOnce = 16;
-constexpr size_t kWorkListBytes = 16u << 20;   // per region: params, segments, block starts
+
+// Per region: members (or params), tasks (or segments), block starts. As many small solves as fitted 16 MB
+// row by row (a member's params, one segment and its count each: 35,246) fit in the column form,
+// whose members are larger and have a task for each of its three launches.
+constexpr size_t kWorkListBytes = 22u << 20;
+static_assert(kWorkListBytes / (sizeof(qieo::ColMember) + 3 * sizeof(qieo::ColTask)) >
+                  ((size_t)16 << 20) / (sizeof(qieo::GenParams) + sizeof(qieo::BatchSeg) + sizeof(int32_t)),
+              "a work list holds fewer solves than its row-by-row form did");
 
 }  // namespace
 
