@@ -843,6 +843,7 @@ qieo_status configure_column(qieo_instance *q)
     c.rest = c.slot + 4;
     c.ctl = reinterpret_cast<int32_t *>(words + 256);
     c.sync = reinterpret_cast<qieo::ColSync *>(words + 384);
+    c.run_best = reinterpret_cast<int64_t *>(words + 448);
     c.post = reinterpret_cast<qieo::ColSync *>(words + 512);
     c.qctr = reinterpret_cast<unsigned int *>(words + 512 + 2 * qieo::kColPosted * sizeof(qieo::ColSync));
     return QIEO_OK;
@@ -1086,44 +1087,70 @@ qieo_status ensure_column(qieo_instance *q)
 }
 
 typedef void (*ColumnObserveFn)(qieo::GenParams, qieo::ColParams, int32_t, int32_t);
-ColumnObserveFn column_observe_fn(int form)
+ColumnObserveFn column_observe_fn(int form, bool next)
 {
-    return form == 0 ? &qieo::column_observe_kernel<0>
-                     : form == 1 ? &qieo::column_observe_kernel<1> : &qieo::column_observe_kernel<2>;
+    if (next)
+        return form == 0 ? &qieo::column_observe_kernel<0, true>
+                         : form == 1 ? &qieo::column_observe_kernel<1, true> : &qieo::column_observe_kernel<2, true>;
+    return form == 0 ? &qieo::column_observe_kernel<0, false>
+                     : form == 1 ? &qieo::column_observe_kernel<1, false> : &qieo::column_observe_kernel<2, false>;
 }
 
-// One generation of a row block: a block takes a tile and as many rows as make one wave of two
-// blocks per SM.
-cudaError_t launch_column_observe(qieo_instance *q, int32_t t)
+// Blocks of column_observe for about `want` of them: each takes a tile and part_rows rows.
+int64_t observe_blocks(const qieo_instance *q, int64_t want, int64_t &part_rows)
 {
     const int64_t ntile = plane_tiles(q), rpp = ntile > 1 ? 1 : qieo::kThreads / pow2_ceil(q->svec);
-    const int64_t nu = (q->np + rpp - 1) / rpp, parts = std::max<int64_t>(1, std::min(nu, 2 * (int64_t)q->sm_count / ntile));
-    const int64_t part_rows = (nu + parts - 1) / parts * rpp;
-    const int64_t blocks = ntile * ((q->np + part_rows - 1) / part_rows);
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = launch_config(q, dim3((unsigned)blocks), 0, attr);
-    return cudaLaunchKernelEx(&cfg, column_observe_fn(q->col_form), q->gp, q->cp, t, (int32_t)part_rows);
+    const int64_t nu = (q->np + rpp - 1) / rpp, parts = std::max<int64_t>(1, std::min(nu, want / ntile));
+    part_rows = (nu + parts - 1) / parts * rpp;
+    return ntile * ((q->np + part_rows - 1) / part_rows);
 }
 
-// Runs of so few generations of at most so many genes are two plain launches a generation that draw
-// every gene, fixed or not: a pair takes 7 us for a small population (64 x 100; 19 us for 1,024 x
-// 10,000), the cooperative launches, the plane and the end of a run 15 us and 1 to 2 a generation (37
-// and 10). At 2^24 genes the draws of a generation take 8 us.
-constexpr int32_t kStepRun = 3;
-constexpr int64_t kStepGenes = (int64_t)1 << 24;
+// One generation of a row block, or one of an instance's run (t = -1 - g): one wave of two blocks per SM.
+cudaError_t launch_column_observe(qieo_instance *q, int32_t t)
+{
+    int64_t part_rows = 0;
+    const int64_t blocks = observe_blocks(q, 2 * (int64_t)q->sm_count, part_rows);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = launch_config(q, dim3((unsigned)blocks), 0, attr);
+    return cudaLaunchKernelEx(&cfg, column_observe_fn(q->col_form, t < -1), q->gp, q->cp, t, (int32_t)part_rows);
+}
+
+// Short runs are plain launches that draw every gene, fixed or not: one a generation, each of which
+// takes the CIP of the one before, and one that ends the run, 4 us each for a small population.
+// The cooperative launches, the plane (which draws the last generation again) and the end take
+// 16 us and 2 to 3 a generation, but drop the genes that are fixed. Measured, us a run of 1, 2, 3 and
+// 4 generations, plain | cooperative (every gene drawn; nearly every gene fixed):
+//   64 x 100          9, 13, 17, 21 | 16, 18, 21, 24; 12, 13, 14, 14
+//   1,024 x 10,000    19, 36, 50, 61 | 38, 51, 57, 67; 20, 20, 19, 20
+//   3,000 x 30,000    89, 189, 302, 378 | 135, 218, 303, 377; 20, 20, 21, 22
+// A gene needs K steps from pi/4 to a bound, and takes about three times as many in a solve. So: up to
+// four generations while none can be fixed, and while few are where launches are most of the time
+// (2^20 genes); later on one, or two of a small population. Two shapes for which the cooperative form
+// is slow: a few rows of very many genes, which take the CIP for every tile and turn (2 x 1,000,003,
+// 12 generations: 120 | 155), and a million rows of a few genes, whose fitness one block fills once
+// every gene is fixed (1,000,000 x 8, 4 generations: 111 | 393, 130).
+bool step_run(const qieo_instance *q, int32_t G)
+{
+    const int64_t genes = (int64_t)q->np * q->svec * 8, end = (int64_t)q->t + G;
+    if (q->gp.converge && G > 2) return false;   // (two launches a generation)
+    if (end <= q->K) return G <= 4 || (q->np <= 4 && q->svec >= 1 << 16);
+    if (G <= 2) return genes <= (G == 1 || end <= 3 * (int64_t)q->K ? (int64_t)1 << 24 : (int64_t)1 << 20);
+    return G <= 4 && ((q->np >= 1 << 18 && q->svec <= 4) || (end <= 3 * (int64_t)q->K && genes <= (int64_t)1 << 20));
+}
 
 // A run in the column form: one cooperative launch, the allele plane, the state between runs.
 qieo_status run_column(qieo_instance *q, int32_t G)
 {
-    if (G <= kStepRun && (int64_t)q->np * q->svec * 8 <= kStepGenes &&
-        !(q->flags & (QIEO_FLAG_TIME_KERNELS | QIEO_FLAG_TIME_GENERATIONS))) {
+    if (step_run(q, G) && !(q->flags & (QIEO_FLAG_TIME_KERNELS | QIEO_FLAG_TIME_GENERATIONS))) {
         qieo_status st = ensure_column(q);
         if (st != QIEO_OK) return st;
+        const bool each = q->gp.converge != 0;     // (the stop is decided by column_step_kernel)
         for (int32_t g = 0; g < G; ++g) {
-            CUDA_TRY(launch_column_observe(q, -1));
+            CUDA_TRY(launch_column_observe(q, each ? -1 : -1 - g));
+            if (!each && g + 1 < G) continue;
             cudaLaunchAttribute attr[1];
             cudaLaunchConfig_t cfg = launch_config(q, dim3(plane_tiles(q)), 0, attr);
-            CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_step_kernel, q->gp, q->cp));
+            CUDA_TRY(cudaLaunchKernelEx(&cfg, qieo::column_step_kernel, q->gp, q->cp, each ? 0 : g));
         }
         q->state_valid = false;
         return QIEO_OK;

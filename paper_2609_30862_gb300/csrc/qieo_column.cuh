@@ -76,6 +76,7 @@ struct ColParams {
     ColSlot *head;                // the list at the start of a run (in list 0)
     ColSlot *rest;                // the list and the dropped quads' sums at the hand-over
     int32_t *ctl;                 // [16]
+    int64_t *run_best;            // [2] runs of column_observe_kernel: best fitness before generation t in t & 1
     uint32_t one;                 // 1 (see mad_add)
     int32_t sum_bits;             // kForm 1: a row's weights, its values and its tiles' count share a word of
                                   // acc, the sums in this many bits each (0: a word each and cnt)
@@ -934,7 +935,7 @@ __device__ __forceinline__ bool column_stopped(const GenParams &p, const ColPara
 // another block may set the word meanwhile). The words of such a run are not those of any
 // generation, so nothing runs on them until a reset: column_begin has left kCtlRan 0, and the
 // launches that follow change neither the records nor the generation counter.
-__device__ __forceinline__ bool column_failed(const GenParams &p) { return ld_acquire(p.error) != 0; }
+__device__ __forceinline__ bool column_failed(const GenParams &p) { return __ldcg(p.error) != 0; }
 
 __device__ __forceinline__ void column_begin(const GenParams &p, const ColParams &c, int32_t t0, bool draws)
 {
@@ -1648,47 +1649,85 @@ __global__ void __launch_bounds__(kThreads) column_expand_kernel(const GenParams
         p.state[i] = __ldg(row + i % (size_t)p.svec);
 }
 
-// One generation of a row block from equal rows (a population sharded by rows, whose elite is picked
-// outside): the block's alleles, fitness and best key. A block keeps one tile's thresholds and items
-// for its rows, as in a run; the angle indices stay as they are until column_rotate_kernel.
-// t < 0: generation *p.gen of an instance, which column_step_kernel closes.
+template <int kForm>
+struct ColObserveShared {
+    uint32_t thr[kMaxThr];
+    unsigned long long acc64[kForm == 2 ? 2 * kColRows : 1];
+    uint32_t acc32[kForm == 2 ? 1 : 2 * kColRows];
+    int32_t row[kColRows];
+    int64_t fix[2];
+};
+
+// Before column_observe, whose first barrier follows.
+template <int kForm>
+__device__ __forceinline__ void column_observe_begin(const GenParams &p, ColObserveShared<kForm> &sh)
+{
+    load_thresholds(p, sh.thr);
+    for (int i = threadIdx.x; i < 2 * kColRows; i += kThreads) {
+        if constexpr (kForm == 2) sh.acc64[i] = 0ull;
+        else sh.acc32[i] = 0u;
+    }
+    if (threadIdx.x < 2) sh.fix[threadIdx.x] = 0;
+}
+
+// One generation from equal rows: the alleles, fitness and best key of np rows. A block keeps one
+// tile's thresholds and items for its rows, as in a run.
+//   t >= 0: generation t of a row block (a population sharded by rows, whose elite is picked outside);
+//     the angle indices stay as they are until column_rotate_kernel.
+//   t = -1 - g: generation g of an instance's run, which column_step_kernel ends. From the second on
+//     (kNext) the block first takes the generation before's CIP, toward the elite of its key: the
+//     leading blocks leave the angle indices in their parity and the best row, block 0 the records.
 // Bound by the integer pipes and, with 50 rows a block, by its start: 1,500 rows of 20,000 genes
 // 30 us, 38 us row by row with the state read (and the rotation 2.5 us, 15 us row by row).
-template <int kForm>
-__global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenParams p, const ColParams c, int32_t t,
-                                                                     int32_t part_rows)
+template <int kForm, bool kNext>
+__device__ __forceinline__ void column_observe(const GenParams &p, const ColParams &c, int32_t t, int32_t part_rows,
+                                               int block, int blocks, ColObserveShared<kForm> &sh)
 {
-    __shared__ uint32_t s_thr[kMaxThr];
-    __shared__ unsigned long long s_acc64[kForm == 2 ? 2 * kColRows : 1];
-    __shared__ uint32_t s_acc32[kForm == 2 ? 1 : 2 * kColRows];
-    __shared__ int32_t s_row[kColRows];
-    __shared__ int64_t s_fix[2];
     const int tid = threadIdx.x;
-    load_thresholds(p, s_thr);
-    for (int i = tid; i < 2 * kColRows; i += kThreads) {
-        if constexpr (kForm == 2) s_acc64[i] = 0ull;
-        else s_acc32[i] = 0u;
-    }
-    if (tid < 2) s_fix[tid] = 0;
-    grid_dependency_wait();
     __syncthreads();
-    const bool step = t < 0;
+    const bool step = t < 0, rec = block == 0 && tid == 0;
+    const int32_t g = kNext ? -1 - t : 0;
+    unsigned long long last = 0ull;               // the key and the best fitness before generation t - 1
+    int64_t best = 0;
     if (step) {
-        if (column_stopped(p, c, (int)blockIdx.x)) return;
-        if (*p.error != 0) {                      // (no launch before this one is still running)
-            if (blockIdx.x == 0 && tid == 0) c.ctl[kCtlRan] = 0;
+        if (column_stopped(p, c, block)) return;
+        // (every word that may be needed is asked for at once: one trip to L2)
+        const int32_t failed = *p.error, t0 = *p.gen;
+        unsigned long long k0 = 0ull, k1 = 0ull, k2 = 0ull;
+        int64_t b0 = 0, b1 = 0;
+        if (kNext) {
+            k0 = p.keys[0];
+            k1 = p.keys[1];
+            k2 = p.keys[2];
+            b0 = c.run_best[0];
+            b1 = c.run_best[1];
+        } else if (rec) {
+            b0 = p.best[0];
+            b1 = p.best[1];
+        }
+        if (failed) {                             // (no launch before this one is still running)
+            if (rec) c.ctl[kCtlRan] = 0;
             return;
         }
-        t = *p.gen;
-        // (no block of this launch reads the list's counts; column_step_kernel fills them again)
-        if (blockIdx.x == 0 && tid == 0) {
-            c.ctl[kCtlRan] = 1;
-            *c.head = ColSlot{};
+        t = t0 + g;
+        if (kNext) {
+            const int32_t slot = (t + 2) % 3;
+            last = slot == 0 ? k0 : slot == 1 ? k1 : k2;
+            best = (t & 1) ? b0 : b1;
+        }
+        if (rec) {
+            p.keys[(t + 1) % 3] = 0ull;           // (generation t - 2's, which nobody reads any more)
+            if (!kNext) {
+                // (no block of this launch reads the list's counts; column_step_kernel fills them again)
+                c.ctl[kCtlRan] = 1;
+                *c.head = ColSlot{};
+                c.run_best[t & 1] = b1 < 0 ? INT64_MIN : b0;
+            }
         }
     }
-    const ColGeom m = column_geometry((uint32_t)p.svec, 0u, p.np, (int)gridDim.x);
+    const ColGeom m = column_geometry((uint32_t)p.svec, 0u, p.np, blocks);
     const BlockShare b = tile_geometry(m.lanes, m.warps);
-    const int tile = (int)blockIdx.x % m.ntile, part = (int)blockIdx.x / m.ntile;
+    const int tile = block % m.ntile, part = block / m.ntile;
     const int r_end = (int)min((int64_t)p.np, (int64_t)(part + 1) * part_rows);
     const int vec = tile * m.width + b.v_in;
     const bool active = b.v_in < m.width && vec < p.svec;
@@ -1696,17 +1735,37 @@ __global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenPa
     it.qa = active ? 2 * vec : -1;
     it.qb = active ? 2 * vec + 1 : -1;
     it.whole = true;
-    column_load<kForm>(p, it, c.canon);
+    column_load<kForm>(p, it, g < 2 ? c.canon : column_parity(c, p.svec, t - 1));
+    const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(sh.thr);
+    const uint32_t off_top = (uint32_t)(8 * p.K);
     uint32_t T[8], top = 0u;
     ColSum<kForm> base;
-    column_thresholds<kForm>(it, reinterpret_cast<const unsigned char *>(s_thr), (uint32_t)(8 * p.K), T, top, base);
+    column_thresholds<kForm>(it, thr_bytes, off_top, T, top, base);
+    if (kNext) {
+        const int32_t e0 = (int32_t)(0xffffffu - (uint32_t)(last & 0xffffffull)), e = e0 >= 0 && e0 < p.np ? e0 : 0;
+        const int64_t f = (int64_t)(last >> 24) - kKeyBias;
+        const bool improved = f > best;
+        const uint32_t x = column_cip<kForm>(p, it, e, t, T, top, off_top * 0x00010001u);
+        column_thresholds<kForm>(it, thr_bytes, off_top, T, top, base);
+        if (part == 0 && b.r_sub == 0 && active) {
+            uint2 *row = column_parity(c, p.svec, t);
+            row[it.qa] = it.sa;
+            row[it.qb] = it.sb;
+            if (improved) p.best_row[vec] = (uint8_t)x;
+        }
+        if (rec) {
+            c.run_best[t & 1] = improved ? f : best;
+            if (e != e0) atomicOr(p.error, kErrEliteRange);
+            column_record(p, t - 1, e, f, improved, 0, (uint32_t)p.svec);
+        }
+    }
     const RowKeys k = row_keys(p, (uint32_t)t);
     const QuadWords wa = quad_words(p, (uint32_t)it.qa, (uint32_t)t), wb = quad_words(p, (uint32_t)it.qb, (uint32_t)t);
     uint8_t *const plane = p.xbits + (size_t)(t & 1) * p.xplane + vec;
     unsigned long long *const key = p.keys + t % 3;
     for (int ra = part * part_rows; ra < r_end; ra += kColRows) {
         const int n = min(kColRows, r_end - ra);
-        if (tid < n) s_row[tid] = ra + tid;
+        if (tid < n) sh.row[tid] = ra + tid;
 #pragma unroll 2
         for (int q = b.r_sub; q < n + b.r_sub; q += m.rpp) {         // the same trips for every thread
             const uint64_t z = row_product(k, (uint32_t)(p.row0 + ra + q));
@@ -1734,43 +1793,51 @@ __global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenPa
                     }
                 }
             }
-            if (b.leader && q < n) column_add<kForm>(s, q, s_acc32, s_acc64);
+            if (b.leader && q < n) column_add<kForm>(s, q, sh.acc32, sh.acc64);
         }
-        column_flush<kForm>(p, c.sum_bits, m.ntile, s_row, n, s_fix, key, s_acc32, s_acc64);
+        column_flush<kForm>(p, c.sum_bits, m.ntile, sh.row, n, sh.fix, key, sh.acc32, sh.acc64);
     }
     // the generation counter then names the next generation, as after a run
-    if (!step && blockIdx.x == 0 && tid == 0) *p.gen = t + 1;
+    if (!step && rec) *p.gen = t + 1;
+}
+
+template <int kForm, bool kNext>
+__global__ void __launch_bounds__(kThreads, 2) column_observe_kernel(const GenParams p, const ColParams c, int32_t t,
+                                                                     int32_t part_rows)
+{
+    __shared__ ColObserveShared<kForm> sh;
+    column_observe_begin(p, sh);
+    grid_dependency_wait();
+    column_observe<kForm, kNext>(p, c, t, part_rows, (int)blockIdx.x, (int)gridDim.x, sh);
     allow_dependent_launch();
 }
 
-// Closes a generation that column_observe_kernel drew for an instance: the elite from its key, CIP
+// Ends a run of column_observe_kernel's generations, of which g is the last: its elite from its key, CIP
 // of the one row, the best row if it improved, the list the next run starts with, and by the
-// last block the records. Runs of a few generations are these two launches each (see kStepRun): 64
-// rows of 100 genes, one generation: 7.8 us from call to call; 15.4 with the cooperative kernel, the
-// plane and the end, 9.4 in the resident form.
-__global__ void __launch_bounds__(kThreads) column_step_kernel(const GenParams p, const ColParams c)
+// last block the records. (When a run is worth these launches: see step_run.)
+__device__ __forceinline__ void column_step(const GenParams &p, const ColParams &c, int32_t g, int block, int blocks,
+                                            const uint32_t *s_thr)
 {
-    __shared__ uint32_t s_thr[kMaxThr];
     __shared__ int s_last;
-    load_thresholds(p, s_thr);
-    grid_dependency_wait();
-    __syncthreads();
-    if (c.ctl[kCtlRan] == 0) return;              // (stopped by convergence)
     const unsigned char *thr_bytes = reinterpret_cast<const unsigned char *>(s_thr);
     const uint32_t off_top = (uint32_t)(8 * p.K), k8 = off_top * 0x00010001u;
-    const int32_t t = *p.gen;
-    const unsigned long long key = p.keys[t % 3];
+    // (every word that may be needed is asked for at once: one trip to L2)
+    const int32_t ran = c.ctl[kCtlRan], t = *p.gen + g, slot = t % 3;
+    const unsigned long long k0 = p.keys[0], k1 = p.keys[1], k2 = p.keys[2], key = slot == 0 ? k0 : slot == 1 ? k1 : k2;
+    const int64_t best_f = p.best[0], best_t = p.best[1];
+    if (ran == 0) return;                         // (stopped by convergence)
+    const uint2 *state = g == 0 ? c.canon : column_parity(c, p.svec, t);
     const int32_t e0 = (int32_t)(0xffffffu - (uint32_t)(key & 0xffffffull)), e = e0 >= 0 && e0 < p.np ? e0 : 0;
     const int64_t f = (int64_t)(key >> 24) - kKeyBias;
-    const bool improved = p.best[1] < 0 || f > p.best[0];
-    const int vec = blockIdx.x * kThreads + threadIdx.x;
+    const bool improved = best_t < 0 || f > best_f;
+    const int vec = block * kThreads + threadIdx.x;
     const bool act = vec < p.svec;
     uint2 s[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
     uint32_t bits = 0u;
     if (act) {
         for (int h = 0; h < 2; ++h) {
             const int q = 2 * vec + h;
-            const uint2 o = c.canon[q];
+            const uint2 o = state[q];
             const Draw4 d = philox4x32_10_rk((uint32_t)q, (uint32_t)e, (uint32_t)t, 0u, p.rk0, p.rk1);
             const uint32_t x = observe_quad(d, o, thr_bytes, off_top);
             s[h] = step_quad(o, x, k8);
@@ -1785,7 +1852,7 @@ __global__ void __launch_bounds__(kThreads) column_step_kernel(const GenParams p
     if (act && fb) quad_sums(p, 2 * vec + 1, s[1], fw, fv);
     column_append(c.head, column_list(c, p.svec, 0), p.svec, act, true, 2 * vec, 2 * vec + 1, fa, fb, fw, fv);
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atom_add_acq_rel(reinterpret_cast<unsigned int *>(c.ctl + kCtlTicket), 1u) == gridDim.x - 1u ? 1 : 0;
+    if (threadIdx.x == 0) s_last = atom_add_acq_rel(reinterpret_cast<unsigned int *>(c.ctl + kCtlTicket), 1u) == (unsigned int)blocks - 1u ? 1 : 0;
     __syncthreads();
     if (!s_last || threadIdx.x != 0) return;
     c.ctl[kCtlTicket] = 0;
@@ -1803,6 +1870,15 @@ __global__ void __launch_bounds__(kThreads) column_step_kernel(const GenParams p
     *p.gen = t + 1;
     *p.bar_gen = t + 1;
     p.keys[0] = p.keys[1] = p.keys[2] = 0ull;
+}
+
+__global__ void __launch_bounds__(kThreads) column_step_kernel(const GenParams p, const ColParams c, int32_t g)
+{
+    __shared__ uint32_t s_thr[kMaxThr];
+    load_thresholds(p, s_thr);
+    grid_dependency_wait();
+    __syncthreads();
+    column_step(p, c, g, (int)blockIdx.x, (int)gridDim.x, s_thr);
 }
 
 // CIP of a row block with equal rows toward an elite row supplied from outside: bytes of 0 or 1,
