@@ -1913,7 +1913,7 @@ struct ColMember {
 struct ColTask {
     int32_t member;
     int32_t block, blocks;        // of the member's blocks
-    int32_t gens;                 // most generations of this run
+    int32_t gens;                 // most generations of this run (column_batch_observe_kernel: rows a block)
 };
 
 // A member's words in shared memory (whole block).
@@ -1939,6 +1939,31 @@ __global__ void __launch_bounds__(kThreads, 2) column_batch_kernel(const ColMemb
         load_member(s_m, members + k.member);
         column_run<kForm, true>(s_m.p, s_m.c, min(G, k.gens), k.block, k.blocks, sh);
     }
+}
+
+// A run of one generation, task by task: column_observe and column_step (see qieo_batch_run for when).
+template <int kForm>
+__global__ void __launch_bounds__(kThreads, 2) column_batch_observe_kernel(const ColMember *members, const ColTask *tasks)
+{
+    __shared__ ColMember s_m;
+    __shared__ ColObserveShared<kForm> sh;
+    grid_dependency_wait();
+    const ColTask k = tasks[blockIdx.x];
+    load_member(s_m, members + k.member);
+    column_observe_begin(s_m.p, sh);
+    column_observe<kForm, false>(s_m.p, s_m.c, -1, k.gens, k.block, k.blocks, sh);
+}
+
+__global__ void __launch_bounds__(kThreads) column_batch_step_kernel(const ColMember *members, const ColTask *tasks)
+{
+    __shared__ ColMember s_m;
+    __shared__ uint32_t s_thr[kMaxThr];
+    grid_dependency_wait();
+    const ColTask k = tasks[blockIdx.x];
+    load_member(s_m, members + k.member);
+    load_thresholds(s_m.p, s_thr);
+    __syncthreads();
+    column_step(s_m.p, s_m.c, 0, k.block, k.blocks, s_thr);
 }
 
 // column_plane_kernel and column_end_kernel for every member, task by task. (A plane task of no blocks

@@ -499,3 +499,33 @@ def test_short_runs(ng, np_, D, items, chunks):
                 I.run(g)
             check(I, st, gens)
             I.reset()
+
+
+@pytest.mark.parametrize("items,D,chunks", [("byte", 100, [1] * 12 + [5] + [1] * 3), ("mid", 12, [1] * 14), ("wide", 8, [2, 1, 1, 3, 1])])
+def test_batched_runs_of_one_generation(items, D, chunks):
+    """Runs of one generation of a batch (two plain launches), through 3 K generations, from which on they are
+    cooperative; a member of rule R2 and one that stops by convergence among them."""
+    specs = [(1, 1), (40, 30), (2049, 33), (4100, 90), (300, 257)]
+    insts = [Q.Instance(_problem(ng, items), np_, seed=ng, D=D) for ng, np_ in specs]
+    insts.append(Q.Instance(_problem(700, items), 40, seed=7, D=D, rule=1))
+    conv = W.knapsack(60, 21)
+    insts.append(Q.Instance(conv, 17, seed=21, flags=Q.QIEO_FLAG_CONVERGE))
+    gens = sum(chunks)
+    with Q.Batch(insts) as b:
+        for solve in range(2):
+            for g in chunks:
+                b.run(g)
+            for I, (ng, np_) in zip(insts, specs):
+                check(I, O.run(_problem(ng, items), np_, gens, seed=ng, D=D), gens)
+            check(insts[5], O.run(_problem(700, items), 40, gens, seed=7, D=D, rule=1), gens)
+            check(insts[6], O.run(conv, 17, gens, seed=21), gens)
+            for I in insts:
+                I.reset()
+        ref = O.run(conv, 17, 600, seed=21, window=20)
+        n = int(ref.t[0])
+        for _ in range(n + 5):
+            b.run(1)
+        k, t = insts[6].state()
+        assert ref.stopped and t == n and np.array_equal(k, ref.k) and insts[6].convergence() == (True, 20)
+    for I in insts:
+        I.close()
