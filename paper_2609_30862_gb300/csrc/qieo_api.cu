@@ -886,7 +886,6 @@ qieo_status ensure_history(qieo_instance *q, int32_t need)
     q->gp.hist_e = e;
     q->gp.hist_f = f;
     q->gp.hist_d = d;
-    q->gp.hist_cap_d = (size_t)cap;
     drop_graphs(q);
     return QIEO_OK;
 }
@@ -1742,14 +1741,15 @@ qieo_status qieo_reset(qieo_instance *q)
     const size_t words = (size_t)q->np * q->svec * (q->state8 ? 2 : 4);
     const size_t xbytes = 2 * (size_t)q->np * q->xstride;
     const int blocks = std::max(1, std::min(q->sm_count * 4, (int)std::min<size_t>((words + 255) / 256, 1 << 20)));
+    const size_t hist_words = q->hist_d ? (size_t)q->hist_cap : 0;
     q->rows_equal = true;
     if (q->col_mem && column_capable(q)) {
         qieo::column_reset_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, q->cp, q->keep_state ? words : 0, xbytes,
-                                                                           (size_t)q->np * 2);
+                                                                           (size_t)q->np * 2, hist_words);
         q->col_valid = true;
         q->state_valid = q->keep_state;
     } else {
-        qieo::init_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, words, xbytes, (size_t)q->np * 2);
+        qieo::init_kernel<<<blocks, qieo::kThreads, 0, q->stream>>>(q->gp, words, xbytes, (size_t)q->np * 2, hist_words);
         q->col_valid = false;
         q->state_valid = true;
     }

@@ -1603,10 +1603,10 @@ __global__ void __launch_bounds__(kThreads) column_end_kernel(const GenParams p,
 // at pi/4, every vector on the list, no recorded best row. The full state is written if state_words
 // is not 0 (column_expand_kernel makes it otherwise, when another form needs it).
 __global__ void __launch_bounds__(kThreads) column_reset_kernel(const GenParams p, const ColParams c, size_t state_words,
-                                                                size_t xbytes, size_t acc_words)
+                                                                size_t xbytes, size_t acc_words, size_t hist_words)
 {
     grid_dependency_wait();
-    init_words(p, state_words, xbytes, acc_words);
+    init_words(p, state_words, xbytes, acc_words, hist_words);
     const uint32_t kk = (uint32_t)(4 * p.K) * 0x00010001u;
     const int i0 = blockIdx.x * kThreads + threadIdx.x, stride = (int)gridDim.x * kThreads;
     for (int vec = i0; vec < p.svec; vec += stride) {

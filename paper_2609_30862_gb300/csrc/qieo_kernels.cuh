@@ -163,7 +163,6 @@ struct GenParams {
     unsigned long long *hist_d;   // [capacity] vectors that did not draw, per generation
                                   // (copied from fcnt once the generation is complete), or
                                   // NULL
-    size_t hist_cap_d;            // entries of hist_d (0: NULL)
     unsigned long long *fprev;    // [np] packed row totals (SV << 26 | SW) of the last
                                   // generation, kept by the kernel that keeps F
     const uint32_t *ftile;        // [2 ntile] sums of the weights and of the values of each
@@ -2780,7 +2779,8 @@ __global__ void __launch_bounds__(kThreads) gather_stop_kernel(int32_t *const *c
 
 // Generation 0 state: every qubit at theta = pi/4 (n = K), no elite, no best record.
 // state_words = 0 leaves the full state and the fixed-vector words as they are.
-__device__ __forceinline__ void init_words(const GenParams &p, size_t state_words, size_t xbytes, size_t acc_words)
+__device__ __forceinline__ void init_words(const GenParams &p, size_t state_words, size_t xbytes, size_t acc_words,
+                                           size_t hist_words)
 {
     const uint32_t kk = (uint32_t)(4 * p.K) * (p.state8 ? 0x01010101u : 0x00010001u);
     uint32_t *s = reinterpret_cast<uint32_t *>(p.state);
@@ -2805,7 +2805,7 @@ __device__ __forceinline__ void init_words(const GenParams &p, size_t state_word
         if (i0 == 0)
             for (int i = 0; i < 7; ++i) p.fcnt[i] = 0ull;
     }
-    for (size_t i = i0; i < p.hist_cap_d; i += stride) p.hist_d[i] = 0ull;
+    for (size_t i = i0; i < hist_words; i += stride) p.hist_d[i] = 0ull;
     if (i0 == 0) {
         *p.gen = 0;
         *p.ticket = 0u;
@@ -2823,11 +2823,11 @@ __device__ __forceinline__ void init_words(const GenParams &p, size_t state_word
     }
 }
 
-__global__ void __launch_bounds__(kThreads) init_kernel(GenParams p, size_t state_words,
-                                                        size_t xbytes, size_t acc_words)
+__global__ void __launch_bounds__(kThreads) init_kernel(GenParams p, size_t state_words, size_t xbytes,
+                                                        size_t acc_words, size_t hist_words)
 {
     grid_dependency_wait();
-    init_words(p, state_words, xbytes, acc_words);
+    init_words(p, state_words, xbytes, acc_words, hist_words);
 }
 
 __global__ void philox_kernel(const uint32_t *ck, uint32_t *out, int32_t n)
