@@ -2927,8 +2927,10 @@ qieo_status build_col_group(qieo_batch *bt, qieo_batch::ColGroup &g)
     const size_t total = column_batch_layout(g.plan, 0, off, src, bytes);
     CUDA_TRY(cudaMalloc(&g.dev, total));
     place_column_batch(g.plan, (const char *)g.dev, off);
+    std::vector<char> stage(total);      // (one copy: each from pageable memory is a wait of its own)
     for (int i = 0; i < kColumnBatchParts; ++i)
-        CUDA_TRY(cudaMemcpyAsync((char *)g.dev + off[i], src[i], bytes[i], cudaMemcpyHostToDevice, bt->stream));
+        if (bytes[i]) std::memcpy(stage.data() + off[i], src[i], bytes[i]);
+    CUDA_TRY(cudaMemcpyAsync(g.dev, stage.data(), total, cudaMemcpyHostToDevice, bt->stream));
     return wait_stream(bt->stream);
 }
 
