@@ -2479,6 +2479,7 @@ void plan_column_batch(const std::vector<qieo_instance *> &members, const std::v
     const auto gens_of = [&](int i) { return gens.empty() ? INT32_MAX : gens[(size_t)i]; };
     const int n = (int)members.size(), grid = b.grid;
     b.members.clear();
+    b.members.reserve((size_t)n);
     std::vector<double> alone((size_t)n);
     double lo = 0.0, total = 0.0, longest = 0.0;
     for (int i = 0; i < n; ++i) {
@@ -2534,6 +2535,8 @@ void plan_column_batch(const std::vector<qieo_instance *> &members, const std::v
         } else {
             lo = t;
         }
+        // (a smaller time than the mean does not fit: every other round would give the same, one block a member)
+        if (longest <= total / grid) break;
         if (hi - lo < 0.02 * hi) break;
     }
     // the blocks' lists, each in the members' order
@@ -3355,6 +3358,7 @@ struct qieo_server {
     std::unordered_map<int64_t, std::unique_ptr<SolveRequest>> all;
     std::deque<StepRecord> inflight;
     std::vector<cudaEvent_t> spare_events;
+    ColumnBatch plans[3];                // the last step's, by item form (their memory is used again)
     int64_t next_id = 1;
     std::chrono::steady_clock::time_point t0;
     std::thread worker;
@@ -3403,7 +3407,7 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
         qieo::BatchArgs args;
     };
     std::vector<Launch> launches;
-    std::vector<ColumnBatch> columns;             // the solves in the column form, by item form
+    std::vector<ColumnBatch *> columns;           // the solves in the column form, by item form
     for (int form = 0; form < 3; ++form) {
         std::vector<qieo_instance *> grp;
         std::vector<int32_t> gens;
@@ -3413,8 +3417,8 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
                 gens.push_back(remaining[i]);
             }
         if (grp.empty()) continue;
-        columns.emplace_back();
-        ColumnBatch &b = columns.back();
+        ColumnBatch &b = S->plans[form];
+        columns.push_back(&b);
         b.form = form;
         qieo_status st = column_batch_grid(grp[0], b);
         if (st != QIEO_OK) return st;
@@ -3466,8 +3470,8 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
         }
     }
     CUDA_TRY(cudaMemcpyAsync(dev, host, used, cudaMemcpyHostToDevice, S->stream));
-    for (const ColumnBatch &b : columns) {
-        qieo_status st = launch_column_batch(b, G, S->stream);
+    for (const ColumnBatch *b : columns) {
+        qieo_status st = launch_column_batch(*b, G, S->stream);
         if (st != QIEO_OK) return st;
     }
     for (int32_t gen = 0; gen < G; ++gen) {
