@@ -529,3 +529,63 @@ def test_batched_runs_of_one_generation(items, D, chunks):
         assert ref.stopped and t == n and np.array_equal(k, ref.k) and insts[6].convergence() == (True, 20)
     for I in insts:
         I.close()
+
+
+@pytest.mark.parametrize("ng,np_,flags,shape,lam,items", [
+    (5000, 90, 0, None, 1, "byte"), (5000, 90, Q.QIEO_FLAG_FORCE_WIDE, None, 1, "byte"), (5000, 90, 0, (32, 2, 0), 1, "byte"),
+    (5000, 90, 0, (4, 1, 7), 1, "byte"), (5000, 90, 0, (32, 8, 40), 1, "byte"), (5000, 90, 0, (1, 1, 64), 1, "byte"),
+    (5000, 90, Q.QIEO_FLAG_TIME_GENERATIONS, None, 1, "byte"), (900, 70, 0, None, 7, "mid"), (700, 40, 0, None, 1, "wide"),
+    (2100, 12, 0, (1, 1, 0), 1, "byte"), (32800, 12, 0, (1, 1, 0), 1, "byte"),     # 263 and 4,100 tiles of one lane
+    (263000, 4, 0, None, 1, "255"), (263200, 4, 0, None, 1, "255"),                # packed row sums just below and above 2^26
+    (2050, 6000, 0, (32, 8, 2), 1, "byte"),
+])
+def test_rule_r1_row_by_row(ng, np_, flags, shape, lam, items):
+    """Rule R1 from rows that differ, which the column form cannot hold: the resident form, the streamed
+    one and their shapes, as the older tests of these forms had them run before the column form."""
+    prob = W.custom_problem(np.full(ng, 255), np.full(ng, 255), 255 * ng // 2) if items == "255" else _problem(ng, items)
+    k0 = np.random.default_rng(ng).integers(-25, 26, size=(np_, ng)).astype(np.int16)
+    st = O.State(np_, ng)
+    st.k[:] = k0
+    st = O.run(prob, np_, 16, seed=ng, lam=lam, state=st, kind="omp")
+    with Q.Instance(prob, np_, seed=ng, lam=lam, flags=flags) as I:
+        if shape:
+            I.set_shape(*shape)
+        load_state(I, k0)
+        for g in (7, 7, 2):
+            I.run(g)
+        check(I, st, 16)
+
+
+def test_rule_r1_row_by_row_in_a_batch():
+    """The persistent row-by-row form of a batch under rule R1: members whose rows differ; a wait that runs
+    out; then one launch per generation (a member asks for it)."""
+    prob, sizes = W.knapsack(3000, 41), ((120, 3), (90, 4))
+    k0 = [np.random.default_rng(s).integers(-25, 26, size=(n, 3000)).astype(np.int16) for n, s in sizes]
+    refs = []
+    for (n, s), k in zip(sizes, k0):
+        st = O.State(n, 3000)
+        st.k[:] = k
+        refs.append(O.run(prob, n, 12, seed=s, state=st))
+    insts = [Q.Instance(prob, n, seed=s) for n, s in sizes]
+    other = Q.Instance(prob, 20, seed=5, flags=Q.QIEO_FLAG_PER_GENERATION)
+    for members in (insts, insts + [other]):
+        with Q.Batch(members) as b:
+            for I, k in zip(insts, k0):
+                load_state(I, k)
+            if members is insts:
+                insts[0].set_wait_timeout(1)
+                b.run(6)
+                with pytest.raises(Q.QieoError) as e:
+                    insts[0].synchronize()
+                assert e.value.status == Q.QIEO_ERR_TIMEOUT
+                insts[0].set_wait_timeout(10 * 10**9)
+                for I, k in zip(insts, k0):
+                    I.reset()
+                    load_state(I, k)
+            b.run(7)
+            b.run(5)
+            for I, st in zip(insts, refs):
+                check(I, st, 12)
+                I.reset()
+    for I in members:
+        I.close()
