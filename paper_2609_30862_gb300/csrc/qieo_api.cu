@@ -1024,6 +1024,9 @@ qieo_status run_cooperative(qieo_instance *q, int32_t G)
         CUDA_TRY(cudaMallocAsync(&q->gen_ns, (size_t)(G + 1) * sizeof(unsigned long long), q->stream));
         q->gen_ns_cap = G + 1;
     }
+    // (a run that stops by convergence leaves the rest: no time)
+    if (stamps && q->gp.converge)
+        CUDA_TRY(cudaMemsetAsync(q->gen_ns, 0, (size_t)(G + 1) * sizeof(unsigned long long), q->stream));
     for (int32_t done = 0; done < G; done += chunk)
         CUDA_TRY(resident ? launch_resident(q, std::min(chunk, G - done), stamps ? q->gen_ns + done : nullptr)
                           : launch_run(q, std::min(chunk, G - done)));
@@ -1165,6 +1168,9 @@ qieo_status run_column(qieo_instance *q, int32_t G)
         CUDA_TRY(cudaMallocAsync(&q->gen_ns, (size_t)(G + 1) * sizeof(unsigned long long), q->stream));
         q->gen_ns_cap = G + 1;
     }
+    // (a run that stops by convergence leaves the rest: no time)
+    if (stamps && q->gp.converge)
+        CUDA_TRY(cudaMemsetAsync(q->gen_ns, 0, (size_t)(G + 1) * sizeof(unsigned long long), q->stream));
     // the barrier counts G x grid arrivals in 32 bits: longer runs are split
     const int32_t chunk = (int32_t)std::max<int64_t>(1, std::min<int64_t>(G, ((int64_t)1 << 30) / std::max(1, q->col_grid)));
     const int tiles = plane_tiles(q);
@@ -2045,7 +2051,8 @@ qieo_status qieo_get_generation_times(qieo_instance *q, int32_t n, float *ms_out
         std::vector<unsigned long long> ns((size_t)m + 1);
         st = fetch(q, ns.data(), q->gen_ns, ns.size() * sizeof(unsigned long long));
         if (st != QIEO_OK) return st;
-        for (int32_t i = 0; i < m; ++i) ms_out[i] = (float)((double)(ns[(size_t)i + 1] - ns[(size_t)i]) * 1e-6);
+        for (int32_t i = 0; i < m; ++i)
+            ms_out[i] = ns[(size_t)i + 1] > ns[(size_t)i] ? (float)((double)(ns[(size_t)i + 1] - ns[(size_t)i]) * 1e-6) : 0.0f;
     } else {
         for (int32_t i = 0; i < m; ++i)
             CUDA_TRY(cudaEventElapsedTime(ms_out + i, q->gen_ev[(size_t)i], q->gen_ev[(size_t)i + 1]));

@@ -589,3 +589,17 @@ def test_rule_r1_row_by_row_in_a_batch():
                 I.reset()
     for I in members:
         I.close()
+
+
+@pytest.mark.parametrize("np_", [30, 3000])
+def test_generation_times_of_a_run_that_stops(np_):
+    """The generations that a converged run does not execute take no time; nor does a run after it."""
+    prob = W.knapsack(200, 3)
+    with Q.Instance(prob, np_, seed=3, flags=Q.QIEO_FLAG_CONVERGE | Q.QIEO_FLAG_TIME_GENERATIONS) as I:
+        I.run(700)
+        n = I.state()[1]
+        assert n < 690 and I.convergence() == (True, 20)
+        ms = np.asarray(I.generation_times(700))
+        assert len(ms) == 700 and ms[:n].min() > 0 and ms[:n].max() < 10 and not ms[n:].any()
+        I.run(700)
+        assert not np.asarray(I.generation_times(700)).any()
