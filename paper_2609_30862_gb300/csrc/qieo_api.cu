@@ -1579,8 +1579,13 @@ qieo_status create_instance_impl(const qieo_problem *pr, const qieo_params *pa,
         // stream-ordered allocation from the device's pool: no device-wide synchronisation
         // at allocation or release, and a freed block is reused by the next instance
         keep_pool_memory(q->device);
-        const size_t col = column_capable(q) ? column_bytes(q->svec) : 0;
+        size_t col = column_capable(q) ? column_bytes(q->svec) : 0;
         ce = cudaMallocAsync(&q->block, total + col, q->stream);
+        if (ce == cudaErrorMemoryAllocation && col) {   // row by row it may fit
+            cudaGetLastError();
+            col = 0;
+            ce = cudaMallocAsync(&q->block, total, q->stream);
+        }
         if (ce != cudaSuccess)
             return bail(fail(ce == cudaErrorMemoryAllocation ? QIEO_ERR_OOM : QIEO_ERR_CUDA,
                              "device allocation of %zu bytes: %s", total + col, cudaGetErrorString(ce)));
