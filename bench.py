@@ -414,15 +414,20 @@ def run_gpu(a):
     # drawn pass's integer work (a quarter Philox4x32-10 call, CIP, the compare, the allele
     # bit, the item sums); its two ceilings are the measured HBM copy bandwidth and the
     # measured integer ceiling (qieo_measure_integer_ceiling, the same per-gene arithmetic
-    # with nothing streamed), and the bound is the slower of the two.
+    # with nothing streamed), and the bound is the slower of the two. The column form streams
+    # no state and neither rotates nor looks up a qubit: its ceiling is the draws alone (the
+    # measured Philox rate), and what it achieves is counted in draws, not in gene-updates,
+    # where the instance counts them.
     launch_s = run_total_ms / 1e3 / (a.steps * G)
     peaks, peak_src = load_peaks()
     genes_per_launch = np_ * ng
     hbm_peak = float(peaks["hbm_gbs"])
     state_bpg = 2 if a.state_i8 else STATE_BYTES_PER_GENE   # byte state: 1 B read + 1 B written
-    t_hbm = state_bpg * genes_per_launch / (hbm_peak * 1e9)
+    t_hbm = 0.0 if column else state_bpg * genes_per_launch / (hbm_peak * 1e9)
     ceiling = None if a.no_phases else Q.qieo_measure_integer_ceiling(5)
-    int_peak = ceiling.drawn_genes_per_s if ceiling is not None else None
+    int_peak = None
+    if ceiling is not None:
+        int_peak = ceiling.philox_genes_per_s if column else ceiling.drawn_genes_per_s
     t_int = genes_per_launch / int_peak if int_peak else 0.0
     l2_resident = state_bytes < L2_BYTES
     hbm_achieved = state_bpg * genes_per_launch / launch_s / 1e9
@@ -433,16 +438,17 @@ def run_gpu(a):
         achieved = genes_per_launch / launch_s / 1e9
         roof = {"bound": "alu", "achieved": achieved, "peak": int_peak / 1e9,
                 "unit": "Ggene-updates/s", "frac": achieved / (int_peak / 1e9),
-                "peak_source": "measured: qieo_measure_integer_ceiling (the drawn pass's per-gene "
-                               "integer work, state in registers, %d blocks, best of %d)" % (
-                                   ceiling.grid_ctas, ceiling.reps)}
+                "peak_source": "measured: qieo_measure_integer_ceiling (%s, %d blocks, best of %d)" % (
+                    "Philox4x32-10 alone" if column else
+                    "the drawn pass's per-gene integer work, state in registers",
+                    ceiling.grid_ctas, ceiling.reps)}
     roof["frac_hbm_4B_formula"] = hbm_achieved / hbm_peak
     roof["fixed_words"] = bool(shape.fixed_words)
     if column:
         roof["note"] = ("column form: the rows of the population share one row of angle indices (rule R1), so "
                         "no state is streamed, and genes that have reached a bound are not drawn any more "
-                        "(identical results); the 4 B and full-draw per gene-update formula behind frac can "
-                        "exceed 1")
+                        "(identical results); frac_hbm_4B_formula counts bytes that do not move and can "
+                        "exceed 1, and so can frac where the instance does not count its draws")
     elif shape.fixed_words:
         roof["note"] = ("fixed-vector words: generations in which most vectors are fixed skip their "
                         "draws and state traffic exactly (identical results), so the 4 B and full-draw "
@@ -450,7 +456,7 @@ def run_gpu(a):
                         "the roofline of the work each generation needed")
     roof["hbm_peak_gbs"] = hbm_peak
     if int_peak:
-        roof["int_ceiling_gene_updates_per_s"] = int_peak
+        roof["int_ceiling_gene_updates_per_s"] = ceiling.drawn_genes_per_s
         roof["philox_only_gene_updates_per_s"] = ceiling.philox_genes_per_s
         roof["t_hbm_us"] = t_hbm * 1e6
         roof["t_int_us"] = t_int * 1e6
@@ -473,6 +479,11 @@ def run_gpu(a):
     if not a.no_phases and (column or shape.resident or not shape.persistent):
         roof["phases"] = generation_phases(Q, prob, c, np_, G, rank, flags, stream, torch,
                                            hbm_peak, int_peak)
+        drew = roof["phases"].get("work_adjusted")
+        if column and drew and roof["bound"] == "alu":
+            roof["achieved"] *= drew["drawn_fraction"]
+            roof["unit"] = "G genes drawn/s"
+            roof["frac"] = roof["achieved"] / roof["peak"]
 
     # end to end through the C ABI with host buffers: create (uploads the items), run,
     # read the best record back, destroy -- every step
@@ -575,8 +586,8 @@ def generation_phases(Q, prob, c, np_, G, rank, flags, stream, torch, hbm_peak, 
     out = {"spread": window(*SPREAD_WINDOW), "saturated": window(*SATURATED_WINDOW),
            "per_25": [round(1e3 * float(np.mean(ms[i:i + step])), 2) for i in range(0, len(ms), step)],
            "sum_of_launches_us": 1e3 * float(np.sum(ms)),
-           "what": "device clock at each generation's start (resident form) or CUDA events before "
-                   "every generation launch of one run (launches serialised)"}
+           "what": "device clock at each generation's start (column and resident forms) or CUDA events "
+                   "before every generation launch of one run (launches serialised)"}
     if drawn is not None and int_peak:
         column = not flags & (Q.QIEO_FLAG_STATE_I8 | Q.QIEO_FLAG_STREAMED | Q.QIEO_FLAG_NO_FIXED_WORDS)
         out["work_adjusted"] = work_adjusted(ms, drawn, np_ * ((ng + 7) // 8), hbm_peak, int_peak, column)
@@ -595,7 +606,7 @@ def work_adjusted(ms, drawn, nvec, hbm_peak, int_peak, column=False):
     previous alleles read and its alleles written (STABLE_BYTES = 1/8 + 1 + 1 B). Per
     generation the bound is the slower of the two; the fraction is the sum of the bounds
     over the sum of the measured times. column: the column form, whose rows share one row of
-    angle indices and store no alleles: the draws alone."""
+    angle indices and store no alleles: the draws alone, at the rate of Philox (int_peak)."""
     import numpy as np
     d = np.asarray(drawn, dtype=np.float64)
     t_int = 8.0 * d / int_peak
@@ -608,7 +619,9 @@ def work_adjusted(ms, drawn, nvec, hbm_peak, int_peak, column=False):
             "drawn_per_25": [round(float(d[i:i + 25].mean()) / nvec, 4) for i in range(0, len(d), 25)],
             "frac_per_25": [round(float(bound[i:i + 25].sum() / meas[i:i + 25].sum()), 3)
                             for i in range(0, len(d), 25)],
-            "what": "per generation: max(8 draws per vector that drew at the measured integer "
+            "what": "8 draws per vector that drew at the measured rate of Philox4x32-10 alone, summed, "
+                    "over the measured generation times" if column else
+                    "per generation: max(8 draws per vector that drew at the measured integer "
                     "ceiling, (32 B per vector that drew + 2.125 B per one that did not) at the "
                     "measured HBM bandwidth), summed, over the measured generation times"}
 
@@ -761,13 +774,14 @@ def run_batched(a):
     # Roofline of the batched kernels: per generation the algorithmic work is every member's
     # genes -- 4 B of state each, read and written, and the drawn pass's integer work --
     # timed as the run / G; the bound is the slower of the two measured ceilings (HBM copy
-    # bandwidth, the integer ceiling of the same per-gene arithmetic).
+    # bandwidth, the integer ceiling of the same per-gene arithmetic). In the column form (all
+    # but --per-generation) it is the draws alone, at the measured rate of Philox.
     peaks, peak_src = load_peaks()
     hbm_peak = float(peaks["hbm_gbs"])
     launch_s = run_s / (a.steps * G)
     ceiling = Q.qieo_measure_integer_ceiling(5)
-    int_peak = ceiling.drawn_genes_per_s
-    t_hbm = STATE_BYTES_PER_GENE * genes_per_gen / (hbm_peak * 1e9)
+    int_peak = ceiling.drawn_genes_per_s if a.per_generation else ceiling.philox_genes_per_s
+    t_hbm = STATE_BYTES_PER_GENE * genes_per_gen / (hbm_peak * 1e9) if a.per_generation else 0.0
     t_int = genes_per_gen / int_peak
     achieved = STATE_BYTES_PER_GENE * genes_per_gen / launch_s / 1e9
     if t_hbm >= t_int:
@@ -777,11 +791,11 @@ def run_batched(a):
         ach = genes_per_gen / launch_s / 1e9
         roof = {"bound": "alu", "achieved": ach, "peak": int_peak / 1e9, "unit": "Ggene-updates/s",
                 "frac": ach / (int_peak / 1e9),
-                "peak_source": "measured: qieo_measure_integer_ceiling (the drawn pass's per-gene "
-                               "integer work, state in registers, %d blocks, best of %d)" % (
-                                   ceiling.grid_ctas, ceiling.reps)}
+                "peak_source": "measured: qieo_measure_integer_ceiling (%s, %d blocks, best of %d)" % (
+                    "the drawn pass's per-gene integer work, state in registers" if a.per_generation else
+                    "Philox4x32-10 alone", ceiling.grid_ctas, ceiling.reps)}
     roof.update({"frac_hbm_4B_formula": achieved / hbm_peak, "hbm_peak_gbs": hbm_peak,
-                 "int_ceiling_gene_updates_per_s": int_peak, "t_hbm_us": t_hbm * 1e6,
+                 "int_ceiling_gene_updates_per_s": ceiling.drawn_genes_per_s, "t_hbm_us": t_hbm * 1e6,
                  "t_int_us": t_int * 1e6,
                  "state_in_l2": state_bytes < L2_BYTES,
                  "traffic": profile_traffic("batch_generation_kernel" if a.per_generation
@@ -789,7 +803,8 @@ def run_batched(a):
                  "kernel": ("batch_generation_kernel (one launch per generation for all members)"
                             if a.per_generation else
                             "column_batch_kernel (one cooperative launch per run for all members; one row "
-                            "of angle indices a member, no state streamed: the 4 B figures do not apply)"),
+                            "of angle indices a member, no state streamed: the 4 B figures do not apply; its "
+                            "draws are not counted, so frac, of a full draw per gene-update, can exceed 1)"),
                  "us_per_generation": launch_s * 1e6,
                  "traffic_per": "generation (the persistent launch divided by its generations)"})
     if roof["traffic"]:

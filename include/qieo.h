@@ -164,7 +164,7 @@ qieo_status qieo_reset(qieo_instance *inst);
  * Rule R1 from equal rows (every run from generation 0 on) is the column form: R1 steps all
  * qubits of a gene alike, so one row of angle indices is the population's state, and a run
  * is one or two cooperative launches whose blocks wait, bounded, for one another between
- * generations. Not with elite_on_host, byte state, a fitness that does not fit the packed
+ * generations, or, for a few generations, one plain launch each and one to end them. Not with elite_on_host, byte state, a fitness that does not fit the packed
  * elite key, or QIEO_FLAG_UNFUSED, _COOPERATIVE, _REGISTER_PREFETCH, _PER_GENERATION,
  * _STREAMED, _SIXTEEN, _NO_FIXED_WORDS or _SPARSE_ALWAYS. Results do not depend on it.
  * Otherwise each generation is one kernel
@@ -174,7 +174,11 @@ qieo_status qieo_reset(qieo_instance *inst);
  * a bounded grid barrier after each generation (qieo_launch_shape.persistent tells which).
  * Stream-ordered: returns after enqueueing unless QIEO_FLAG_SYNC_RUN is set or
  * elite_on_host is 1. A barrier wait that runs out is reported as QIEO_ERR_TIMEOUT by the
- * next call that waits for the device; the state is then undefined until qieo_reset. */
+ * next call that waits for the device; the state is then undefined until qieo_reset, and in the
+ * column form no later run changes it. A run may be captured into a CUDA graph once the
+ * history has room for its generations; every replay goes on from the state that it finds, in
+ * the form that the run had: capture again after loading a checkpoint whose rows differ, or after
+ * resetting an instance that had one. */
 qieo_status qieo_run(qieo_instance *inst, int32_t generations);
 
 /* Bound of one grid-barrier wait inside a cooperative run, in nanoseconds (default 10 s;
@@ -213,8 +217,8 @@ qieo_status qieo_get_elite_history(qieo_instance *inst, int32_t first, int32_t n
  * that drew (ran QIP, Sec. III-B, with a Philox draw per qubit, after their CIP); the rest
  * were fixed (every qubit at theta = 0 or pi/2, |alpha|^2 or |beta|^2 = 1, Sec. I), so
  * their alleles were known without a draw (the fixed-allele pass of the dense form, the
- * stable vectors of the sparse form, the dropped quads of the column form). np * ceil(ng / 8) means every vector drew; generations
- * run in a batch, or restored by a checkpoint load, report that value (they are not counted).
+ * stable vectors of the sparse form, the dropped quads of the column form). np * ceil(ng / 8)
+ * means every vector drew, as in the column form's runs of a few generations; generations run in a batch, or restored by a checkpoint load, report that value (they are not counted).
  * QIEO_ERR_INVALID for an instance without the words, out NULL or a range outside [0, t). */
 qieo_status qieo_get_drawn_vectors(qieo_instance *inst, int32_t first, int32_t n, int64_t *out);
 
@@ -222,8 +226,9 @@ qieo_status qieo_get_drawn_vectors(qieo_instance *inst, int32_t first, int32_t n
 qieo_status qieo_get_threshold_table(qieo_instance *inst, uint64_t *t_out);
 
 /* Launch shape of the fused generation kernel, for the runs that are not in the column form
- * (see qieo_run; that form cuts its work by the genes that still draw). Results do not depend on it (all sums are
- * exact integers and every draw is keyed by gene, chromosome and generation). A row is cut
+ * (see qieo_run; that form cuts its work by the genes that still draw, and for its runs every
+ * field but `narrow` says only what a row-by-row run would do). Results do not depend on it (all sums
+ * are exact integers and every draw is keyed by gene, chromosome and generation). A row is cut
  * into tiles of lanes_per_row * warps_per_row vectors of 8 genes; a persistent grid of
  * grid_ctas blocks covers the ntile * np tile-rows, in equal contiguous shares when a share
  * is below 64 tile-rows, otherwise (runs with the packed elite key) by taking segments of
@@ -270,6 +275,7 @@ qieo_status qieo_get_kernel_time(qieo_instance *inst, double *ms, int64_t *launc
  * QIEO_FLAG_TIME_GENERATIONS: ms_out[i] = the time (ms) from the start of the run's
  * generation i to the start of the next one (for the last generation: to the end of the
  * run's last generation, before its final rotation), for i < min(n, generations of that run);
+ * 0 for generations that a converged run did not execute;
  * *count = that number. Waits (bounded) for the run to finish. The times cover one fused
  * generation kernel each (CIP of the generation before, QIP, Evaluation, DetermineElite);
  * the run's final CIP launch is not included. QIEO_ERR_INVALID without the flag. */
@@ -394,8 +400,9 @@ qieo_status qieo_destroy_batch(qieo_batch *batch);
  * work list and graphs are built once). */
 qieo_status qieo_run_batch(qieo_instance *const *instances, int32_t n, int32_t generations);
 
-/* Picks the launch shape (tile of lanes x warps vectors) of an instance at generation 0 by
- * timing `trial_generations` generations of each candidate shape, keeps the fastest, and
+/* Picks the launch shape (tile of lanes x warps vectors) of an instance at generation 0, for its
+ * runs that are not in the column form (see qieo_launch_shape: it has no effect on those
+ * that are), by timing `trial_generations` generations of each candidate shape, keeps the fastest, and
  * records it in a process-wide table keyed by (ng, np, D, rule, sum form) so that
  * instances created later with the same key start with it. The instance is left at
  * generation 0 (qieo_reset). Results never depend on the shape. *shape_out may be NULL. */

@@ -2097,7 +2097,7 @@ qieo_status qieo_create_row_block(const qieo_problem *problem, const qieo_params
     q->row_block = true;
     q->gp.row0 = row0;
     st = configure(q);   // a row block keeps no fixed-vector words
-    if (st == QIEO_OK) st = qieo_reset(q);   // ... and the full state
+    if (st == QIEO_OK) st = qieo_reset(q);
     if (st != QIEO_OK) {
         qieo_destroy_instance(q);
         return st;

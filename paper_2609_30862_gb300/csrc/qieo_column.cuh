@@ -19,9 +19,10 @@
 // The results are those of the row-by-row forms, which the instance keeps for rule R2, for
 // states whose rows differ (a checkpoint may hold one) and for the forms that flags ask for.
 //
-// One cooperative launch per run (column_run_kernel), then column_plane_kernel and
-// column_end_kernel. Measured on the GB300 against the forms it replaces for these runs:
-// see the table at column_run_kernel.
+// A run is one cooperative launch, or two (column_run_kernel while the blocks' shares are long,
+// column_small_kernel after it), then column_plane_kernel and column_end_kernel; a run of a few
+// generations is plain launches of column_observe_kernel and column_step_kernel. What each measured
+// against the form it replaces stands at the kernel.
 #pragma once
 
 #include "qieo_kernels.cuh"
