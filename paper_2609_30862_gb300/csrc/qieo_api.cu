@@ -1822,6 +1822,18 @@ qieo_status fetch(qieo_instance *q, void *dst, const void *src, size_t bytes)
     return wait_stream(q->stream);
 }
 
+// The allele plane of the last generation that ran (a run that converged stopped before q->t).
+qieo_status last_plane(qieo_instance *q, const uint8_t **plane)
+{
+    int32_t t = q->t;
+    if (q->gp.converge) {
+        qieo_status st = fetch(q, &t, q->gp.gen, sizeof t);
+        if (st != QIEO_OK) return st;
+    }
+    *plane = q->gp.xbits + (size_t)((t + 1) & 1) * q->gp.xplane;
+    return QIEO_OK;
+}
+
 void unpack_row(const uint8_t *packed, int32_t ng, uint8_t *out)
 {
     for (int32_t j = 0; j < ng; ++j) out[j] = (uint8_t)((packed[j >> 3] >> (j & 7)) & 1u);
@@ -1916,8 +1928,9 @@ qieo_status qieo_get_allele_row(qieo_instance *q, int32_t c, uint8_t *x_out)
     st = set_device(q);
     if (st != QIEO_OK) return st;
     std::vector<uint8_t> x((size_t)q->xstride);
-    const uint8_t *row = q->gp.xbits + (size_t)((q->t + 1) & 1) * q->gp.xplane + (size_t)c * q->xstride;
-    st = fetch(q, x.data(), row, x.size());
+    const uint8_t *plane = nullptr;
+    st = last_plane(q, &plane);
+    if (st == QIEO_OK) st = fetch(q, x.data(), plane + (size_t)c * q->xstride, x.size());
     if (st != QIEO_OK) return st;
     unpack_row(x.data(), q->ng, x_out);
     return QIEO_OK;
@@ -1931,8 +1944,9 @@ qieo_status qieo_get_alleles(qieo_instance *q, uint8_t *x_out)
     st = set_device(q);
     if (st != QIEO_OK) return st;
     std::vector<uint8_t> x((size_t)q->np * q->xstride);
-    const uint8_t *plane = q->gp.xbits + (size_t)((q->t + 1) & 1) * q->gp.xplane;
-    st = fetch(q, x.data(), plane, x.size());
+    const uint8_t *plane = nullptr;
+    st = last_plane(q, &plane);
+    if (st == QIEO_OK) st = fetch(q, x.data(), plane, x.size());
     if (st != QIEO_OK) return st;
     for (int32_t c = 0; c < q->np; ++c)
         unpack_row(x.data() + (size_t)c * q->xstride, q->ng, x_out + (size_t)c * q->ng);

@@ -603,3 +603,19 @@ def test_generation_times_of_a_run_that_stops(np_):
         assert len(ms) == 700 and ms[:n].min() > 0 and ms[:n].max() < 10 and not ms[n:].any()
         I.run(700)
         assert not np.asarray(I.generation_times(700)).any()
+
+
+@pytest.mark.parametrize("rule,ng,np_,D", [(0, 200, 30, 100), (1, 40, 60, 8)])
+@pytest.mark.parametrize("extra", [0, 1, 2])
+def test_alleles_after_a_stop(rule, ng, np_, D, extra):
+    """The alleles of the last generation that ran, whatever parity the generations asked for have."""
+    prob = W.knapsack(ng, 3)
+    ref = O.run(prob, np_, 900, seed=3, rule=rule, D=D, window=20)
+    n = int(ref.t[0])
+    assert ref.stopped
+    for chunks in ([n + 5 + extra], [n + extra], [n - 2, 9 + extra]):
+        with Q.Instance(prob, np_, seed=3, D=D, rule=rule, flags=Q.QIEO_FLAG_CONVERGE) as I:
+            for g in chunks:
+                I.run(g)
+            assert I.state()[1] == n
+            assert np.array_equal(I.alleles(), ref.x) and np.array_equal(I.allele_row(7), ref.x[7])
