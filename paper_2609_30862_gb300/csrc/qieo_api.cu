@@ -1239,7 +1239,9 @@ qieo_status run_device(qieo_instance *q, int32_t G)
     if (q->gp.fword) q->fword_dirty = true;
     const bool timing = (q->flags & QIEO_FLAG_TIME_KERNELS) != 0;
     const bool first_time = q->run_lengths_seen[G]++ == 0;
-    if ((q->flags & (QIEO_FLAG_NO_GRAPH | QIEO_FLAG_TIME_GENERATIONS)) || (first_time && !q->graphs.count(G))) {
+    // (an event recorded inside a graph cannot be timed)
+    if ((q->flags & (QIEO_FLAG_NO_GRAPH | QIEO_FLAG_TIME_GENERATIONS | QIEO_FLAG_TIME_KERNELS)) ||
+        (first_time && !q->graphs.count(G))) {
         qieo_status st = enqueue_device_run(q, G);
         if (st != QIEO_OK) return st;
     } else {

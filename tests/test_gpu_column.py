@@ -619,3 +619,14 @@ def test_alleles_after_a_stop(rule, ng, np_, D, extra):
                 I.run(g)
             assert I.state()[1] == n
             assert np.array_equal(I.alleles(), ref.x) and np.array_equal(I.allele_row(7), ref.x[7])
+
+
+def test_kernel_times_of_repeated_runs():
+    """Runs of one length, one launch per generation and timed: the second would replay a graph."""
+    prob = W.knapsack(2603, 5)
+    with Q.Instance(prob, 60, seed=5, rule=1, flags=Q.QIEO_FLAG_PER_GENERATION | Q.QIEO_FLAG_TIME_KERNELS) as I:
+        for k in range(1, 5):
+            I.run(6)
+            ms, launches = I.kernel_time()
+            assert launches == 6 * k and ms > 0
+        check(I, O.run(prob, 60, 24, seed=5, rule=1), 24)
