@@ -208,7 +208,7 @@ struct qieo_instance {
     bool col_valid = false;        // cp's state between runs holds it
     bool force_rows = false;       // autotuning: time the row-by-row forms
     bool keep_state = false;       // member of a batch that runs row by row: a reset writes the full
-                                   // state too
+                                   // state too, and a run in the column form makes it
 };
 
 namespace {
@@ -1229,7 +1229,10 @@ qieo_status run_device(qieo_instance *q, int32_t G)
         CUDA_TRY(cudaStreamIsCapturing(q->stream, &capture));
         column = capture == cudaStreamCaptureStatusNone;
     }
-    if (column) return run_column(q, G);
+    if (column) {
+        qieo_status st = run_column(q, G);
+        return st == QIEO_OK && q->keep_state ? ensure_state(q) : st;
+    }
     if (q->col_mem) {
         qieo_status st = ensure_state(q);
         if (st != QIEO_OK) return st;
@@ -3048,8 +3051,8 @@ qieo_status group_members(qieo_batch *bt)
     }
     bt->as_column = as_column;
     // Members that could run in the column form but do not here have their full state from now on after
-    // a reset too: made by the batch's next run, it would be made again by every replay of a graph
-    // that this run was captured in.
+    // resets and runs of their own too: made by the batch's next run, it would be made again by every
+    // replay of a graph that this run was captured in.
     for (size_t i = 0; i < bt->members.size(); ++i) {
         qieo_instance *q = bt->members[i];
         if (!q->col_mem || as_column[i]) continue;
@@ -3206,6 +3209,11 @@ qieo_status qieo_batch_run(qieo_batch *bt, int32_t G)
     if (!bt->other_streams.empty()) {
         CUDA_TRY(cudaEventRecord(bt->ev_out, bt->stream));
         for (cudaStream_t s : bt->other_streams) CUDA_TRY(cudaStreamWaitEvent(s, bt->ev_out, 0));
+    }
+    for (qieo_instance *q : bt->members) {
+        if (!q->keep_state) continue;
+        qieo_status st = ensure_state(q);
+        if (st != QIEO_OK) return st;
     }
     for (qieo_instance *q : bt->members) q->t += G;
     return QIEO_OK;

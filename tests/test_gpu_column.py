@@ -452,9 +452,10 @@ def test_checkpoint_rows_are_compared(ng, np_, row):
         check(I, st, 9)
 
 
-def test_captured_row_by_row_batch_goes_on_with_every_replay():
-    """A member that could run in the column form, in a batch that runs row by row: reset, then a captured
-    run of the batch, replayed."""
+@pytest.mark.parametrize("before", ["", "run", "batch"])
+def test_captured_row_by_row_batch_goes_on_with_every_replay(before):
+    """A member that could run in the column form, in a batch that runs row by row: reset, perhaps a run in
+    the column form, alone or in another batch, then a captured run of the batch, replayed."""
     torch = pytest.importorskip("torch")
     prob, np_ = W.knapsack(2603, 5), 90
     stream = torch.cuda.Stream()
@@ -464,6 +465,11 @@ def test_captured_row_by_row_batch_goes_on_with_every_replay():
             b.run(3)
             I.reset()
             J.reset()
+            if before == "run":
+                I.run(8)
+            if before == "batch":
+                with Q.Batch([I]) as alone:
+                    alone.run(8)
             I.synchronize()
             graph = torch.cuda.CUDAGraph()
             with torch.cuda.graph(graph, stream=stream):
@@ -471,10 +477,10 @@ def test_captured_row_by_row_batch_goes_on_with_every_replay():
             for _ in range(4):
                 graph.replay()
             torch.cuda.synchronize()
-            for X, seed in ((I, 5), (J, 6)):
-                st = O.run(prob, np_, 24, seed=seed)
+            for X, seed, gens in ((I, 5, 32 if before else 24), (J, 6, 24)):
+                st = O.run(prob, np_, gens, seed=seed)
                 k, t = X.state()
-                assert t == 24 and np.array_equal(k, st.k)
+                assert t == gens and np.array_equal(k, st.k)
                 assert np.array_equal(X.best()[0], st.best_x) and np.array_equal(X.fitness(), st.f)
         I.run(30)                # a run of its own goes on from there
         I.reset()
