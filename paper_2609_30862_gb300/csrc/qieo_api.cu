@@ -1127,17 +1127,20 @@ cudaError_t launch_column_observe(qieo_instance *q, int32_t t)
 //   3,000 x 30,000    89, 189, 302, 378 | 135, 218, 303, 377; 20, 20, 21, 22
 // A gene needs K steps from pi/4 to a bound, and takes about three times as many in a solve. So: up to
 // four generations while none can be fixed, and while few are where launches are most of the time
-// (2^20 genes); later on one, or two of a small population. Two shapes for which the cooperative form
-// is slow: a few rows of very many genes, which take the CIP for every tile and turn (2 x 1,000,003,
-// 12 generations: 120 | 155), and a million rows of a few genes, whose fitness one block fills once
-// every gene is fixed (1,000,000 x 8, 4 generations: 111 | 393, 130).
+// (2^20 genes); five where a row has several tiles, so that the blocks of the cooperative form meet
+// at a counter (32 x 2,500: 27 | 30; 300 x 3,000: 33 | 42); later on one, or two of a small
+// population. Two shapes for which the cooperative form is slow: a few rows of very many genes, which
+// take the CIP for every tile and turn (2 x 1,000,003, 12 generations: 120 | 155), and a million
+// rows of a few genes, whose fitness one block fills once every gene is fixed (1,000,000 x 8, four
+// generations: 111 | 393; 130).
 bool step_run(const qieo_instance *q, int32_t G)
 {
     const int64_t genes = (int64_t)q->np * q->svec * 8, end = (int64_t)q->t + G;
+    const int32_t most = q->svec > qieo::kThreads ? 5 : 4;
     if (q->gp.converge && G > 2) return false;   // (two launches a generation)
-    if (end <= q->K) return G <= 4 || (q->np <= 4 && q->svec >= 1 << 16);
+    if (end <= q->K) return G <= most || (q->np <= 4 && q->svec >= 1 << 16);
     if (G <= 2) return genes <= (G == 1 || end <= 3 * (int64_t)q->K ? (int64_t)1 << 24 : (int64_t)1 << 20);
-    return G <= 4 && ((q->np >= 1 << 18 && q->svec <= 4) || (end <= 3 * (int64_t)q->K && genes <= (int64_t)1 << 20));
+    return G <= most && ((q->np >= 1 << 18 && q->svec <= 4) || (end <= 3 * (int64_t)q->K && genes <= (int64_t)1 << 20));
 }
 
 // A run in the column form: one cooperative launch, the allele plane, the state between runs.
