@@ -3368,14 +3368,15 @@ struct StepRecord {
 // Solves admitted between two looks at the steps: an admission takes the host about 50 us, and the GPU
 // starts on the first ones meanwhile.
 constexpr size_t kAdmitAtOnce = 16;
-
-// Per region: members (or params), tasks (or segments), block starts. As many small solves as fitted 16 MB
-// row by row (a member's params, one segment and its count each: 35,246) fit in the column form,
-// whose members are larger and have a task for each of its three launches.
-constexpr size_t kWorkListBytes = 22u << 20;
-static_assert(kWorkListBytes / (sizeof(qieo::ColMember) + 3 * sizeof(qieo::ColTask)) >
-                  ((size_t)16 << 20) / (sizeof(qieo::GenParams) + sizeof(qieo::BatchSeg) + sizeof(int32_t)),
-              "a work list holds fewer solves than its row-by-row form did");
+// Per region of a work list: members (or params), tasks (or segments), block starts. A small solve's
+// entry is 608 bytes in the column form, 476 row by row, so a region grows with the solves in the
+// column form: all lists that fit 16 MB row by row fit.
+constexpr size_t kWorkListBytes = (size_t)33 << 19, kColumnListBytes = 2u << 20, kWorkListStep = 8u << 20;
+static_assert((kColumnListBytes / (sizeof(qieo::ColMember) + 3 * sizeof(qieo::ColTask))) *
+                      (sizeof(qieo::ColMember) + 3 * sizeof(qieo::ColTask) -
+                       (sizeof(qieo::GenParams) + sizeof(qieo::BatchSeg) + sizeof(int32_t))) <
+                  kWorkListBytes - ((size_t)16 << 20),
+              "a region that does not grow holds fewer solves than its row-by-row form did");
 
 }  // namespace
 
@@ -3388,6 +3389,7 @@ struct qieo_server {
     ArenaAlloc alloc;
     char *wl_dev[2] = {nullptr, nullptr};
     char *wl_host[2] = {nullptr, nullptr};
+    size_t wl_bytes[2] = {0, 0};
     int wl_next = 0;
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
@@ -3423,6 +3425,26 @@ void destroy_instance_nosync(qieo_instance *q)
     delete q;
 }
 
+// Region r of the work lists with room for `bytes` (its last step is over).
+qieo_status ensure_work_list(qieo_server *S, int r, size_t bytes)
+{
+    if (bytes <= S->wl_bytes[r]) return QIEO_OK;
+    char *dev = nullptr, *host = nullptr;
+    cudaError_t ce = cudaMalloc(&dev, bytes);
+    if (ce == cudaSuccess) ce = cudaMallocHost(&host, bytes);
+    if (ce != cudaSuccess) {
+        cudaGetLastError();      // (reported here; not again by the next launch)
+        if (dev) cudaFree(dev);
+        return fail(QIEO_ERR_OOM, "work list of %zu bytes: %s", bytes, cudaGetErrorString(ce));
+    }
+    if (S->wl_dev[r]) cudaFree(S->wl_dev[r]);
+    if (S->wl_host[r]) cudaFreeHost(S->wl_host[r]);
+    S->wl_dev[r] = dev;
+    S->wl_host[r] = host;
+    S->wl_bytes[r] = bytes;
+    return QIEO_OK;
+}
+
 // Enqueues `G` generations (+ the final rotation) of every member on the server stream, for members in
 // the column form the remaining ones if fewer, with the batched kernels; the work list goes
 // through the next double-buffered region.
@@ -3435,8 +3457,6 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
     *stop_host = nullptr;
     const int r = S->wl_next;
     S->wl_next ^= 1;
-    char *host = S->wl_host[r];
-    char *dev = S->wl_dev[r];
     size_t used = 0;
     struct Launch {
         bool narrow;
@@ -3462,12 +3482,20 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
         qieo_status st = column_batch_grid(grp[0], b);
         if (st != QIEO_OK) return st;
         plan_column_batch(grp, gens, S->sm_count, false, b);
-        size_t off[kColumnBatchParts], bytes[kColumnBatchParts];
-        const void *src[kColumnBatchParts];
-        used = column_batch_layout(b, used, off, src, bytes);
-        if (used > kWorkListBytes) return fail(QIEO_ERR_INVALID, "too many resident solves for one work list");
-        for (int i = 0; i < kColumnBatchParts; ++i) std::memcpy(host + off[i], src[i], bytes[i]);
-        place_column_batch(b, dev, off);
+    }
+    size_t off[kColumnBatchParts], bytes[kColumnBatchParts], column_bytes = 0;
+    const void *src[kColumnBatchParts];
+    for (const ColumnBatch *b : columns) column_bytes = column_batch_layout(*b, column_bytes, off, src, bytes);
+    if (column_bytes > kColumnListBytes) {
+        const qieo_status st = ensure_work_list(S, r, kWorkListBytes + align_up(column_bytes, kWorkListStep));
+        if (st != QIEO_OK) return st;
+    }
+    char *const host = S->wl_host[r], *const dev = S->wl_dev[r];
+    for (ColumnBatch *b : columns) {
+        used = column_batch_layout(*b, used, off, src, bytes);
+        for (int i = 0; i < kColumnBatchParts; ++i)
+            if (bytes[i]) std::memcpy(host + off[i], src[i], bytes[i]);
+        place_column_batch(*b, dev, off);
     }
     for (int narrow = 0; narrow < 2; ++narrow) {
         for (int rule = 0; rule < 2; ++rule) {
@@ -3487,7 +3515,7 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
                 off[i] = used;
                 used = align_up(used + sizes[i], 256);
             }
-            if (used > kWorkListBytes)
+            if (used > S->wl_bytes[r])
                 return fail(QIEO_ERR_INVALID, "too many resident solves for one work list");
             for (size_t i = 0; i < grp.size(); ++i)
                 std::memcpy(host + off[0] + i * sizeof(qieo::GenParams), &grp[i]->gp, sizeof(qieo::GenParams));
@@ -3538,7 +3566,7 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
         const size_t nw = watch.size();
         const size_t p_off = used, o_off = align_up(p_off + nw * sizeof(int32_t *), 256);
         const size_t end = align_up(o_off + nw * sizeof(int32_t), 256);
-        if (end > kWorkListBytes) return fail(QIEO_ERR_INVALID, "too many resident solves for one work list");
+        if (end > S->wl_bytes[r]) return fail(QIEO_ERR_INVALID, "too many resident solves for one work list");
         for (size_t i = 0; i < nw; ++i) std::memcpy(host + p_off + i * sizeof(int32_t *), &watch[i]->gp.conv, sizeof(int32_t *));
         CUDA_TRY(cudaMemcpyAsync(dev + p_off, host + p_off, nw * sizeof(int32_t *), cudaMemcpyHostToDevice, S->stream));
         const int blocks = (int)std::min<size_t>(64, (nw + qieo::kThreads - 1) / qieo::kThreads);
@@ -3793,9 +3821,8 @@ qieo_status qieo_server_create(const qieo_server_config *config, qieo_server **o
         return bail(fail(QIEO_ERR_OOM, "arena of %lld bytes: %s", (long long)cfg.memory_bytes, cudaGetErrorString(ce)));
     S->alloc.init((size_t)cfg.memory_bytes);
     for (int r = 0; r < 2; ++r) {
-        ce = cudaMalloc(&S->wl_dev[r], kWorkListBytes);
-        if (ce == cudaSuccess) ce = cudaMallocHost(&S->wl_host[r], kWorkListBytes);
-        if (ce != cudaSuccess) return bail(fail(QIEO_ERR_OOM, "work lists: %s", cudaGetErrorString(ce)));
+        const qieo_status st = ensure_work_list(S, r, kWorkListBytes);
+        if (st != QIEO_OK) return bail(st);
     }
     for (int narrow = 0; narrow < 2; ++narrow) {
         const size_t smem_max = qieo::kRingBytes + (size_t)qieo::kMaxSegRows * (narrow ? 8 : 16);

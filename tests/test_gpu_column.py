@@ -636,3 +636,18 @@ def test_kernel_times_of_repeated_runs():
             ms, launches = I.kernel_time()
             assert launches == 6 * k and ms > 0
         check(I, O.run(prob, 60, 24, seed=5, rule=1), 24)
+
+
+def test_more_resident_solves_than_a_work_list_starts_with():
+    """4,500 small solves at once: the work lists grow between steps."""
+    probs = [W.knapsack(320, s) for s in range(3)]
+    with Q.Server(memory_bytes=1 << 30, max_active=5000, gens_per_step=1) as srv:
+        ids = [srv.submit(probs[i % 3], 40, 400, seed=i + 1) for i in range(4500)]
+        for i, rid in enumerate(ids):
+            res, bits = srv.poll(rid, wait_ms=60000)
+            assert res.state == Q.QIEO_SOLVE_DONE and res.generations_run == 400
+            if i % 300 == 0:
+                st = O.run(probs[i % 3], 40, 400, seed=i + 1)
+                assert (res.fitness, res.generation, res.chromosome) == tuple(int(v) for v in st.best)
+                assert np.array_equal(bits, st.best_x)
+        assert srv.stats()["max_active"] > 3450
