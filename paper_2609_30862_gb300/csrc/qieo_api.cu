@@ -3486,9 +3486,9 @@ qieo_status enqueue_server_step(qieo_server *S, const std::vector<qieo_instance 
     size_t off[kColumnBatchParts], bytes[kColumnBatchParts], column_bytes = 0;
     const void *src[kColumnBatchParts];
     for (const ColumnBatch *b : columns) column_bytes = column_batch_layout(*b, column_bytes, off, src, bytes);
-    if (column_bytes > kColumnListBytes) {
+    if (column_bytes > kColumnListBytes) {        // (without memory for more, the region may do)
         const qieo_status st = ensure_work_list(S, r, kWorkListBytes + align_up(column_bytes, kWorkListStep));
-        if (st != QIEO_OK) return st;
+        if (st != QIEO_OK && column_bytes > S->wl_bytes[r]) return st;
     }
     char *const host = S->wl_host[r], *const dev = S->wl_dev[r];
     for (ColumnBatch *b : columns) {
